@@ -300,9 +300,18 @@ void harvest(fpd_sim *s) {
     s->recs.clear();
 }
 
-// current bead table: the one that drove the last collision (step 0: the
-// initial table)
-int cur_tab(const fpd_sim *s) { return s->nstep == 0 ? 0 : (int)((s->nstep - 1) & 1); }
+// bead table after n steps: the one that drove the last collision (step 0:
+// the initial table)
+int cur_of(int64_t n) { return n == 0 ? 0 : (int)((n - 1) & 1); }
+int cur_tab(const fpd_sim *s) { return cur_of(s->nstep); }
+
+// The instance record as a checkpoint holds it: without the places of the
+// kept profiles, which are not part of the state.
+fpd::Inst ckpt_record(const fpd_sim *s) {
+    fpd::Inst I = s->inst;
+    I.phi_cap = I.phi_off = 0;
+    return I;
+}
 
 }  // namespace
 
@@ -321,7 +330,7 @@ int enqueue_step(fpd_sim *s, cudaStream_t st, int64_t t, bool profiled) {
             b = take_event(s);
             cudaEventRecord(a, st);
         }
-        e = fpd::launch_beads(s->precision, s->inst_d, nullptr, I.nb, s->pool, s->tab[0], s->tab[1],
+        e = fpd::launch_beads(s->precision, s->inst_d, nullptr, I.nb, I.ntx * I.nty, s->pool, s->tab, s->phi,
                               s->masks[t % fpd::kMaskBufs], parity, 1, s->counters, profiled ? 0 : 1, st,
                               fpd::BeadExport{s->ex_ring_d, s->ex_count, s->ex_slots, s->ex_stride}, s->status);
         if (e != cudaSuccess) return cuda_fail(s, e, "bead kernel launch");
@@ -342,8 +351,8 @@ int enqueue_step(fpd_sim *s, cudaStream_t st, int64_t t, bool profiled) {
     // the previous buffer
     const fpd::SweepMasks mk{s->masks[t % M], s->masks[(t + M - 1) % M], s->masks[(t + 1) % M],
                              (t >= 1 && s->early_cold) ? 1 : 0, s->status, s->copy_shortfall};
-    e = fpd::launch_lattice(s->precision, s->inst_d, I, s->pool, s->tab[parity], mk, parity, after_beads,
-                            s->variant, st);
+    e = fpd::launch_lattice(s->precision, s->inst_d, I, s->pool, s->tab[parity], s->phi[parity], mk, parity,
+                            after_beads, s->variant, st);
     if (e != cudaSuccess) return cuda_fail(s, e, "lattice kernel launch");
     if (profiled) {
         cudaEventRecord(b, st);
@@ -466,7 +475,8 @@ namespace {
 // counter and the instance record.
 constexpr size_t kStateAlign = 256;
 struct StateLayout {
-    size_t pool, tab, masks, counters, inst, total;  // offsets; total = block size
+    size_t pool, tab, masks, counters, inst, phi, box, total;  // offsets; total = block size
+    size_t phi_one;  // bytes of one table's kept profiles (0: not kept)
     size_t pool_bytes, tab_bytes, tab_one, mask_bytes, mask_words;
 };
 size_t up(size_t v) { return (v + kStateAlign - 1) / kStateAlign * kStateAlign; }
@@ -485,7 +495,13 @@ StateLayout state_layout(const fpd::Inst &I, size_t elem) {
     L.counters = up(L.masks + L.mask_bytes);
     // last-block counter, the 64-bit export counter at +8, the status word at +16
     L.inst = up(L.counters + 32);
-    L.total = up(L.inst + sizeof(fpd::Inst));
+    // FP64: the beads' profiles over their support boxes (PhiTab), unless
+    // their supports are so wide that the two tables would outgrow kPhiBytes
+    L.phi = up(L.inst + sizeof(fpd::Inst));
+    L.phi_one = elem == 8 ? (size_t)I.nb * fpd::phi_cells(I) * sizeof(double) : 0;
+    if (2 * L.phi_one > fpd::kPhiBytes) L.phi_one = 0;
+    L.box = up(L.phi + 2 * L.phi_one);
+    L.total = up(L.box + (L.phi_one ? 2 * nbm * sizeof(int4) : 0));
     return L;
 }
 
@@ -552,6 +568,7 @@ int create_impl(const fpd_params *p, void *stream, void *workspace, uint64_t wor
     } while (0)
     FPD_TRY(fpd::prepare_lattice_kernels(), "sweep kernel attributes");
     const StateLayout L = state_layout(I, s->elem);
+    s->inst.phi_cap = L.phi_one ? fpd::phi_cells(I) : 0;
     if (workspace) {
         if (workspace_bytes < L.total || ((uintptr_t)workspace % kStateAlign) != 0) {
             fail(nullptr, FPD_EINVAL, "workspace must hold %llu bytes at a %zu-byte aligned address",
@@ -577,6 +594,10 @@ int create_impl(const fpd_params *p, void *stream, void *workspace, uint64_t wor
         s->tab[t] = fpd::BeadTab{b,           b + nbm,     b + 2 * nbm, b + 3 * nbm, b + 4 * nbm,
                                  b + 5 * nbm, b + 6 * nbm, b + 7 * nbm, b + 8 * nbm, f,
                                  f + nbm,     f + 2 * nbm, f + 3 * nbm, f + 4 * nbm, f + 5 * nbm};
+        if (L.phi_one) {
+            s->phi[t].phi = (double *)(base + L.phi + t * L.phi_one);
+            s->phi[t].box = (int4 *)(base + L.box) + t * nbm;
+        }
     }
     // tile masks, one buffer per step of the rotation (zeroed with the block)
     s->masks[0] = (unsigned *)(base + L.masks);
@@ -599,7 +620,7 @@ int create_impl(const fpd_params *p, void *stream, void *workspace, uint64_t wor
                 "copy beads");
         FPD_TRY(cudaMemcpyAsync(s->tab[0].Ry, Ry.data(), nb * sizeof(double), cudaMemcpyHostToDevice, s->stream),
                 "copy beads");
-        FPD_TRY(fpd::launch_beads(s->precision, s->inst_d, nullptr, nb, s->pool, s->tab[0], s->tab[1],
+        FPD_TRY(fpd::launch_beads(s->precision, s->inst_d, nullptr, nb, I.ntx * I.nty, s->pool, s->tab, s->phi,
                                   s->masks[0], 0, 0, s->counters, 0, s->stream),
                 "initial bead table");
     }
@@ -920,7 +941,8 @@ int fpd_save(fpd_sim *s, const char *path) {
     h.nstep = s->nstep;
     std::FILE *f = std::fopen(path, "wb");
     if (!f) return fail(s, FPD_EINVAL, "fpd_save: cannot open %s for writing", path);
-    bool ok = std::fwrite(&h, sizeof h, 1, f) == 1 && std::fwrite(&s->inst, sizeof(fpd::Inst), 1, f) == 1 &&
+    const fpd::Inst rec = ckpt_record(s);
+    bool ok = std::fwrite(&h, sizeof h, 1, f) == 1 && std::fwrite(&rec, sizeof rec, 1, f) == 1 &&
               std::fwrite(pool.data(), 1, pool.size(), f) == pool.size() &&
               std::fwrite(tabs.data(), 1, tabs.size(), f) == tabs.size() &&
               std::fwrite(masks.data(), 1, masks.size(), f) == masks.size();
@@ -936,6 +958,7 @@ int fpd_load(fpd_sim *s, const char *path) {
     if (!f) return fail(s, FPD_EINVAL, "fpd_load: cannot open %s", path);
     CkptHeader h{};
     fpd::Inst inst;
+    const fpd::Inst rec = ckpt_record(s);
     std::vector<char> pool, tabs, masks;
     const char *why = nullptr;
     if (std::fread(&h, sizeof h, 1, f) != 1 || std::memcmp(h.tag, kCkptTag, sizeof h.tag) != 0) {
@@ -944,7 +967,7 @@ int fpd_load(fpd_sim *s, const char *path) {
         why = "written by another ABI version";
     } else if (std::fread(&inst, sizeof inst, 1, f) != 1) {
         why = "truncated";
-    } else if (std::memcmp(&inst, &s->inst, sizeof inst) != 0 || h.pool_bytes != s->pool_bytes ||
+    } else if (std::memcmp(&inst, &rec, sizeof inst) != 0 || h.pool_bytes != s->pool_bytes ||
                h.tab_bytes != s->tab_bytes || h.mask_bytes != s->mask_bytes || h.nstep < 0) {
         why = "written with other parameters";
     } else {
@@ -965,6 +988,10 @@ int fpd_load(fpd_sim *s, const char *path) {
     cudaError_t e = cudaMemcpy(s->pool, pool.data(), pool.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(s->tabmem, tabs.data(), tabs.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(s->masks[0], masks.data(), masks.size(), cudaMemcpyHostToDevice);
+    // the kept profiles follow from the restored positions
+    if (e == cudaSuccess && s->inst.phi_cap)
+        e = fpd::launch_phi(s->inst_d, nullptr, s->inst.nb, s->tab, s->phi, cur_of(h.nstep) ^ 1, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     // the status flags describe the replaced run: they start over
     if (e == cudaSuccess) e = cudaMemset(s->status, 0, sizeof(unsigned));
     if (e != cudaSuccess) return cuda_fail(s, e, "fpd_load");

@@ -100,6 +100,7 @@ struct fpd_batch {
     RangeAlloc pop_alloc, bead_alloc;
     double *tabmem = nullptr;
     fpd::BeadTab tab[2]{};
+    fpd::PhiTab phi[2]{};
     fpd::Inst *insts_d = nullptr;
     unsigned *counters = nullptr;
     unsigned *status = nullptr;  // sticky FPD_FLAG_* bits per slot (device)
@@ -107,7 +108,7 @@ struct fpd_batch {
     int2 *tiles_d = nullptr;
     int tiles_cap = 0, ntiles = 0;
     unsigned *masks = nullptr;  // kMaskBufs * tiles_cap * mask_words, in rotation by global step
-    int2 *beads_all_d = nullptr, *beads_old_d = nullptr, *beads_fresh_d = nullptr;  // (slot, bead)
+    int4 *beads_all_d = nullptr, *beads_old_d = nullptr, *beads_fresh_d = nullptr;  // as launch_beads takes them
     int n_all = 0, n_old = 0, n_fresh = 0;
     std::vector<Slot> slots;
     std::vector<fpd::Inst> insts_h;
@@ -121,6 +122,8 @@ struct fpd_batch {
     // (global step mod kMaskBufs); valid until the next rebuild or tuning change
     cudaGraphExec_t graph[fpd::kMaskBufs] = {};
     cudaStream_t cap_stream = nullptr;
+    double *phi_mem = nullptr;  // FP64: both tables' kept profiles (PhiTab::phi)
+    int64_t phi_len = 0;        // doubles in phi_mem
     double *scratch = nullptr;
     size_t scratch_bytes = 0;
     std::string err;
@@ -168,6 +171,8 @@ void free_batch(fpd_batch *b) {
     cudaFree(b->beads_all_d);
     cudaFree(b->beads_old_d);
     cudaFree(b->beads_fresh_d);
+    cudaFree(b->phi_mem);
+    for (auto &p : b->phi) cudaFree(p.box);
     cudaFree(b->scratch);
 }
 
@@ -180,6 +185,41 @@ int ensure_bscratch(fpd_batch *b, size_t bytes) {
     if (e != cudaSuccess) return bfail(b, FPD_ENOMEM, "cudaMalloc of %zu scratch bytes: %s", bytes, cudaGetErrorString(e));
     b->scratch_bytes = bytes;
     return FPD_OK;
+}
+
+// Places of the active instances' kept profiles (FP64).  The buffer grows as
+// needed; without memory for it, or for an instance whose supports are very
+// wide, profiles are evaluated instead of kept (the same values).
+void place_phi(fpd_batch *b) {
+    if (b->precision != 0) return;
+    int64_t n = 0;
+    for (auto &sl : b->slots) {
+        fpd::Inst &I = sl.inst;
+        if (sl.state != kActive) continue;
+        I.phi_cap = I.phi_off = 0;
+        const int64_t cells = fpd::phi_cells(I);
+        if (I.nb == 0 || 2 * sizeof(double) * I.nb * cells > fpd::kPhiBytes || n + I.nb * cells > INT32_MAX) continue;
+        I.phi_cap = (int)cells;
+        I.phi_off = (int)n;
+        n += I.nb * cells;
+    }
+    if (2 * n > b->phi_len) {
+        cudaFree(b->phi_mem);  // waits for queued steps, which may still read it
+        b->phi_mem = nullptr;
+        b->phi_len = 0;
+        const int64_t want = 2 * n + n / 2;
+        void *p = nullptr;
+        if (cudaMalloc(&p, want * sizeof(double)) == cudaSuccess) {
+            b->phi_mem = (double *)p;
+            b->phi_len = want;
+        } else {
+            (void)cudaGetLastError();
+            for (auto &sl : b->slots)
+                if (sl.state == kActive) sl.inst.phi_cap = sl.inst.phi_off = 0;
+        }
+    }
+    b->phi[0].phi = b->phi_mem;
+    b->phi[1].phi = b->phi_mem ? b->phi_mem + n : nullptr;
 }
 
 // Rebuild the packed tile list, the bead lists and the instance records
@@ -199,6 +239,7 @@ int rebuild(fpd_batch *b) {
         b->mask_words = W;
         b->tiles_cap = 0;  // reallocate the masks below
     }
+    place_phi(b);
     for (int s = 0; s < b->max_slots; ++s) {
         Slot &sl = b->slots[s];
         if (sl.state != kActive) continue;
@@ -238,20 +279,22 @@ int rebuild(fpd_batch *b) {
                              b->stream)) !=
             cudaSuccess)
         return bcuda(b, e, "clear masks");
-    // bead lists: (slot, global bead index) for every bead, for the beads of
+    // bead lists (launch_beads): every bead, for the beads of
     // instances past their first step, and for the newly admitted ones
-    auto upload = [&](int2 *dst, int &n, int which) -> int {
-        std::vector<int2> lst;
+    auto upload = [&](int4 *dst, int &n, int which) -> int {
+        std::vector<int4> lst;
         for (int s = 0; s < b->max_slots; ++s) {
             Slot &sl = b->slots[s];
             if (sl.state != kActive) continue;
             const bool take = which == 0 || (which == 1 && !sl.first) || (which == 2 && sl.fresh);
             if (!take) continue;
-            for (int q = 0; q < sl.inst.nb; ++q) lst.push_back(make_int2(s, sl.inst.bead_off + q));
+            const fpd::Inst &I = sl.inst;
+            for (int q = 0; q < I.nb; ++q)
+                lst.push_back(make_int4(2 * s + I.par_xor, I.bead_off + q, I.bead_off, I.nb));
         }
         n = (int)lst.size();
         if (n > 0) {
-            cudaError_t e2 = cudaMemcpyAsync(dst, lst.data(), n * sizeof(int2), cudaMemcpyHostToDevice, b->stream);
+            cudaError_t e2 = cudaMemcpyAsync(dst, lst.data(), n * sizeof(int4), cudaMemcpyHostToDevice, b->stream);
             // the copy must finish before lst goes out of scope
             if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(b->stream);
             if (e2 != cudaSuccess) return bcuda(b, e2, "copy bead lists");
@@ -262,9 +305,14 @@ int rebuild(fpd_batch *b) {
     if ((rc = upload(b->beads_all_d, b->n_all, 0))) return rc;
     if ((rc = upload(b->beads_old_d, b->n_old, 1))) return rc;
     if ((rc = upload(b->beads_fresh_d, b->n_fresh, 2))) return rc;
+    // the other instances' profiles, in their new places
+    if (b->n_old > 0 && b->phi_mem) {
+        e = fpd::launch_phi(b->insts_d, b->beads_old_d, b->n_old, b->tab, b->phi, gp, b->stream);
+        if (e != cudaSuccess) return bcuda(b, e, "bead profiles");
+    }
     // initial bead tables of new instances (local parity 0 -> table 0)
     if (b->n_fresh > 0) {
-        e = fpd::launch_beads(b->precision, b->insts_d, b->beads_fresh_d, b->n_fresh, b->pool, b->tab[0], b->tab[1],
+        e = fpd::launch_beads(b->precision, b->insts_d, b->beads_fresh_d, b->n_fresh, b->ntiles, b->pool, b->tab, b->phi,
                               b->masks + (size_t)(b->gstep % fpd::kMaskBufs) * b->tiles_cap * b->mask_words, gp, 0,
                               b->counters, 0, b->stream);
         if (e != cudaSuccess) return bcuda(b, e, "initial bead tables");
@@ -306,14 +354,18 @@ int fpd_batch_create(int32_t precision, int32_t max_slots, int64_t pool_bytes, i
         (e = cudaMalloc(&b->insts_d, max_slots * sizeof(fpd::Inst))) != cudaSuccess ||
         (e = cudaMalloc(&b->counters, max_slots * sizeof(unsigned))) != cudaSuccess ||
         (e = cudaMalloc(&b->status, max_slots * sizeof(unsigned))) != cudaSuccess ||
-        (e = cudaMalloc(&b->beads_all_d, nbm * sizeof(int2))) != cudaSuccess ||
-        (e = cudaMalloc(&b->beads_old_d, nbm * sizeof(int2))) != cudaSuccess ||
-        (e = cudaMalloc(&b->beads_fresh_d, nbm * sizeof(int2))) != cudaSuccess) {
+        (e = cudaMalloc(&b->beads_all_d, nbm * sizeof(int4))) != cudaSuccess ||
+        (e = cudaMalloc(&b->beads_old_d, nbm * sizeof(int4))) != cudaSuccess ||
+        (e = cudaMalloc(&b->beads_fresh_d, nbm * sizeof(int4))) != cudaSuccess ||
+        (precision == 0 && ((e = cudaMalloc(&b->phi[0].box, nbm * sizeof(int4))) != cudaSuccess ||
+                            (e = cudaMalloc(&b->phi[1].box, nbm * sizeof(int4))) != cudaSuccess))) {
         free_batch(b);
         delete b;
         return e == cudaErrorMemoryAllocation ? FPD_ENOMEM : FPD_ECUDA;
     }
     cudaMemsetAsync(b->tabmem, 0, 2 * tab_bytes, b->stream);
+    for (auto &p : b->phi)
+        if (p.box) cudaMemsetAsync(p.box, 0, nbm * sizeof(int4), b->stream);
     cudaMemsetAsync(b->counters, 0, max_slots * sizeof(unsigned), b->stream);
     cudaMemsetAsync(b->status, 0, max_slots * sizeof(unsigned), b->stream);
     for (int t = 0; t < 2; ++t) {
@@ -413,7 +465,7 @@ namespace {
 // or those of instances past their first step) and the batched sweep.
 int enqueue_bstep(fpd_batch *b, cudaStream_t st, int64_t gstep, bool any_first) {
     const int gp = (int)(gstep & 1);
-    const int2 *blist = any_first ? b->beads_old_d : b->beads_all_d;
+    const int4 *blist = any_first ? b->beads_old_d : b->beads_all_d;
     const int nbl = any_first ? b->n_old : b->n_all;
     constexpr int M = fpd::kMaskBufs;
     const size_t mstride = (size_t)b->tiles_cap * b->mask_words;
@@ -424,11 +476,11 @@ int enqueue_bstep(fpd_batch *b, cudaStream_t st, int64_t gstep, bool any_first) 
                              b->masks + (size_t)((gstep + 1) % M) * mstride, gstep > b->rebuild_gstep ? 1 : 0};
     cudaError_t e;
     if (nbl > 0) {
-        e = fpd::launch_beads(b->precision, b->insts_d, blist, nbl, b->pool, b->tab[0], b->tab[1], mw, gp, 1,
+        e = fpd::launch_beads(b->precision, b->insts_d, blist, nbl, b->ntiles, b->pool, b->tab, b->phi, mw, gp, 1,
                               b->counters, 1, st, fpd::BeadExport{}, b->status);
         if (e != cudaSuccess) return bcuda(b, e, "batched bead phase");
     }
-    e = fpd::launch_lattice_batch(b->precision, b->insts_d, b->tiles_d, b->ntiles, b->pool, b->tab[0], b->tab[1], mk,
+    e = fpd::launch_lattice_batch(b->precision, b->insts_d, b->tiles_d, b->ntiles, b->pool, b->tab, b->phi, mk,
                                   gp, nbl > 0 ? 1 : 0, b->variant, b->any_mrt, st);
     if (e != cudaSuccess) return bcuda(b, e, "batched lattice sweep");
     return FPD_OK;

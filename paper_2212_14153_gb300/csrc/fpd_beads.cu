@@ -1,6 +1,7 @@
 // fpd_beads.cu -- the bead phase of the FPD step.
 //
-// One CTA per bead b (any number of instances in one launch):
+// One CTA, or a cluster of up to kBeadParts CTAs, per bead b (any number of
+// instances in one launch):
 //   Eq. 5   V_b = sum_x phi_b(x; R_b) u(x) / S_b, with u = (sum_k f_k c_k +
 //           f/2) / rho and f the force density of the table that drove the
 //           last collision (recomputed from that table, Eq. 4);
@@ -11,25 +12,30 @@
 //   Eq. 11 springs, Eq. 12 bending in its general form (tangents of missing
 //   segments are zero, which reproduces the edge cases of Eqs. 12b-12e),
 //   plus the excluded-volume repulsion k_ev (d - r) r_hat of non-bonded beads
-//   closer than d, and G = F / S for the spreading of Eq. 4; it also writes
-//   the FP32 overlay table (positions split hi + lo, G) read by the lattice
-//   sweep of the reduced-precision paths.
+//   closer than d, and G = F / S for the spreading of Eq. 4.  Each bead's CTA
+//   writes its place in the FP32 overlay table (positions split hi + lo) read
+//   by the lattice sweep of the reduced-precision paths, the last CTA the G.
 //
-// Arithmetic: positions, velocities, forces and the reductions over the
-// support are FP64.  In the FP64 (parity) path phi is evaluated in FP64
-// exactly as a plain IEEE evaluation would; in the FP32/FP16-storage paths
-// phi and u are FP32 from bead-relative offsets, each of 256 virtual lanes
-// adds its few support cells (ceil(cells / 256), 3 for a = 4, xi = 1) in
-// FP32 and the lanes are reduced to FP64.  FP64 instructions are kept out of
-// per-cell work: this GPU issues one FP64 warp instruction per ~16 cycles
-// per SM.  Only beads whose support can overlap bead b's support are visited
-// per cell.  Reductions use a fixed tree over the virtual lanes, so results
-// depend neither on scheduling nor on the CTA size (256 threads while the
-// beads of a launch fit on the SMs one per SM, 128 otherwise).
+// What bounds it: a chain of latencies.  A step of a small lattice is the
+// sweep plus everything between the sweep's end and the overlay table, so
+// work is moved off that chain: the bead's support cells, their profiles and
+// the force density there depend only on the table of the previous step, and
+// are listed in shared memory before the kernel waits for the sweep (it is
+// launched while the sweep still runs).  Left on the chain are one round of
+// population loads, one sum, the move, the support sum, and the last CTA.
 //
-// Chaining: the kernel first waits for the preceding sweep and then lets the
-// next sweep launch; that sweep's unmarked tiles run beside this phase, its
-// marked tiles wait for it to complete.
+// Sums are taken in fixed point (Fix below): exact integer additions, so
+// they do not depend on which thread or CTA adds which cell, and a warp adds
+// its lanes with redux instructions.  A bead gives the same bits in every
+// launch shape (alone, in a batch, split over a cluster).
+//
+// Arithmetic: positions, velocities and forces of the FP64 (parity) path are
+// FP64, phi evaluated exactly as a plain IEEE evaluation would; in the
+// FP32/FP16-storage paths phi, u and the forces are FP32 from bead-relative
+// offsets, positions and velocities FP64.  FP64 instructions are kept out of
+// the reduced-precision paths' per-cell work: this GPU issues one FP64 warp
+// instruction per ~16 cycles per SM.  Only beads whose support can overlap
+// bead b's support are visited per cell.
 #include <cuda_fp16.h>
 
 #include <atomic>
@@ -41,101 +47,165 @@ namespace fpd {
 
 namespace {
 
-// The per-bead sums over the support (Eqs. 4-5) are taken over kBeadLanes
-// virtual lanes whatever the CTA size NT: lane v adds the cells v, v +
-// kBeadLanes, ... in that order, thread t holds lanes t and t + NT (when NT <
-// kBeadLanes), and the lanes are reduced in one fixed tree.  A bead therefore
-// gives the same bits in a CTA of either size (a batch may use the other
-// size than the instance alone).
-constexpr int kLaneGroups = kBeadLanes / 32;
-
-// Sum of two doubles over the virtual lanes; partial j of this thread
-// belongs to lane threadIdx.x + j NT.  Result valid in thread 0.
-template <int NT>
-__device__ __forceinline__ void lanes_sum2_to0(double a0, double b0, double a1, double b1, double &ra, double &rb,
-                                               double (*sh)[kLaneGroups]) {
-    constexpr int L = kBeadLanes / NT;
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
+// ------------------------------------------------------- fixed-point sums
+// Sum of n terms x with |x| < 2^ex as integers x 2^s, s = kTop - ex -
+// ceil(log2(n + 1)): no sum can overflow, every addition is exact and order
+// does not matter.  One term is rounded at 2^-(s + 1): for velocities (ex =
+// kVelBits) over 784 box cells at 2^-41 (float) and 2^-117 (double), below a
+// float term's own unit roundoff for velocities above 1e-5 and, with the few
+// hundred roundings of a sum averaging out, below the sum's above 1e-6.  A
+// caller that meets a larger term (mag) repeats the sum with a larger ex.
+constexpr int kVelBits = 0;
+template <class R> struct Fix;
+template <> struct Fix<float> {
+    using T = long long;
+    static constexpr int kTop = 50;
+    static __device__ __forceinline__ T term(float x, int s) {
+        return __float2ll_rn(x * __int_as_float((s + 127) << 23));  // |s| < 126: x scaled by 2^s
+    }
+    // size of |x|, ordered like |x|; the ex it needs; whether it is finite
+    static __device__ __forceinline__ unsigned mag(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+    static __device__ __forceinline__ int need(unsigned m) { return (int)(m >> 23) - 126; }
+    static __device__ __forceinline__ bool finite(unsigned m) { return m < 0x7f800000u; }
+    // sum over the warp, in every lane: two pieces whose 32-lane sums fit 32 bits
+    static __device__ __forceinline__ T warp_sum(T v) {
+        const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)v & 0x1ffffffu);
+        const int b = __reduce_add_sync(0xffffffffu, (int)(v >> 25));
+        return (T)b * (1 << 25) + a;
+    }
+};
+template <> struct Fix<double> {
+    using T = __int128;
+    static constexpr int kTop = 126;
+    static __device__ __forceinline__ T term(double x, int s) {
+        // from the bits: no FP64 instruction
+        const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+        const int e = (int)(u >> 52) & 0x7ff;
+        const unsigned long long m = (u & 0xfffffffffffffull) | (e ? 0x10000000000000ull : 0ull);
+        const int sh = (e ? e : 1) - 1075 + s;
+        T v = 0;
+        if (sh >= 0) v = sh < 75 ? (T)m << sh : (T)0;  // a term in range has sh <= 73
+        else if (sh > -64) v = (T)(m >> -sh);
+        return (u >> 63) ? -v : v;
+    }
+    static __device__ __forceinline__ unsigned mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+    static __device__ __forceinline__ int need(unsigned m) { return (int)(m >> 20) - 1022; }
+    static __device__ __forceinline__ bool finite(unsigned m) { return m < 0x7ff00000u; }
+    static __device__ __forceinline__ T warp_sum(T v) {
+        T r = 0;
 #pragma unroll
-    for (int j = 0; j < L; ++j) {
-        double a = j ? a1 : a0, b = j ? b1 : b0;
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_down_sync(0xffffffffu, a, o);
-            b += __shfl_down_sync(0xffffffffu, b, o);
-        }
-        if (l == 0) {
-            sh[0][w + j * (NT / 32)] = a;
-            sh[1][w + j * (NT / 32)] = b;
+        for (int k = 0; k < 4; ++k)
+            r += (T)__reduce_add_sync(0xffffffffu, (unsigned)(v >> (26 * k)) & 0x3ffffffu) << (26 * k);
+        const int c = __reduce_add_sync(0xffffffffu, (int)(v >> 104));
+        return r + (T)((unsigned __int128)(T)c << 104);
+    }
+};
+// 2^k, -1022 <= k <= 1023
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((k + 1023) << 20, 0); }
+// bits of n: the smallest l with n < 2^l
+__device__ __forceinline__ int bit_length(int n) { return 32 - __clz(n); }
+
+// ----------------------------------------------------------- CTA clusters
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ unsigned cluster_ctas() {
+    unsigned r;
+    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// v to the place of the local shared-memory word p in the cluster's CTA `rank`
+__device__ __forceinline__ void st_cluster(const void *p, unsigned rank, unsigned long long v) {
+    unsigned a = static_cast<unsigned>(__cvta_generic_to_shared(p));
+    asm volatile("mapa.shared::cluster.u32 %0, %0, %1;\n\tst.shared::cluster.u64 [%0], %2;"
+                 : "+r"(a)
+                 : "r"(rank), "l"(v)
+                 : "memory");
+}
+__device__ __forceinline__ void push_cluster(const __int128 *p, unsigned rank, __int128 v) {
+    st_cluster(p, rank, (unsigned long long)v);
+    st_cluster(reinterpret_cast<const unsigned long long *>(p) + 1, rank, (unsigned long long)(v >> 64));
+}
+
+// Partial sums of a CTA's warps, and of the cluster's CTAs (two buffers in
+// turn: a CTA may push its next partials while a slower one still reads).
+template <class T, int NW> struct SumShared {
+    T a[NW], b[NW];
+    unsigned long long m[NW];
+    T ca[2][kBeadParts], cb[2][kBeadParts];
+    unsigned long long cm[2][kBeadParts];
+};
+
+// Totals of a (and b, N = 2) and the maximum of m (N = 2) over the CTA, or
+// over all CTAs of its cluster; valid in every lane of warp 0.  Every thread
+// calls it; use = how often this CTA has called it before (the cluster's
+// first barrier phase, arrived at when the kernel starts, makes sure that
+// all CTAs run).
+template <class R, int NT, int N>
+__device__ __forceinline__ void total(typename Fix<R>::T &a, typename Fix<R>::T &b, unsigned &m,
+                                      SumShared<typename Fix<R>::T, NT / 32> &sh, int &use) {
+    using F = Fix<R>;
+    using T = typename F::T;
+    constexpr int NW = NT / 32;
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    a = F::warp_sum(a);
+    if constexpr (N == 2) {
+        b = F::warp_sum(b);
+        m = __reduce_max_sync(0xffffffffu, m);
+    }
+    if (l == 0) {
+        sh.a[w] = a;
+        if constexpr (N == 2) {
+            sh.b[w] = b;
+            sh.m[w] = m;
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double ta = 0.0, tb = 0.0;
-        for (int i = 0; i < kLaneGroups; ++i) {
-            ta += sh[0][i];
-            tb += sh[1][i];
+    if (w == 0) {
+        a = F::warp_sum(l < NW ? sh.a[l] : (T)0);
+        if constexpr (N == 2) {
+            b = F::warp_sum(l < NW ? sh.b[l] : (T)0);
+            m = __reduce_max_sync(0xffffffffu, l < NW ? (unsigned)sh.m[l] : 0u);
         }
-        ra = ta;
-        rb = tb;
+    }
+    if constexpr (std::is_same<R, double>::value) {
+        const int parts = (int)cluster_ctas();
+        if (parts > 1) {
+            const int buf = use & 1;
+            if (use == 0) cluster_wait();
+            if (w == 0 && l < parts) {
+                const unsigned me = cluster_rank();
+                push_cluster(&sh.ca[buf][me], l, a);
+                if constexpr (N == 2) {
+                    push_cluster(&sh.cb[buf][me], l, b);
+                    st_cluster(&sh.cm[buf][me], l, m);
+                }
+            }
+            __syncwarp();
+            cluster_arrive();
+            cluster_wait();
+            if (w == 0) {
+                a = F::warp_sum(l < parts ? sh.ca[buf][l] : (T)0);
+                if constexpr (N == 2) {
+                    b = F::warp_sum(l < parts ? sh.cb[buf][l] : (T)0);
+                    m = __reduce_max_sync(0xffffffffu, l < parts ? (unsigned)sh.cm[buf][l] : 0u);
+                }
+            }
+        }
+        ++use;
     }
 }
 
-// Error-free sum of two floats (Knuth): s + e == a + b exactly.
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-    s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
-}
-
-// The same for FP32 partials, with FP64-level accuracy: compensated (hi, lo)
-// float pairs inside each group of 32 lanes, FP64 for the final value.  The
-// FP64 pipe of this GPU issues a warp instruction only every few tens of
-// cycles, so FP64 is kept to the last step.  Result valid in thread 0.
-template <int NT>
-__device__ __forceinline__ void lanes_sum2f_to0(float a0, float b0, float a1, float b1, double &ra, double &rb,
-                                                double (*sh)[kLaneGroups]) {
-    constexpr int L = kBeadLanes / NT;
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    float *shf = (float *)sh;  // 4 floats a group fit in its 2 doubles
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < L; ++j) {
-        float ah = j ? a1 : a0, al = 0.f, bh = j ? b1 : b0, bl = 0.f;
-        for (int o = 16; o > 0; o >>= 1) {
-            const float oah = __shfl_down_sync(0xffffffffu, ah, o), oal = __shfl_down_sync(0xffffffffu, al, o);
-            const float obh = __shfl_down_sync(0xffffffffu, bh, o), obl = __shfl_down_sync(0xffffffffu, bl, o);
-            float s, e;
-            two_sum(ah, oah, s, e);
-            e += al + oal;
-            two_sum(s, e, ah, al);
-            two_sum(bh, obh, s, e);
-            e += bl + obl;
-            two_sum(s, e, bh, bl);
-        }
-        if (l == 0) {
-            const int g = w + j * (NT / 32);
-            shf[4 * g + 0] = ah;
-            shf[4 * g + 1] = al;
-            shf[4 * g + 2] = bh;
-            shf[4 * g + 3] = bl;
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float th = shf[0], tl = shf[1], uh = shf[2], ul = shf[3];
-        for (int i = 1; i < kLaneGroups; ++i) {
-            float s, e;
-            two_sum(th, shf[4 * i], s, e);
-            e += tl + shf[4 * i + 1];
-            two_sum(s, e, th, tl);
-            two_sum(uh, shf[4 * i + 2], s, e);
-            e += ul + shf[4 * i + 3];
-            two_sum(s, e, uh, ul);
-        }
-        ra = (double)th + (double)tl;
-        rb = (double)uh + (double)ul;
-    }
+// Release what this thread wrote and observed, add, acquire: the last
+// arrival of a counter sees what the earlier ones released.
+__device__ __forceinline__ unsigned arrive_acq_rel(unsigned *p, unsigned v) {
+    unsigned old;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
 }
 
 // d reduced to its nearest periodic image (period L = nx, or ny): the image
@@ -144,28 +214,6 @@ __device__ __forceinline__ double min_image(double d, int nx, float inv_nx) {
     const float k = rintf((float)d * inv_nx);
     return d - (double)k * (double)nx;
 }
-// A box widened by one cell on every side: wrapped (x, and y when periodic),
-// clipped at the walls, covering each direction at most once.
-__device__ __forceinline__ Box widen_box(const Inst &I, Box b) {
-    if (b.w <= 0 || b.h <= 0) return b;
-    if (b.w < I.nx) {
-        b.i0 = (b.i0 == 0) ? I.nx - 1 : b.i0 - 1;
-        b.w = (b.w + 2 < I.nx) ? b.w + 2 : I.nx;
-    }
-    if (I.periodic_y) {
-        if (b.h < I.ny) {
-            b.j0 = (b.j0 == 0) ? I.ny - 1 : b.j0 - 1;
-            b.h = (b.h + 2 < I.ny) ? b.h + 2 : I.ny;
-        }
-    } else {
-        const int lo = b.j0 > 0 ? b.j0 - 1 : 0;
-        const int hi = (b.j0 + b.h < I.ny) ? b.j0 + b.h : I.ny - 1;
-        b.j0 = lo;
-        b.h = hi - lo + 1;
-    }
-    return b;
-}
-
 // the same for the y separation, applied only when y is periodic
 __device__ __forceinline__ double min_image_y(const Inst &I, double d) {
     return I.periodic_y ? min_image(d, I.ny, I.f_inv_ny) : d;
@@ -174,604 +222,706 @@ __device__ __forceinline__ float min_image_yf(const Inst &I, float d) {
     return I.periodic_y ? d - (float)I.ny * rintf(d * I.f_inv_ny) : d;
 }
 
-// Force on bead q (instance-local index), given the instance's positions
-// and the unit tangents/lengths of every segment (index j joins beads j and
-// j+1 of the instance-local numbering), all staged in shared memory.
-__device__ __forceinline__ void bead_force(const Inst &I, const double *Rx, const double *Ry, const float *Xf,
-                                           const float *Yf, const double *Tx, const double *Ty, const double *Ln, int q,
-                                           double &Fx, double &Fy) {
-    const int N = I.n_beads;
-    const int fib = q / N, i0 = q - fib * N;  // 0-based index within the fiber
-    // segments around bead q, as in Eqs. 11-12 with 1-based i = i0 + 1:
-    // t_{i-2}, t_{i-1} (ends at q), t_i (starts at q), t_{i+1}; missing = 0
-    const bool h_m2 = i0 >= 2, h_m1 = i0 >= 1, h_i = i0 <= N - 2, h_p1 = i0 + 1 <= N - 2;
-    const double tm2x = h_m2 ? Tx[q - 2] : 0.0, tm2y = h_m2 ? Ty[q - 2] : 0.0;
-    const double tm1x = h_m1 ? Tx[q - 1] : 0.0, tm1y = h_m1 ? Ty[q - 1] : 0.0;
-    const double tix = h_i ? Tx[q] : 0.0, tiy = h_i ? Ty[q] : 0.0;
-    const double tp1x = h_p1 ? Tx[q + 1] : 0.0, tp1y = h_p1 ? Ty[q + 1] : 0.0;
-    const double ks = I.ks_l02;
-    Fx = 0.0;
-    Fy = 0.0;
-    if (h_m1) {
-        const double Lm1 = Ln[q - 1];
-        // Eq. 11, spring to the previous bead
-        Fx -= ks * (Lm1 - I.l0) * tm1x;
-        Fy -= ks * (Lm1 - I.l0) * tm1y;
-        // Eq. 12, first term: (t_i + t_{i-2}).(I - t_{i-1} t_{i-1}) / R_{i-1,i}
-        const double vx = tix + tm2x, vy = tiy + tm2y;
-        const double vt = vx * tm1x + vy * tm1y;
-        Fx += I.k_b * (vx - vt * tm1x) / Lm1;
-        Fy += I.k_b * (vy - vt * tm1y) / Lm1;
-    }
-    if (h_i) {
-        const double Li = Ln[q];
-        // Eq. 11, spring to the next bead
-        Fx += ks * (Li - I.l0) * tix;
-        Fy += ks * (Li - I.l0) * tiy;
-        // Eq. 12, second term: -(t_{i+1} + t_{i-1}).(I - t_i t_i) / R_{i,i+1}
-        const double vx = tp1x + tm1x, vy = tp1y + tm1y;
-        const double vt = vx * tix + vy * tiy;
-        Fx -= I.k_b * (vx - vt * tix) / Li;
-        Fy -= I.k_b * (vy - vt * tiy) / Li;
-    }
-    // excluded volume between beads that share no spring; an FP32 distance
-    // test (1% margin) selects the pairs evaluated in FP64
-    if (I.k_ev != 0.0) {
-        const double Rqx = Rx[q], Rqy = Ry[q];
-        const float l0f2 = (float)(I.l0 * I.l0) * 1.0201f;
-        const float fnx = (float)I.nx;
+// Excluded-volume candidates of every bead of the instance into cand: beads
+// that share no spring with it, nearer than l0 by an FP32 distance test with
+// 1% margin.  Xf, Yf: positions relative to bead 0 of the instance.  Warp w
+// of NW screens for beads w, w + NW, ..., 32 beads at a time.
+template <int NW>
+__device__ __forceinline__ void screen_close(const Inst &I, const float *Xf, const float *Yf, unsigned *cand) {
+    const int N = I.n_beads, nb = I.nb, nw = (nb + 31) / 32;
+    const int lane = threadIdx.x & 31;
+    const float l0s2 = I.f_l0 * I.f_l0 * 1.0201f, fnx = (float)I.nx;
+    for (int q = threadIdx.x >> 5; q < nb; q += NW) {
+        const int lo = q / N * N;
         const float xq = Xf[q], yq = Yf[q];
-        const int lo = fib * N;
-        for (int p = 0; p < I.nb; ++p) {
-            float fx = xq - Xf[p];
-            fx -= fnx * rintf(fx * I.f_inv_nx);
-            const float fy = min_image_yf(I, yq - Yf[p]);
-            if (fx * fx + fy * fy >= l0f2) continue;
-            if (p == q || (p >= lo && p < lo + N && abs(p - q) < 2)) continue;
-            const double dx = min_image(Rqx - Rx[p], I.nx, I.f_inv_nx);
-            const double dy = min_image_y(I, Rqy - Ry[p]);
-            const double r = sqrt(dx * dx + dy * dy);
-            if (r < I.l0 && r > 0.0) {
-                const double m = I.k_ev * (I.l0 - r) / r;
-                Fx += m * dx;
-                Fy += m * dy;
-            }
-        }
-    }
-    // constant external force F_0 (driven particle, Sec. 3.2)
-    Fx += I.ext_fx;
-    Fy += I.ext_fy;
-}
-
-// FP32 version of bead_force for the reduced-precision paths.  Positions
-// stay FP64; each segment's tangent and length are FP32, and its stretch
-// L - l0 = (|d|^2 - l0^2) / (L + l0) is formed from the FP64 |d|^2 so that
-// the small strain of a stiff spring does not cancel away in FP32.
-__device__ __forceinline__ void bead_force_f32(const Inst &I, const double *Rx, const double *Ry, const float *Xf,
-                                               const float *Yf, const float *Tx, const float *Ty, const float *Ln,
-                                               const float *Dl, int q, float &Fx, float &Fy) {
-    // the record's fields in registers, the force in local accumulators:
-    // with stores through Fx, Fy inside the loop the fields would be
-    // reloaded from the shared record on every pass
-    const int N = I.n_beads, nb = I.nb, nx = I.nx, ny = I.ny;
-    const bool py = I.periodic_y != 0;
-    const float inv_nx = I.f_inv_nx, inv_ny = I.f_inv_ny, fnx = (float)nx, fny = (float)ny;
-    const int fib = q / N, i0 = q - fib * N;
-    const bool h_m2 = i0 >= 2, h_m1 = i0 >= 1, h_i = i0 <= N - 2, h_p1 = i0 + 1 <= N - 2;
-    const float tm2x = h_m2 ? Tx[q - 2] : 0.f, tm2y = h_m2 ? Ty[q - 2] : 0.f;
-    const float tm1x = h_m1 ? Tx[q - 1] : 0.f, tm1y = h_m1 ? Ty[q - 1] : 0.f;
-    const float tix = h_i ? Tx[q] : 0.f, tiy = h_i ? Ty[q] : 0.f;
-    const float tp1x = h_p1 ? Tx[q + 1] : 0.f, tp1y = h_p1 ? Ty[q + 1] : 0.f;
-    const float ks = I.f_ks_l02, kb = I.f_kb;
-    float ax = 0.f, ay = 0.f;
-    if (h_m1) {
-        const float Lm1 = Ln[q - 1], dl = Dl[q - 1];
-        ax -= ks * dl * tm1x;
-        ay -= ks * dl * tm1y;
-        const float vx = tix + tm2x, vy = tiy + tm2y;
-        const float vt = vx * tm1x + vy * tm1y;
-        ax += kb * (vx - vt * tm1x) / Lm1;
-        ay += kb * (vy - vt * tm1y) / Lm1;
-    }
-    if (h_i) {
-        const float Li = Ln[q], dl = Dl[q];
-        ax += ks * dl * tix;
-        ay += ks * dl * tiy;
-        const float vx = tp1x + tm1x, vy = tp1y + tm1y;
-        const float vt = vx * tix + vy * tiy;
-        ax -= kb * (vx - vt * tix) / Li;
-        ay -= kb * (vy - vt * tiy) / Li;
-    }
-    if (I.k_ev != 0.0) {
-        // Xf, Yf: positions relative to bead 0 of the instance in FP32 (a
-        // screen with 1% margin); a candidate pair is evaluated from the
-        // FP64 positions
-        const float l0 = I.f_l0, l0s2 = l0 * l0 * 1.0201f, kev = I.f_kev;
-        const float xq = Xf[q], yq = Yf[q];
-        const double Rqx = Rx[q], Rqy = Ry[q];
-        const int lo = fib * N;
-        // screen 32 beads at a time without branches (independent passes
-        // the compiler can overlap), then evaluate the few candidates in
-        // bead order
-        for (int p0 = 0; p0 < nb; p0 += 32) {
-            const int pn = min(32, nb - p0);
-            unsigned cand = 0u;
-#pragma unroll 8
-            for (int k = 0; k < pn; ++k) {
-                const int p = p0 + k;
+        for (int c = 0; c < nw; ++c) {
+            const int p = 32 * c + lane;
+            bool near = false;
+            if (p < nb) {
                 float fx = xq - Xf[p];
-                fx -= fnx * rintf(fx * inv_nx);
-                float fy = yq - Yf[p];
-                if (py) fy -= fny * rintf(fy * inv_ny);
+                fx -= fnx * rintf(fx * I.f_inv_nx);
+                const float fy = min_image_yf(I, yq - Yf[p]);
                 const bool bonded = p == q || (p >= lo && p < lo + N && abs(p - q) < 2);
-                cand |= (unsigned)(fx * fx + fy * fy < l0s2 && !bonded) << k;
+                near = fx * fx + fy * fy < l0s2 && !bonded;
             }
-            while (cand) {
-                const int p = p0 + __ffs(cand) - 1;
-                cand &= cand - 1u;
-                const double dx = min_image(Rqx - Rx[p], nx, inv_nx);
-                const double dy = py ? min_image(Rqy - Ry[p], ny, inv_ny) : Rqy - Ry[p];
-                const float r = sqrtf((float)(dx * dx + dy * dy));
-                if (r < l0 && r > 0.f) {
-                    const float m = kev * (l0 - r) / r;
-                    ax += m * (float)dx;
-                    ay += m * (float)dy;
-                }
-            }
+            const unsigned m = __ballot_sync(0xffffffffu, near);
+            if (lane == 0) cand[q * nw + c] = m;
         }
     }
-    Fx = ax + I.f_ext_fx;
-    Fy = ay + I.f_ext_fy;
 }
 
-// CTA c handles beads c, c + gridDim.x, ... of the list, so any grid size
-// covers every bead; the launcher gives each bead its own CTA.
+// Excluded volume on bead q along axis ax (0 x, 1 y) from the beads in its
+// candidate words, in bead order; r: interleaved x, y positions.
+template <class R>
+__device__ __forceinline__ R close_force(const Inst &I, const double *r, const unsigned *cand, int q, int ax) {
+    const int nw = (I.nb + 31) / 32;
+    R f = (R)0;
+    for (int c = 0; c < nw; ++c)
+        for (unsigned bits = cand[q * nw + c]; bits; bits &= bits - 1u) {
+            const int p = 32 * c + __ffs(bits) - 1;
+            const double dx = min_image(r[2 * q] - r[2 * p], I.nx, I.f_inv_nx);
+            const double dy = min_image_y(I, r[2 * q + 1] - r[2 * p + 1]);
+            if constexpr (std::is_same<R, double>::value) {
+                const double d = sqrt(dx * dx + dy * dy);
+                if (d < I.l0 && d > 0.0) f += I.k_ev * (I.l0 - d) / d * (ax ? dy : dx);
+            } else {
+                const float d = sqrtf((float)(dx * dx + dy * dy));
+                if (d < I.f_l0 && d > 0.f) f += I.f_kev * (I.f_l0 - d) / d * (float)(ax ? dy : dx);
+            }
+        }
+    return f;
+}
+
+// A support cell of the bead: phi of this bead, the spread force density
+// there (Eq. 4 with the previous table), the cell's element offset in plane
+// 0 and whether it lies in the lattice's first / last column / row (bits).
+template <class R> struct alignas(16) SupportCell {
+    R phi, fx, fy;
+    int o, edge;
+};
+template <> struct alignas(16) SupportCell<float> {
+    float phi, fx, fy;
+    int o;
+};
+constexpr int kEdgeL = 1, kEdgeR = 2, kEdgeB = 4, kEdgeT = 8;
+// Another bead whose support can overlap the bead's: the offset from it
+// (FP32 paths) or its position (FP64), and its G.
+template <class R> struct alignas(4 * sizeof(R)) Neighbour {
+    R x, y, gx, gy;
+};
+// Box cells listed at a time (a support box of the usual beads fits at once:
+// 29 x 29 cells for a = 4, xi = 1).
+template <class R> struct ListCap { static constexpr int value = std::is_same<R, double>::value ? 1024 : 1280; };
+
+// The last CTA's view of its instance, in the shared memory the list took;
+// x and y of a bead or segment side by side.
+template <class R> struct ForceShared {
+    double r[2 * kMaxBeads], S[kMaxBeads];
+    float xf[kMaxBeads], yf[kMaxBeads];
+    R t[2 * kMaxBeads], pull[2 * kMaxBeads], len[kMaxBeads], str[kMaxBeads];
+    unsigned cand[kMaxBeads * (kMaxBeads / 32)];
+};
+
+// A bead's support box in the lattice: first column and row (wrapped), size,
+// and the first cell's centre less the bead's position; [0] x, [1] y.
+struct Support {
+    int lo[2], n[2];
+    float rel[2];
+};
+// Row and column of box cell c; rows by an FP32 reciprocal, exact below 2^19
+// cells (two ulps of c / w stay below half of 1 / w), else by division.
+__device__ __forceinline__ void cell_rc(const Support &b, const float inv_w, int c, int &ci, int &cj) {
+    cj = inv_w != 0.0f ? (int)(((float)c + 0.5f) * inv_w) : c / b.n[0];
+    ci = c - cj * b.n[0];
+}
+__device__ __forceinline__ float inv_width(const Support &b) {
+    return b.n[0] * (int64_t)b.n[1] < (1 << 19) ? 1.0f / (float)b.n[0] : 0.0f;
+}
+// One axis (ax: 0 x, 1 y) of the support box of a bead at h + l on it, in
+// FP32 with a cell of margin as support_box; positions of a million cells or
+// more, or not finite, take support_box of the FP64 position (Rx, Ry).
+__device__ __forceinline__ void support_axis(const Inst &I, int ax, float h, float l, bool far, double Rx, double Ry,
+                                             int &lo, int &n, float &rel) {
+    if (far) {
+        const Box b = support_box(I, Rx, Ry);
+        lo = ax ? b.j0 : b.i0;
+        n = b.w > 0 && b.h > 0 ? (ax ? b.h : b.w) : 0;
+        rel = ax ? (float)(b.ju + 0.5 - Ry) : (float)(b.iu + 0.5 - Rx);
+        return;
+    }
+    const int L = ax ? I.ny : I.nx;
+    int a = (int)floorf(h - I.f_rcut - 0.5f) - 1, b = (int)ceilf(h + I.f_rcut - 0.5f) + 1;
+    if (ax && !I.periodic_y) {
+        a = max(a, 0);
+        b = min(b, L - 1);
+    } else if (b - a + 1 >= L) {
+        a = (int)floorf(h - 0.5f * (float)L);
+        b = a + L - 1;
+    }
+    n = max(b - a + 1, 0);
+    rel = ((float)a + 0.5f - h) - l;
+    if (a < 0) a += L;
+    else if (a >= L) a -= L;
+    if ((unsigned)a >= (unsigned)L) a = ((a % L) + L) % L;
+    lo = a;
+}
+__device__ __forceinline__ bool far_off(float xh, float yh) { return !(fabsf(xh) < 1.0e6f && fabsf(yh) < 1.0e6f); }
+
+// A support box widened by one cell on every side: wrapped (x, and y when
+// periodic), clipped at the walls, covering each direction at most once.
+__device__ __forceinline__ Support widen(const Inst &I, Support b) {
+    if (b.n[0] <= 0 || b.n[1] <= 0) return b;
+    for (int ax = 0; ax < 2; ++ax) {
+        const int L = ax ? I.ny : I.nx;
+        if (ax && !I.periodic_y) {
+            const int lo = max(b.lo[1] - 1, 0), hi = min(b.lo[1] + b.n[1], L - 1);
+            b.lo[1] = lo;
+            b.n[1] = hi - lo + 1;
+        } else if (b.n[ax] < L) {
+            b.lo[ax] = (b.lo[ax] == 0) ? L - 1 : b.lo[ax] - 1;
+            b.n[ax] = min(b.n[ax] + 2, L);
+        }
+    }
+    return b;
+}
+
+// Populations of a support cell, g_k.
+template <class S, class R>
+__device__ __forceinline__ void pull_support(const S *__restrict__ A, const Inst &I, const int o, const int edge,
+                                             R g[9]) {
+    const int x = o & 31;  // column within the strip
+    if (edge == 0) {
+        pull_inner<S, R>(A + o, strip_left(I, x), strip_right(I, x), I, g);
+        return;
+    }
+    Cell C;
+    C.o = o;
+    const int last = col_off(I, I.nx - 1);
+    C.shl = (edge & kEdgeL) ? last + 1 : strip_left(I, x);
+    C.shr = (edge & kEdgeR) ? -last - 1 : strip_right(I, x);
+    C.y0 = edge & kEdgeB;
+    C.yn = edge & kEdgeT;
+    C.bot = C.y0 && !I.periodic_y;
+    C.top = C.yn && !I.periodic_y;
+    pull_pops<S, R>(A, I, C, g);
+}
+
 // Resident bead CTAs per SM the reduced-precision kernels are held to (80
-// registers a thread), so that large bead lists of a batch run in few waves;
-// the FP64 parity path keeps its registers.
-template <class S, int NT> struct BeadMinBlocks { static constexpr int value = 6 * kBeadThreads / NT; };
+// registers a thread at 128 threads), so that large bead lists of a batch
+// run in few waves; the FP64 parity path keeps its registers.
+template <class S, int NT> struct BeadMinBlocks { static constexpr int value = 6 * kBeadThreads / NT > 1 ? 6 * kBeadThreads / NT : 2; };
 template <int NT> struct BeadMinBlocks<double, NT> { static constexpr int value = 1; };
 
 // NT threads per bead CTA: kBeadThreads for long bead lists (more CTAs
-// resident), kBeadThreadsFew when every bead has an SM of its own (shorter
-// per-bead loops).
+// resident), more when every bead has an SM of its own (shorter per-bead
+// loops).  A cluster's CTAs (FP64) each take a share of the bead's cells.
+// wait_first: wait for the sweep before listing the support (launch_beads).
 template <class S, int NT>
 __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
-    k_beads(const Inst *__restrict__ insts, const int2 *__restrict__ blist, const int nb_total,
-            const S *__restrict__ pool, const BeadTab tab0, const BeadTab tab1, unsigned *__restrict__ mask_write,
-            int gparity, int advance, unsigned *__restrict__ counters, BeadExport ex,
-            unsigned *__restrict__ status) {
+    k_beads(const Inst *__restrict__ insts, const int4 *__restrict__ blist, const S *__restrict__ pool,
+            const BeadTab tab0, const BeadTab tab1, const typename PhiArg<S>::type phi0,
+            const typename PhiArg<S>::type phi1, unsigned *__restrict__ mask_write, int gparity, int advance,
+            int wait_first, unsigned *__restrict__ counters, BeadExport ex, unsigned *__restrict__ status) {
     constexpr bool kF64 = std::is_same<S, double>::value;
+    using R = typename std::conditional<kF64, double, float>::type;
+    using F = Fix<R>;
+    using T = typename F::T;
+    constexpr int NW = NT / 32;
+    constexpr int kCap = ListCap<R>::value;
+    constexpr size_t kBuf = sizeof(SupportCell<R>) * kCap > sizeof(ForceShared<R>) ? sizeof(SupportCell<R>) * kCap
+                                                                                   : sizeof(ForceShared<R>);
     __shared__ Inst sI;
-    // neighbour beads: old-table position (FP64 path), offset R_b - R_q and
-    // spreading coefficients (FP32 paths); reused by the last CTA to stage
-    // positions, support sums and segment tangents
-    __shared__ double s_rx[kMaxBeads], s_ry[kMaxBeads], s_gx[kMaxBeads], s_gy[kMaxBeads];
-    __shared__ double s_tx[kMaxBeads], s_ty[kMaxBeads], s_ln[kMaxBeads];
-    __shared__ float s_ox[kMaxBeads], s_oy[kMaxBeads], s_gxf[kMaxBeads], s_gyf[kMaxBeads];
-    __shared__ float s_xf[kMaxBeads], s_yf[kMaxBeads];
-    constexpr int kWarps = NT / 32;
-    __shared__ double sh[2][kLaneGroups];
-    // virtual lanes a thread holds (partials 0 and 1: lanes tid, tid + NT)
-    constexpr int kL = kBeadLanes / NT;
-    __shared__ double s_R[2];
-    __shared__ float s_rel[2];
-    __shared__ Box s_box;
-    __shared__ double s_invS;
-    __shared__ unsigned s_hits[kMaxBeads / 32];
-    __shared__ int s_last, s_nn;
-    __shared__ unsigned s_stold;
+    __shared__ __align__(16) unsigned char s_buf[kBuf];
+    __shared__ unsigned char s_edge[kF64 ? 1 : kCap];
+    __shared__ Neighbour<R> s_nbr[kMaxBeads];
+    __shared__ int4 s_nbox[kF64 ? kMaxBeads : 1];  // a neighbour's kept box, and where its profile starts
+    __shared__ int s_noff[kF64 ? kMaxBeads : 1];
+    __shared__ SumShared<T, NW> s_sum;
+    __shared__ double s_R[2], s_unit;
+    __shared__ Support s_sup;
+    __shared__ int s_n, s_redo;
+    __shared__ unsigned s_seen;
+    SupportCell<R> *list = reinterpret_cast<SupportCell<R> *>(s_buf);
 
-    // wait for the preceding sweep (the populations read below, and through
-    // it the previous bead phase), then let the next sweep launch at once:
-    // its tiles that no bead marked start while this phase runs, and the
-    // set-up below (record copy, neighbour screen) does not delay them
-    pdl_wait();
-    pdl_trigger();
-    for (int it = blockIdx.x; it < nb_total; it += gridDim.x) {
-    __syncthreads();  // the shared state of the previous bead is no longer read
-    // blist[i] = (instance slot, global bead index); NULL: instance 0, bead i
-    const int2 bi = blist ? blist[it] : make_int2(0, it);
-    const int ii = bi.x, b = bi.y;
-    const int tid = threadIdx.x;
-    // this instance's step parity selects the table pair and the population
-    // buffer; it is read from the global record so that the old table's
-    // loads below need not wait for the shared copy
-    const int parity = gparity ^ insts[ii].par_xor;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int parts = kF64 ? (int)cluster_ctas() : 1, part = kF64 ? (int)cluster_rank() : 0;
+    if (parts > 1) cluster_arrive();  // waited for by the first total()
+    int uses = 0;
+    // blist[i] = (2 slot + par_xor, global bead index, the instance's first
+    // bead and bead count); NULL: instance 0, bead i
+    const int it = blockIdx.x / parts;
+    const int4 br = blist ? blist[it] : make_int4(0, it, 0, gridDim.x / parts);
+    const int ii = br.x >> 1, b = br.y, first = br.z, nb = br.w;
+    // this instance's step parity selects the table pair and the population buffer
+    const int parity = gparity ^ (br.x & 1);
     const BeadTab &told = parity ? tab0 : tab1;
     const BeadTab &tnew = parity ? tab1 : tab0;
+    const typename PhiArg<S>::type &pold = parity ? phi0 : phi1, &pnew = parity ? phi1 : phi0;
+    if (advance && wait_first) {
+        pdl_wait();
+        pdl_trigger();
+    }
     {
         // cooperative copy of the instance record (one 32-bit word a thread)
         static_assert(sizeof(Inst) % 4 == 0, "Inst is copied as 32-bit words");
         const unsigned *src = (const unsigned *)(insts + ii);
         unsigned *dst = (unsigned *)&sI;
-        for (int wd = tid; wd < (int)(sizeof(Inst) / 4); wd += blockDim.x) dst[wd] = src[wd];
+        for (int wd = tid; wd < (int)(sizeof(Inst) / 4); wd += NT) dst[wd] = src[wd];
     }
-    // the bead's old position (every thread) and support sum
-    double Rx = 0.0, Ry = 0.0, S_old = 1.0;
+    // Up to pdl_wait() only the records and the old table are read: the
+    // preceding launch, a sweep, may still be running, but it was released
+    // after the bead phase that wrote this table had completed (its lead CTA
+    // waits for it).  Table reads go to L2 (an SM's L1 may hold lines of an
+    // earlier step).
+    int any_close = 0;  // some bead may come within the excluded volume's reach of this one
+    double Rx = 0.0, Ry = 0.0;  // the bead's old position
+    float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f;
     if (advance) {
-        Rx = told.Rx[b];
-        Ry = told.Ry[b];
-        if (tid == 0) S_old = told.S[b];
+        xh = __ldcg(told.xh + b);
+        xl = __ldcg(told.xl + b);
+        yh = __ldcg(told.yh + b);
+        yl = __ldcg(told.yl + b);
+        Rx = __ldcg(told.Rx + b);
+        Ry = __ldcg(told.Ry + b);
+        if (tid == NT - 1) s_unit = 1.0 / __ldcg(told.S + b);
     }
-    __syncthreads();
+    // the lattice cell of row cj, column ci of a support box
+    auto cell_of = [](const Inst &I, const Support &bx, int ci, int cj, int &i, int &j) {
+        j = bx.lo[1] + cj;
+        j = (j >= I.ny) ? j - I.ny : j;
+        i = bx.lo[0] + ci;
+        i = (i >= I.nx) ? i - I.nx : i;
+    };
     const Inst &I = sI;
-    // populations are pulled from the current buffer (the instance's parity)
-    const S *A = pop_buffer(pool, I, parity);
-
     if (advance) {
-        if (tid == 0) {
-            const Box bx = support_box(I, Rx, Ry);
-            s_box = bx;
-            s_rel[0] = (float)(bx.iu + 0.5 - Rx);
-            s_rel[1] = (float)(bx.ju + 0.5 - Ry);
-            s_invS = 1.0 / S_old;
-        }
-        {
-            // beads whose support can overlap b's (FP32 screen, 1-cell
-            // margin), listed in bead order: warp w screens the 32-bead
-            // chunks w, w + kWarps, ...; a chunk's hit mask places its hits
-            // after those of the chunks before it
-            const float reach = 2.0f * I.f_rcut + 1.0f, fnx = (float)I.nx;
-            const int lane = tid & 31, w = tid >> 5;
-            const int nchunks = (I.nb + 31) / 32;
-            int n = 0;
-            for (int r0 = 0; r0 < nchunks; r0 += kWarps) {
-                const int c = r0 + w, q = 32 * c + lane;
-                bool hit = false;
-                double qx = 0.0, qy = 0.0, gx = 0.0, gy = 0.0;
-                if (q < I.nb) {
-                    qx = told.Rx[I.bead_off + q];
-                    qy = told.Ry[I.bead_off + q];
-                    gx = told.Gx[I.bead_off + q];
-                    gy = told.Gy[I.bead_off + q];
-                    float dx = (float)(qx - Rx);
-                    dx -= fnx * rintf(dx * I.f_inv_nx);
-                    const float dy = min_image_yf(I, (float)(qy - Ry));
-                    hit = dx * dx + dy * dy < reach * reach;
+        // beads whose support can overlap b's (FP32 screen, 1-cell margin),
+        // in bead order; every warp screens all of them, 32 at a time, so
+        // that no barrier is needed, and warp 0 lists them
+        int nn = 0, self = 0;  // neighbours, the bead's own place among them
+        int fiber = 0;         // first bead of its fiber
+        for (int q0 = 0; q0 < nb; q0 += 32) {
+            const int q = q0 + lane, gq = first + q;
+            float dx = 0.f, dy = 0.f;
+            Neighbour<R> nbr{};
+            int4 qbox = make_int4(0, 0, 0, 0);
+            if (q < nb) {
+                dx = xh - __ldcg(told.xh + gq);
+                const float lx = xl - __ldcg(told.xl + gq);
+                dy = yh - __ldcg(told.yh + gq);
+                const float ly = yl - __ldcg(told.yl + gq);
+                if constexpr (kF64) {
+                    if (pold.box) qbox = __ldcg(pold.box + gq);
+                    nbr.x = __ldcg(told.Rx + gq);
+                    nbr.y = __ldcg(told.Ry + gq);
+                    nbr.gx = __ldcg(told.Gx + gq);
+                    nbr.gy = __ldcg(told.Gy + gq);
+                } else {
+                    nbr.x = lx;
+                    nbr.y = ly;
+                    nbr.gx = __ldcg(told.gxf + gq);
+                    nbr.gy = __ldcg(told.gyf + gq);
                 }
-                const unsigned m = __ballot_sync(0xffffffffu, hit);
-                if (lane == 0 && c < nchunks) s_hits[c] = m;
-                __syncthreads();
-                if (hit) {
-                    int pos = n + __popc(m & ((1u << lane) - 1u));
-                    for (int cc = r0; cc < c; ++cc) pos += __popc(s_hits[cc]);
-                    s_rx[pos] = qx;
-                    s_ry[pos] = qy;
-                    s_ox[pos] = (float)min_image(Rx - qx, I.nx, I.f_inv_nx);
-                    s_oy[pos] = (float)min_image_y(I, Ry - qy);
-                    s_gx[pos] = gx;
-                    s_gy[pos] = gy;
-                    s_gxf[pos] = (float)gx;
-                    s_gyf[pos] = (float)gy;
-                }
-                for (int cc = r0; cc < r0 + kWarps && cc < nchunks; ++cc) n += __popc(s_hits[cc]);
-                __syncthreads();  // s_hits is rewritten by the next round
             }
-            if (tid == 0) s_nn = n;
+            if (q0 == 0) __syncthreads();  // the record is in place
+            // nearest image of the bead from bead q: the high parts' image
+            // shift is a whole number of cells, removed exactly
+            const float fnx = (float)I.nx, fny = (float)I.ny;
+            dx -= fnx * rintf(dx * I.f_inv_nx);
+            if (I.periodic_y) dy -= fny * rintf(dy * I.f_inv_ny);
+            const float d2 = dx * dx + dy * dy, reach = 2.0f * I.f_rcut + 1.0f;
+            const bool hit = q < nb && (d2 < reach * reach || gq == b);  // itself even if not finite
+            const unsigned m = __ballot_sync(0xffffffffu, hit);
+            // two beads that move less than half a cell per component come
+            // at most 1.42 cells nearer in this phase
+            const float lim = I.f_l0 + 1.5f;
+            if (q0 == 0) fiber = (b - first) / I.n_beads * I.n_beads;
+            const bool bonded = abs(gq - b) < 2 && q >= fiber && q < fiber + I.n_beads;
+            any_close |= __any_sync(0xffffffffu, q < nb && !bonded && d2 < lim * lim);
+            const int lb = b - first - q0;
+            if ((unsigned)lb < 32u) self = nn + __popc(m & ((1u << lb) - 1u));
+            if (hit && w == 0) {
+                const int pos = nn + __popc(m & ((1u << lane) - 1u));
+                if constexpr (!kF64) {
+                    nbr.x += dx;
+                    nbr.y += dy;
+                }
+                s_nbr[pos] = nbr;
+                if constexpr (kF64) {
+                    s_nbox[pos] = qbox;
+                    s_noff[pos] = I.phi_off + q * I.phi_cap;
+                }
+            }
+            nn += __popc(m);
         }
-        __syncthreads();
-        const int nn = s_nn;
-        const Box bx = s_box;
-        const float rel0x = s_rel[0], rel0y = s_rel[1];
-        const float hnx = 0.5f * (float)I.nx, fnx = (float)I.nx;
-        const float hny = 0.5f * (float)I.ny, fny = (float)I.ny;
-        // per-lane partials (FP32 paths: few terms a lane); cell c belongs
-        // to partial (c / NT) % kL of its thread
-        double ax0 = 0.0, ay0 = 0.0, ax1 = 0.0, ay1 = 0.0;
-        float axf0 = 0.0f, ayf0 = 0.0f, axf1 = 0.0f, ayf1 = 0.0f;
-        // the box row and column of box cell c, wrapped into the lattice
-        auto cell_ij = [&](int c, int &ci, int &cj, int &i, int &j) {
-            cj = c / bx.w;
-            ci = c - cj * bx.w;
-            j = bx.j0 + cj;
-            j = (j >= I.ny) ? j - I.ny : j;
-            i = bx.i0 + ci;
-            i = (i >= I.nx) ? i - I.nx : i;
-        };
-        if constexpr (kF64) {
-            for (int c = tid; c < bx.w * bx.h; c += blockDim.x) {
-                int ci, cj, i, j;
-                cell_ij(c, ci, cj, i, j);
-                const double xc = i + 0.5, yc = j + 0.5;
-                const double phb = phi_f64(I, xc, yc, Rx, Ry);
-                if (phb == 0.0) continue;
-                double g[9];
-                pull_pops<S, double>(A, I, make_cell(I, i, j), g);
-                double dr = 0.0;
-#pragma unroll
-                for (int k = 0; k < 9; ++k) dr += g[k];
-                const double rho = 1.0 + dr;
-                const double jx = g[1] - g[3] + g[5] - g[6] - g[7] + g[8];
-                const double jy = g[2] - g[4] + g[5] + g[6] - g[7] - g[8];
-                double fx = I.gx, fy = I.gy;
-                for (int q = 0; q < nn; ++q) {
-                    const double ph = phi_f64(I, xc, yc, s_rx[q], s_ry[q]);
-                    if (ph != 0.0) {
-                        fx += ph * s_gx[q];
-                        fy += ph * s_gy[q];
+        if constexpr (kF64) __syncthreads();  // the neighbours are in place (FP32: make_list's barrier)
+        // populations are pulled from the current buffer
+        const S *A = pop_buffer(pool, I, parity);
+        const bool kept = kF64 && I.phi_cap != 0;
+        Support bx;
+        if (kept) {
+            const int4 kb = s_nbox[self];
+            bx.lo[0] = kb.x, bx.lo[1] = kb.y;
+            bx.n[0] = kb.z, bx.n[1] = kb.w;
+        } else {
+            const bool far = far_off(xh, yh);
+            support_axis(I, 0, xh, xl, far, Rx, Ry, bx.lo[0], bx.n[0], bx.rel[0]);
+            support_axis(I, 1, yh, yl, far, Rx, Ry, bx.lo[1], bx.n[1], bx.rel[1]);
+        }
+        const float inv_w = inv_width(bx);
+        // List the support cells (phi_b != 0) among box cells [c0, c1),
+        // c1 - c0 <= kCap, with the force density of the previous table.
+        // Their order differs from run to run; the sums do not depend on it.
+        auto make_list = [&](int c0, int c1) -> int {
+            if (tid == 0) s_n = 0;
+            __syncthreads();
+#pragma unroll 1
+            for (int cb = c0 + 32 * w; cb < c1; cb += NT) {
+                const int c = cb + lane;
+                R ph = (R)0;
+                if (c < c1) {
+                    int ci, cj;
+                    cell_rc(bx, inv_w, c, ci, cj);
+                    if constexpr (kF64) {
+                        if (kept) {
+                            ph = __ldcg(pold.phi + s_noff[self] + c);
+                        } else {
+                            int i, j;
+                            cell_of(I, bx, ci, cj, i, j);
+                            ph = phi_f64(I, i + 0.5, j + 0.5, Rx, Ry);
+                        }
+                    } else {
+                        ph = phi_f32(bx.rel[0] + (float)ci, bx.rel[1] + (float)cj, I.f_a, I.f_inv_xi, I.f_rcut2);
                     }
                 }
-                if ((c / NT) % kL) {
-                    ax1 += phb * ((jx + 0.5 * fx) / rho);
-                    ay1 += phb * ((jy + 0.5 * fy) / rho);
-                } else {
-                    ax0 += phb * ((jx + 0.5 * fx) / rho);
-                    ay0 += phb * ((jy + 0.5 * fy) / rho);
+                const unsigned m = __ballot_sync(0xffffffffu, ph != (R)0);
+                int at = 0;
+                if (lane == 0) at = atomicAdd(&s_n, __popc(m));
+                at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+                if (ph != (R)0) {
+                    list[at].phi = ph;
+                    list[at].o = c;
                 }
             }
-        } else {
-            // each thread visits its cells c = tid, tid + blockDim.x, ...
-            // with phi_b != 0, loading the populations of the next such cell
-            // before it works on the current one
-            const int ncell = bx.w * bx.h;
-            auto seek = [&](int &c, float &dx, float &dy, float &phb) {
-                for (; c < ncell; c += blockDim.x) {
-                    const int cj = c / bx.w, ci = c - cj * bx.w;
-                    dx = rel0x + (float)ci;
-                    dy = rel0y + (float)cj;
-                    phb = phi_f32(dx, dy, I.f_a, I.f_inv_xi, I.f_rcut2);
-                    if (phb != 0.0f) return;
-                }
-            };
-            auto load = [&](int c, float g[9]) {
+            __syncthreads();
+            const int n = s_n;
+            // entries tid, tid + NT, ... are read back by this thread only
+#pragma unroll 1
+            for (int e = tid; e < n; e += NT) {
                 int ci, cj, i, j;
-                cell_ij(c, ci, cj, i, j);
-                pull_pops<S, float>(A, I, make_cell(I, i, j), g);
-            };
-            int c = tid;
-            float dx = 0.f, dy = 0.f, phb = 0.f, g[9];
-            seek(c, dx, dy, phb);
-            if (c < ncell) load(c, g);
-            while (c < ncell) {
-                int cn = c + blockDim.x;
-                float dxn = 0.f, dyn = 0.f, phn = 0.f, gn[9];
-                seek(cn, dxn, dyn, phn);
-                if (cn < ncell) load(cn, gn);
-                const float rho = 1.0f + (((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8]);
-                const float jx = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
-                const float jy = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
-                float fx = I.f_gx, fy = I.f_gy;
-                for (int q = 0; q < nn; ++q) {
-                    float ddx = dx + s_ox[q];
-                    ddx = (ddx > hnx) ? ddx - fnx : ((ddx < -hnx) ? ddx + fnx : ddx);
-                    float ddy = dy + s_oy[q];
-                    if (I.periodic_y) ddy = (ddy > hny) ? ddy - fny : ((ddy < -hny) ? ddy + fny : ddy);
-                    const float ph = phi_f32(ddx, ddy, I.f_a, I.f_inv_xi, I.f_rcut2);
-                    fx += ph * s_gxf[q];
-                    fy += ph * s_gyf[q];
-                }
-                const float irho = 1.0f / rho;
-                if ((c / NT) % kL) {
-                    axf1 += phb * ((jx + 0.5f * fx) * irho);
-                    ayf1 += phb * ((jy + 0.5f * fy) * irho);
+                cell_rc(bx, inv_w, list[e].o, ci, cj);
+                cell_of(I, bx, ci, cj, i, j);
+                R fx, fy;
+                if constexpr (kF64) {
+                    fx = I.gx, fy = I.gy;
+                    if (kept) {
+#pragma unroll 4
+                        for (int q = 0; q < nn; ++q) {
+                            const int at = box_place(I, s_nbox[q], i, j);
+                            const double ph = at >= 0 ? __ldcg(pold.phi + s_noff[q] + at) : 0.0;
+                            fx += ph * s_nbr[q].gx;
+                            fy += ph * s_nbr[q].gy;
+                        }
+                    } else {
+#pragma unroll 1
+                        for (int q = 0; q < nn; ++q) {
+                            const double ph = phi_f64(I, i + 0.5, j + 0.5, s_nbr[q].x, s_nbr[q].y);
+                            fx += ph * s_nbr[q].gx;
+                            fy += ph * s_nbr[q].gy;
+                        }
+                    }
                 } else {
-                    axf0 += phb * ((jx + 0.5f * fx) * irho);
-                    ayf0 += phb * ((jy + 0.5f * fy) * irho);
+                    const float own = list[e].phi;
+                    const float hnx = 0.5f * (float)I.nx, fnx = (float)I.nx;
+                    const float hny = 0.5f * (float)I.ny, fny = (float)I.ny;
+                    const float dx = bx.rel[0] + (float)ci, dy = bx.rel[1] + (float)cj;
+                    fx = I.f_gx, fy = I.f_gy;
+#pragma unroll 2
+                    for (int q = 0; q < nn; ++q) {
+                        const Neighbour<R> nbr = s_nbr[q];
+                        float ddx = dx + nbr.x;
+                        ddx = (ddx > hnx) ? ddx - fnx : ((ddx < -hnx) ? ddx + fnx : ddx);
+                        float ddy = dy + nbr.y;
+                        if (I.periodic_y) ddy = (ddy > hny) ? ddy - fny : ((ddy < -hny) ? ddy + fny : ddy);
+                        const float ph = q == self ? own : phi_f32(ddx, ddy, I.f_a, I.f_inv_xi, I.f_rcut2);
+                        fx += ph * nbr.gx;
+                        fy += ph * nbr.gy;
+                    }
                 }
-                c = cn;
-                dx = dxn;
-                dy = dyn;
-                phb = phn;
-                if (cn < ncell) {
+                list[e].fx = fx;
+                list[e].fy = fy;
+                list[e].o = j * kRowStride + col_off(I, i);
+                const int edge = (i == 0 ? kEdgeL : 0) | (i == I.nx - 1 ? kEdgeR : 0) | (j == 0 ? kEdgeB : 0) |
+                                 (j == I.ny - 1 ? kEdgeT : 0);
+                if constexpr (kF64) list[e].edge = edge;
+                else s_edge[e] = (unsigned char)edge;
+            }
+            return n;
+        };
+        const int ncell = bx.n[0] * bx.n[1], share = (ncell + parts - 1) / parts;
+        const int c_lo = min(part * share, ncell), c_hi = min(c_lo + share, ncell);
+        if (tid == NT - 1) s_unit *= pow2(-(F::kTop - kVelBits - bit_length(ncell)));
+        int n = make_list(c_lo, min(c_lo + kCap, c_hi));
+        // wait for the preceding sweep (the populations read below), then let
+        // the next sweep launch at once: its tiles that no bead marked start
+        // while the rest of this phase runs
+        if (!wait_first) {
+            pdl_wait();
+            pdl_trigger();
+        }
+#pragma unroll 1
+        for (int bound = kVelBits;;) {
+            const int s = F::kTop - bound - bit_length(ncell);
+            T ax = 0, ay = 0;
+            unsigned mx = 0u;
+#pragma unroll 1
+            for (int c0 = c_lo;;) {
+#pragma unroll 1
+                for (int e = tid; e < n; e += NT) {
+                    const SupportCell<R> sc = list[e];
+                    int edge;
+                    if constexpr (kF64) edge = sc.edge;
+                    else edge = s_edge[e];
+                    R g[9];
+                    pull_support<S, R>(A, I, sc.o, edge, g);
+                    R ux, uy;
+                    if constexpr (kF64) {
+                        double dr = 0.0;
 #pragma unroll
-                    for (int k = 0; k < 9; ++k) g[k] = gn[k];
+                        for (int k = 0; k < 9; ++k) dr += g[k];
+                        const double rho = 1.0 + dr;
+                        const double jx = g[1] - g[3] + g[5] - g[6] - g[7] + g[8];
+                        const double jy = g[2] - g[4] + g[5] + g[6] - g[7] - g[8];
+                        ux = (jx + 0.5 * sc.fx) / rho;
+                        uy = (jy + 0.5 * sc.fy) / rho;
+                    } else {
+                        const float rho =
+                            1.0f + (((g[0] + g[1]) + (g[2] + g[3])) + ((g[4] + g[5]) + (g[6] + g[7])) + g[8]);
+                        const float jx = (g[1] - g[3]) + (g[5] - g[6]) + (g[8] - g[7]);
+                        const float jy = (g[2] - g[4]) + (g[5] + g[6]) - (g[7] + g[8]);
+                        const float irho = __frcp_rn(rho);
+                        ux = (jx + 0.5f * sc.fx) * irho;
+                        uy = (jy + 0.5f * sc.fy) * irho;
+                    }
+                    const R tx = sc.phi * ux, ty = sc.phi * uy;
+                    ax += F::term(tx, s);
+                    ay += F::term(ty, s);
+                    mx = max(mx, max(F::mag(tx), F::mag(ty)));
                 }
+                c0 += kCap;
+                if (c0 >= c_hi) break;
+                __syncthreads();  // the list is no longer read
+                n = make_list(c0, min(c0 + kCap, c_hi));
             }
-        }
-        double ax = 0.0, ay = 0.0;
-        if constexpr (kF64) lanes_sum2_to0<NT>(ax0, ay0, ax1, ay1, ax, ay, sh);
-        else lanes_sum2f_to0<NT>(axf0, ayf0, axf1, ayf1, ax, ay, sh);
-        if (tid == 0) {
-            const double inv_S = s_invS;
-            const double Vx = ax * inv_S, Vy = ay * inv_S;
-            const double Rnx = Rx + Vx, Rny = Ry + Vy;
-            tnew.Rx[b] = Rnx;
-            tnew.Ry[b] = Rny;
-            tnew.Vx[b] = Vx;
-            tnew.Vy[b] = Vy;
-            const Box nb_ = support_box(I, Rnx, Rny);
-            s_R[0] = Rnx;
-            s_R[1] = Rny;
-            s_box = nb_;
-            s_rel[0] = (float)(nb_.iu + 0.5 - Rnx);
-            s_rel[1] = (float)(nb_.ju + 0.5 - Rny);
-        }
-    } else if (tid == 0) {
-        const double Rx = tnew.Rx[b], Ry = tnew.Ry[b];
-        const Box bx = support_box(I, Rx, Ry);
-        s_R[0] = Rx;
-        s_R[1] = Ry;
-        s_box = bx;
-        s_rel[0] = (float)(bx.iu + 0.5 - Rx);
-        s_rel[1] = (float)(bx.ju + 0.5 - Ry);
-    }
-    __syncthreads();
-
-    // mark bead b in the mask of every lattice tile its support box, widened
-    // by one cell, reaches (one atomicOr per tile row and tile column the box
-    // starts in); the widening covers the bead's move in the next step, so
-    // the next sweep may update unmarked tiles before its bead phase ends
-    {
-        const Box bx = widen_box(I, s_box);
-        const int lb = b - I.bead_off;
-        const unsigned bit = 1u << (lb & 31);
-        if (!I.periodic_y) {
-            const int tr0 = bx.j0 / kTileY;
-            const int nrows = bx.h > 0 ? (bx.j0 + bx.h - 1) / kTileY - tr0 + 1 : 0;
-            for (int t = tid; t < nrows * bx.w; t += blockDim.x) {
-                const int r = tr0 + t / bx.w, ci = t - (t / bx.w) * bx.w;
-                int col = bx.i0 + ci;
-                col = (col >= I.nx) ? col - I.nx : col;
-                if (ci != 0 && (col % kTileX) != 0) continue;
-                const int tile = I.tile_base + r * I.ntx + col / kTileX;
-                atomicOr(mask_write + tile * I.mask_words + (lb >> 5), bit);
+            total<R, NT, 2>(ax, ay, mx, s_sum, uses);
+            if (w == 0) {
+                const int need = F::need(mx);
+                const bool redo = need > bound && F::finite(mx);
+                if (!redo) {
+                    // lane 0: x, the others: y
+                    const double t = (double)(lane == 0 ? ax : ay);
+                    const double unit = s_unit * pow2(bound - kVelBits);
+                    const double v = F::finite(mx) ? t * unit : __longlong_as_double(0x7ff8000000000000ll);
+                    const double r = (lane == 0 ? Rx : Ry) + v;
+                    const float h = (float)r, l = (float)(r - (double)h);
+                    const double rx = __shfl_sync(0xffffffffu, r, 0), ry = __shfl_sync(0xffffffffu, r, 1);
+                    const bool far = far_off(__shfl_sync(0xffffffffu, h, 0), __shfl_sync(0xffffffffu, h, 1));
+                    if (lane < 2) {
+                        support_axis(I, lane, h, l, far, rx, ry, s_sup.lo[lane], s_sup.n[lane], s_sup.rel[lane]);
+                        s_R[lane] = r;
+                    }
+                    // fast-bead guard (below): this bead's bits, |v| >=
+                    // kFastBead or not finite by the high word
+                    const unsigned hv = (unsigned)__double2hiint(v) & 0x7fffffffu;
+                    const bool fast = hv >= (unsigned)__double2hiint(kFastBead);
+                    any_close |= __any_sync(0xffffffffu, fast);
+                    if (part == 0 && lane < 2) {
+                        (lane ? tnew.Ry : tnew.Rx)[b] = r;
+                        (lane ? tnew.Vy : tnew.Vx)[b] = v;
+                        if (status && fast)
+                            atomicOr(status + ii, kFlagFastBead | (hv >= 0x7ff00000u ? kFlagNonFinite : 0u));
+                    }
+                }
+                if (lane == 0) s_redo = redo ? need : 0;
             }
-        } else {
-            // rows wrap: visit each cell of the box that starts a tile row or
-            // column inside the box
-            for (int t = tid; t < bx.h * bx.w; t += blockDim.x) {
-                const int cj = t / bx.w, ci = t - cj * bx.w;
-                int row = bx.j0 + cj;
-                row = (row >= I.ny) ? row - I.ny : row;
-                int col = bx.i0 + ci;
-                col = (col >= I.nx) ? col - I.nx : col;
-                if ((cj != 0 && (row % kTileY) != 0) || (ci != 0 && (col % kTileX) != 0)) continue;
-                const int tile = I.tile_base + (row / kTileY) * I.ntx + col / kTileX;
-                atomicOr(mask_write + tile * I.mask_words + (lb >> 5), bit);
-            }
+            __syncthreads();
+            if (s_redo == 0) break;
+            // a term of magnitude 2^kVelBits or more (a diverging run): once
+            // more with room for it
+            bound = s_redo;
+            n = make_list(c_lo, min(c_lo + kCap, c_hi));
         }
+    } else {
+        pdl_wait();
+        pdl_trigger();
+        __syncthreads();  // the record is in place
+        any_close = 1;
+        if (tid < 2) {
+            const double rx = tnew.Rx[b], ry = tnew.Ry[b], r = tid ? ry : rx;
+            const float h = (float)r;
+            support_axis(I, tid, h, (float)(r - (double)h), far_off((float)rx, (float)ry), rx, ry, s_sup.lo[tid],
+                         s_sup.n[tid], s_sup.rel[tid]);
+            s_R[tid] = r;
+        }
+        __syncthreads();
     }
 
     // S_b = sum_x phi_b at the new position
-    {
-        const double Rx = s_R[0], Ry = s_R[1];
-        const Box bx = s_box;
-        const float rel0x = s_rel[0], rel0y = s_rel[1];
-        double acc0 = 0.0, acc1 = 0.0, acc = 0.0, dummy = 0.0;
-        float part0 = 0.0f, part1 = 0.0f;
-        for (int c = tid; c < bx.w * bx.h; c += blockDim.x) {
-            const int cj = c / bx.w, ci = c - cj * bx.w;
-            const bool hi = (c / NT) % kL != 0;  // the thread's second lane
-            if constexpr (kF64) {
-                int i = bx.i0 + ci;
-                i = (i >= I.nx) ? i - I.nx : i;
-                int j = bx.j0 + cj;
-                j = (j >= I.ny) ? j - I.ny : j;
-                const double ph = phi_f64(I, i + 0.5, j + 0.5, Rx, Ry);
-                if (hi) acc1 += ph;
-                else acc0 += ph;
-            } else {
-                // each lane sums at most a few terms in FP32 before the
-                // FP64-level reduction
-                const float ph = phi_f32(rel0x + (float)ci, rel0y + (float)cj, I.f_a, I.f_inv_xi, I.f_rcut2);
-                if (hi) part1 += ph;
-                else part0 += ph;
-            }
+    T acc = 0, none = 0;
+    unsigned mx = 0u;
+    const Support bx = s_sup;
+    const float inv_w = inv_width(bx);
+    const int ncell = bx.n[0] * bx.n[1], share = (ncell + parts - 1) / parts;
+    const int c_lo = min(part * share, ncell), c_hi = min(c_lo + share, ncell);
+    const int s_shift = F::kTop - 1 - bit_length(ncell);  // phi < 2
+#pragma unroll 1
+    for (int c = c_lo + tid; c < c_hi; c += NT) {
+        R ph;
+        int ci, cj;
+        cell_rc(bx, inv_w, c, ci, cj);
+        if constexpr (kF64) {
+            int i, j;
+            cell_of(I, bx, ci, cj, i, j);
+            ph = phi_f64(I, i + 0.5, j + 0.5, s_R[0], s_R[1]);
+        } else {
+            ph = phi_f32(bx.rel[0] + (float)ci, bx.rel[1] + (float)cj, I.f_a, I.f_inv_xi, I.f_rcut2);
         }
-        if constexpr (kF64) lanes_sum2_to0<NT>(acc0, 0.0, acc1, 0.0, acc, dummy, sh);
-        else lanes_sum2f_to0<NT>(part0, 0.0f, part1, 0.0f, acc, dummy, sh);
-        if (tid == 0) tnew.S[b] = acc;
+        acc += F::term(ph, s_shift);
+        if constexpr (kF64) {
+            // kept for the sweep and the next bead phase; a box has at most phi_cap cells
+            if (c < I.phi_cap) pnew.phi[I.phi_off + (b - first) * I.phi_cap + c] = ph;
+        }
     }
+    if constexpr (kF64) {
+        if (I.phi_cap && part == 0 && tid == 0) pnew.box[b] = make_int4(bx.lo[0], bx.lo[1], bx.n[0], bx.n[1]);
+    }
+    total<R, NT, 1>(acc, none, mx, s_sum, uses);
+    if (part != 0) return;
 
-    // the last CTA of this instance computes the forces of all its beads
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-        const unsigned prev = atomicAdd(&counters[ii], 1u);
-        s_last = (prev == (unsigned)(I.nb - 1));
+    // The last CTA of this instance computes the forces of all its beads:
+    // warp 0 hands in the bead (R, V and S) while the others mark tiles.  An
+    // arrival counts 1, and 2^16 if the excluded volume may act on the bead.
+    if (w == 0) {
+        if (lane == 0) tnew.S[b] = (double)acc * pow2(-s_shift);
+        __syncwarp();  // lane 1's R and V before lane 0's release
+        if (lane == 0) s_seen = arrive_acq_rel(&counters[ii], any_close ? 0x10001u : 1u) | (any_close ? 0x10000u : 0u);
+    } else {
+        // FP32 overlay table: x (and y when periodic) wrapped into the
+        // lattice, split into hi + lo
+        if (w == 1 && lane < 2) {
+            double v = s_R[lane];
+            if (lane == 0 || I.periodic_y) {
+                const int L = lane ? I.ny : I.nx;
+                v -= (double)floorf((float)v * (lane ? I.f_inv_ny : I.f_inv_nx)) * (double)L;
+                v = (v < 0.0) ? v + L : ((v >= L) ? v - L : v);
+            }
+            const float hi = (float)v;
+            (lane ? tnew.yh : tnew.xh)[b] = hi;
+            (lane ? tnew.yl : tnew.xl)[b] = (float)(v - (double)hi);
+        }
+        // mark bead b in the mask of every lattice tile its support box, widened
+        // by one cell, reaches: one atomicOr per tile row and tile column the
+        // box starts in; the widening covers the bead's move in the next step, so
+        // the next sweep may update unmarked tiles before its bead phase ends
+        const Support wb = widen(I, bx);
+        const float inv_wb = inv_width(wb);
+        const int lb = b - first;
+        const unsigned bit = 1u << (lb & 31);
+#pragma unroll 1
+        for (int t = tid - 32; t < wb.n[0] * wb.n[1]; t += NT - 32) {
+            int ci, cj, col, row;
+            cell_rc(wb, inv_wb, t, ci, cj);
+            cell_of(I, wb, ci, cj, col, row);
+            if ((cj != 0 && (row % kTileY) != 0) || (ci != 0 && (col % kTileX) != 0)) continue;
+            const int tile = I.tile_base + (row / kTileY) * I.ntx + col / kTileX;
+            atomicOr(mask_write + tile * I.mask_words + (lb >> 5), bit);
+        }
     }
     __syncthreads();
-    if (s_last) {
-    __threadfence();
+    const unsigned seen = s_seen;  // arrivals before this one, and this one's flag
+    if ((seen & 0xffffu) != (unsigned)(nb - 1)) return;
+    const bool crowd = I.k_ev != 0.0 && (seen >> 16) != 0u;
+    ForceShared<R> &fs = *reinterpret_cast<ForceShared<R> *>(s_buf);
     // this phase's export number (the previous phase wrote the counter)
     const unsigned long long ex_k = ex.ring ? *(volatile unsigned long long *)ex.count : 0ull;
-    // the instance's status bits as earlier phases left them
-    if (tid == 0) s_stold = (status && advance) ? __ldcg(status + ii) : 0u;
-    // stage the instance's new positions and support sums (written by every
-    // CTA; the L2-coherent loads see them), then every segment once.  The
-    // fast-bead guard below tests this phase's velocities: they are loaded in
-    // the same round of loads, so that the guard adds no memory round trip
-    // to the phase's last CTA
-    const bool guard = status && advance;
-    bool fast = false, bad = false;
-    for (int q = tid; q < I.nb; q += blockDim.x) {
-        s_rx[q] = __ldcg(tnew.Rx + I.bead_off + q);
-        s_ry[q] = __ldcg(tnew.Ry + I.bead_off + q);
-        s_gx[q] = __ldcg(tnew.S + I.bead_off + q);
-        if (guard) {
-            const double vx = __ldcg(tnew.Vx + I.bead_off + q), vy = __ldcg(tnew.Vy + I.bead_off + q);
-            fast |= !(fabs(vx) < kFastBead && fabs(vy) < kFastBead);
-            bad |= !(isfinite(vx) && isfinite(vy));
-        }
+    // the instance's status bits, this phase's among them
+    const unsigned st_now = (status && advance) ? __ldcg(status + ii) : 0u;
+    // The instance's new positions and support sums (written by every CTA;
+    // the L2-coherent loads see them), then every segment, then every bead;
+    // a thread works on one axis (ax) of item q: FP64 instructions cost a
+    // warp 64 cycles each whatever its lanes do, so x and y share them
+    const int items = 2 * nb, N = I.n_beads;
+    const float inv_n = 1.0f / (float)N;
+    for (int k = tid; k < items; k += NT) {
+        fs.r[k] = __ldcg(((k & 1) ? tnew.Ry : tnew.Rx) + first + (k >> 1));
+        if (!(k & 1)) fs.S[k >> 1] = __ldcg(tnew.S + first + (k >> 1));
     }
     __syncthreads();
     // fast-bead guard: the early update of unmarked tiles assumes a bead
-    // moves less than a cell per step.  When one of this phase's velocities
-    // reaches kFastBead per component (or is not finite), flag the instance;
-    // while the flag is set, mark every tile of the instance (bead 0's bit)
-    // in this phase's masks, so that the next sweeps wait on all of them
-    if (guard) {
-        const int any_fast = __syncthreads_or(fast);
-        const int any_bad = __syncthreads_or(bad);
-        if (any_fast && tid == 0) atomicOr(status + ii, kFlagFastBead | (any_bad ? kFlagNonFinite : 0u));
-        if (any_fast || (s_stold & kFlagFastBead))
-            for (int t = tid; t < I.ntx * I.nty; t += blockDim.x)
-                atomicOr(mask_write + (I.tile_base + t) * I.mask_words, 1u);
-    }
-    for (int q = tid; q < I.nb; q += blockDim.x) {
-        s_xf[q] = (float)(s_rx[q] - s_rx[0]);
-        s_yf[q] = (float)(s_ry[q] - s_ry[0]);
-    }
-    for (int q = tid; q < I.nb; q += blockDim.x) {
-        if ((q + 1) % I.n_beads != 0) {
-            const double dx = s_rx[q + 1] - s_rx[q], dy = s_ry[q + 1] - s_ry[q];
-            if constexpr (kF64) {
-                const double L = sqrt(dx * dx + dy * dy);
-                const double iL = 1.0 / L;
-                s_tx[q] = dx * iL;
-                s_ty[q] = dy * iL;
-                s_ln[q] = L;
-            } else {
-                const double d2 = dx * dx + dy * dy;
-                const float L = sqrtf((float)d2);
-                s_ox[q] = (float)dx / L;                                // tangent x
-                s_oy[q] = (float)dy / L;                                // tangent y
-                s_gxf[q] = L;                                           // length
-                s_gyf[q] = (float)(d2 - I.l0 * I.l0) / (L + I.f_l0);  // L - l0
+    // moves less than a cell per step.  When a velocity has reached kFastBead
+    // per component (or is not finite) the instance is flagged; while the
+    // flag is set, mark every tile of the instance (bead 0's bit) in this
+    // phase's masks, so that the next sweeps wait on all of them
+    if (st_now & kFlagFastBead)
+        for (int t = tid; t < I.ntx * I.nty; t += NT) atomicOr(mask_write + (I.tile_base + t) * I.mask_words, 1u);
+    // place of bead q < 256 within its fiber
+    auto in_fiber = [&](int q) { return q - N * (int)(((float)q + 0.5f) * inv_n); };
+    // Segment q (bead q to q + 1 of the fiber): length, tangent, stretch
+    for (int k0 = 0; k0 < items; k0 += NT) {
+        const int k = k0 + tid, q = k >> 1;
+        const bool seg = k < items && in_fiber(q) < N - 1;
+        const double d = seg ? fs.r[k + 2] - fs.r[k] : 1.0;
+        const double d2 = d * d, s = d2 + __shfl_xor_sync(0xffffffffu, d2, 1);
+        R L, t, str;
+        if constexpr (kF64) {
+            L = sqrt(s);
+            t = d * (1.0 / L);
+            str = L - I.l0;
+        } else {
+            // positions stay FP64; the stretch L - l0 = (|d|^2 - l0^2) /
+            // (L + l0) is formed from the FP64 |d|^2 so that the small strain
+            // of a stiff spring does not cancel away in FP32
+            L = sqrtf((float)s);
+            t = (float)d / L;
+            str = (float)(s - I.l0 * I.l0) / (L + I.f_l0);
+        }
+        if (seg) {
+            fs.t[k] = t;
+            if (!(k & 1)) {
+                fs.len[q] = L;
+                fs.str[q] = str;
             }
         }
     }
+    if (crowd) {
+        for (int q = tid; q < nb; q += NT) {
+            fs.xf[q] = (float)(fs.r[2 * q] - fs.r[0]);
+            fs.yf[q] = (float)(fs.r[2 * q + 1] - fs.r[1]);
+        }
+        __syncthreads();
+        screen_close<NW>(I, fs.xf, fs.yf, fs.cand);
+    }
     __syncthreads();
-    for (int q = tid; q < I.nb; q += blockDim.x) {
-        double Fx, Fy, Gx, Gy;
-        if constexpr (kF64) {
-            bead_force(I, s_rx, s_ry, s_xf, s_yf, s_tx, s_ty, s_ln, q, Fx, Fy);
-            const double inv_S = 1.0 / s_gx[q];
-            Gx = Fx * inv_S;
-            Gy = Fy * inv_S;
-        } else {
-            float fx, fy;
-            bead_force_f32(I, s_rx, s_ry, s_xf, s_yf, s_ox, s_oy, s_gxf, s_gyf, q, fx, fy);
-            const float inv_S = 1.0f / (float)s_gx[q];
-            Fx = fx;
-            Fy = fy;
-            Gx = fx * inv_S;
-            Gy = fy * inv_S;
+    // What segment q pulls bead q with (and bead q + 1 the other way): Eq. 11's
+    // spring, and Eq. 12's bending, k_b (t_{q+1} + t_{q-1}).(I - t_q t_q) / L
+    // with the tangents of missing segments zero
+    for (int k0 = 0; k0 < items; k0 += NT) {
+        const int k = k0 + tid, q = k >> 1, i0 = in_fiber(q);
+        const bool seg = k < items && i0 < N - 1;
+        R v = (R)0, t = (R)0;
+        if (seg) {
+            t = fs.t[k];
+            if (i0 < N - 2) v = fs.t[k + 2];
+            if (i0 > 0) v += fs.t[k - 2];
         }
-        const int gq = I.bead_off + q;
-        tnew.Fx[gq] = Fx;
-        tnew.Fy[gq] = Fy;
-        tnew.Gx[gq] = Gx;
-        tnew.Gy[gq] = Gy;
-        // FP32 overlay table: x (and y when periodic) wrapped into the
-        // lattice, split into hi + lo
-        const double rx = s_rx[q];
-        double xw = rx - (double)floorf((float)rx * I.f_inv_nx) * (double)I.nx;
-        xw = (xw < 0.0) ? xw + I.nx : ((xw >= I.nx) ? xw - I.nx : xw);
-        double yw = s_ry[q];
-        if (I.periodic_y) {
-            yw -= (double)floorf((float)yw * I.f_inv_ny) * (double)I.ny;
-            yw = (yw < 0.0) ? yw + I.ny : ((yw >= I.ny) ? yw - I.ny : yw);
+        const R vt1 = v * t, vt = vt1 + __shfl_xor_sync(0xffffffffu, vt1, 1);
+        if (seg) {
+            const R ks = kF64 ? (R)I.ks_l02 : (R)I.f_ks_l02, kb = kF64 ? (R)I.k_b : (R)I.f_kb;
+            fs.pull[k] = ks * fs.str[q] * t - kb * (v - vt * t) / fs.len[q];
         }
-        const float xh = (float)xw, yh = (float)yw;
-        tnew.xh[gq] = xh;
-        tnew.xl[gq] = (float)(xw - (double)xh);
-        tnew.yh[gq] = yh;
-        tnew.yl[gq] = (float)(yw - (double)yh);
-        tnew.gxf[gq] = (float)Gx;
-        tnew.gyf[gq] = (float)Gy;
+    }
+    __syncthreads();
+    for (int k = tid; k < items; k += NT) {
+        const int q = k >> 1, ax = k & 1, gq = first + q, i0 = in_fiber(q);
+        R f = (R)0;
+        if (i0 > 0) f -= fs.pull[k - 2];
+        if (i0 < N - 1) f += fs.pull[k];
+        if (crowd) f += close_force<R>(I, fs.r, fs.cand, q, ax);
+        // constant external force F_0 (driven particle, Sec. 3.2)
+        if constexpr (kF64) f += ax ? I.ext_fy : I.ext_fx;
+        else f += ax ? I.f_ext_fy : I.f_ext_fx;
+        R g;
+        if constexpr (kF64) g = f * (1.0 / fs.S[q]);
+        else g = f * (1.0f / (float)fs.S[q]);
+        (ax ? tnew.gyf : tnew.gxf)[gq] = (float)g;
+        (ax ? tnew.Gy : tnew.Gx)[gq] = g;
+        (ax ? tnew.Fy : tnew.Fx)[gq] = f;
         if (ex.ring) {
             // export: R, V, F, S of bead q into the ring slot of this phase
             double *d = ex.ring + (size_t)(ex_k % (unsigned long long)ex.slots) * ex.stride + kExportHeader;
-            const int nbq = I.nb;
-            d[q] = s_rx[q];
-            d[nbq + q] = s_ry[q];
-            d[2 * nbq + q] = __ldcg(tnew.Vx + gq);
-            d[3 * nbq + q] = __ldcg(tnew.Vy + gq);
-            d[4 * nbq + q] = Fx;
-            d[5 * nbq + q] = Fy;
-            d[6 * nbq + q] = s_gx[q];
+            d[ax * nb + q] = fs.r[k];
+            d[(2 + ax) * nb + q] = __ldcg((ax ? tnew.Vy : tnew.Vx) + gq);
+            d[(4 + ax) * nb + q] = f;
+            if (!ax) d[6 * nb + q] = fs.S[q];
         }
     }
     if (ex.ring) {
@@ -786,8 +936,33 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         }
     }
     if (tid == 0) counters[ii] = 0u;
-    }  // last bead of the instance
-    }  // beads of this CTA
+}
+
+// The profiles a bead phase keeps (PhiTab), from a table's positions.
+__global__ void k_phi(const Inst *__restrict__ insts, const int4 *__restrict__ blist, const BeadTab tab0,
+                      const BeadTab tab1, const PhiTab phi0, const PhiTab phi1, int gparity) {
+    const int4 br = blist ? blist[blockIdx.x] : make_int4(0, blockIdx.x, 0, gridDim.x);
+    const Inst &I = insts[br.x >> 1];
+    const bool one = gparity ^ (br.x & 1);
+    const BeadTab &tab = one ? tab0 : tab1;
+    const PhiTab &pt = one ? phi0 : phi1;
+    if (I.phi_cap == 0) return;
+    const int b = br.y;
+    const double rx = tab.Rx[b], ry = tab.Ry[b];
+    const float xh = (float)rx, yh = (float)ry;
+    const bool far = far_off(xh, yh);
+    Support bx;
+    support_axis(I, 0, xh, (float)(rx - (double)xh), far, rx, ry, bx.lo[0], bx.n[0], bx.rel[0]);
+    support_axis(I, 1, yh, (float)(ry - (double)yh), far, rx, ry, bx.lo[1], bx.n[1], bx.rel[1]);
+    const int ncell = bx.n[0] * bx.n[1];
+    if (threadIdx.x == 0) pt.box[b] = make_int4(bx.lo[0], bx.lo[1], bx.n[0], bx.n[1]);
+    double *phi = pt.phi + I.phi_off + (b - br.z) * I.phi_cap;
+    for (int c = threadIdx.x; c < ncell && c < I.phi_cap; c += blockDim.x) {
+        int i = bx.lo[0] + c % bx.n[0], j = bx.lo[1] + c / bx.n[0];
+        i = (i >= I.nx) ? i - I.nx : i;
+        j = (j >= I.ny) ? j - I.ny : j;
+        phi[c] = phi_f64(I, i + 0.5, j + 0.5, rx, ry);
+    }
 }
 
 }  // namespace
@@ -806,21 +981,24 @@ int sm_count() {
 }
 
 template <class S>
-cudaError_t launch_beads_t(cudaLaunchConfig_t &cfg, bool few, const Inst *inst_d, const int2 *blist, int nb_total,
-                           const void *pool, BeadTab tab0, BeadTab tab1, unsigned *mask_write, int gparity,
-                           int advance, unsigned *counters, BeadExport ex, unsigned *status) {
-    cfg.blockDim = dim3(few ? kBeadThreadsFew : kBeadThreads);
+cudaError_t launch_beads_t(cudaLaunchConfig_t &cfg, bool few, const Inst *inst_d, const int4 *blist, const void *pool,
+                           const BeadTab tab[2], const PhiTab phi[2], unsigned *mask_write, int gparity, int advance, int wait_first,
+                           unsigned *counters, BeadExport ex, unsigned *status) {
+    constexpr int kFew = std::is_same<S, double>::value ? kBeadThreadsFew64 : kBeadThreadsFew;
+    cfg.blockDim = dim3(few ? kFew : kBeadThreads);
+    typename PhiArg<S>::type p0, p1;
+    if constexpr (std::is_same<S, double>::value) p0 = phi[0], p1 = phi[1];
     if (few)
-        return cudaLaunchKernelEx(&cfg, k_beads<S, kBeadThreadsFew>, inst_d, blist, nb_total, (const S *)pool, tab0,
-                                  tab1, mask_write, gparity, advance, counters, ex, status);
-    return cudaLaunchKernelEx(&cfg, k_beads<S, kBeadThreads>, inst_d, blist, nb_total, (const S *)pool, tab0, tab1,
-                              mask_write, gparity, advance, counters, ex, status);
+        return cudaLaunchKernelEx(&cfg, k_beads<S, kFew>, inst_d, blist, (const S *)pool, tab[0], tab[1], p0, p1, mask_write,
+                                  gparity, advance, wait_first, counters, ex, status);
+    return cudaLaunchKernelEx(&cfg, k_beads<S, kBeadThreads>, inst_d, blist, (const S *)pool, tab[0], tab[1], p0, p1, mask_write,
+                              gparity, advance, wait_first, counters, ex, status);
 }
 
 }  // namespace
 
-cudaError_t launch_beads(int precision, const Inst *inst_d, const int2 *blist, int nb_total, const void *pool,
-                         BeadTab tab0, BeadTab tab1, unsigned *mask_write, int gparity, int advance,
+cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, int nb_total, int ntiles,
+                         const void *pool, const BeadTab tab[2], const PhiTab phi[2], unsigned *mask_write, int gparity, int advance,
                          unsigned *counters, int pdl, cudaStream_t st, BeadExport ex, unsigned *status) {
     if (nb_total <= 0) return cudaSuccess;
     // one CTA per bead: a grid capped at the resident CTAs (persistent) keeps
@@ -828,27 +1006,61 @@ cudaError_t launch_beads(int precision, const Inst *inst_d, const int2 *blist, i
     // too few registers to start its unmarked tiles with (measured with
     // 256-thread CTAs: the batched step 8 % slower), so every bead gets its
     // own CTA; a list that fits on the SMs one bead per SM gets wider CTAs
-    const bool few = nb_total <= sm_count();
+    const int sms = sm_count();
+    const bool few = nb_total <= sms;
+    // FP64: an SM issues one FP64 warp instruction per 16 cycles, so a short
+    // list's beads are split over as many SMs as there are, up to kBeadParts
+    // CTAs a bead
+    int parts = 1;
+    if (precision == 0)
+        while (2 * parts <= kBeadParts && 2 * parts * nb_total <= 2 * sms) parts *= 2;
+    // A sweep of up to a few waves has room for the bead CTAs beside it: they
+    // list their supports while it runs.  They enter a longer sweep's SMs
+    // only as it drains; then the next sweep's release comes first
+    const int wait_first = ntiles > kEarlyListTiles ? 1 : 0;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nb_total);
+    cfg.gridDim = dim3(nb_total * parts);
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    int na = 0;
+    if (pdl) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (parts > 1) {
+        attr[na].id = cudaLaunchAttributeClusterDimension;
+        attr[na].val.clusterDim.x = parts;
+        attr[na].val.clusterDim.y = 1;
+        attr[na++].val.clusterDim.z = 1;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = na;
     switch (precision) {
         case 0:
-            return launch_beads_t<double>(cfg, few, inst_d, blist, nb_total, pool, tab0, tab1, mask_write, gparity,
-                                          advance, counters, ex, status);
+            return launch_beads_t<double>(cfg, few, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
+                                          wait_first, counters, ex, status);
         case 1:
-            return launch_beads_t<float>(cfg, few, inst_d, blist, nb_total, pool, tab0, tab1, mask_write, gparity,
-                                         advance, counters, ex, status);
+            return launch_beads_t<float>(cfg, few, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
+                                         wait_first, counters, ex, status);
         case 2:
-            return launch_beads_t<__half>(cfg, few, inst_d, blist, nb_total, pool, tab0, tab1, mask_write, gparity,
-                                          advance, counters, ex, status);
+            return launch_beads_t<__half>(cfg, few, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
+                                          wait_first, counters, ex, status);
     }
     return cudaErrorInvalidValue;
+}
+
+int phi_cells(const Inst &I) {
+    // support_axis: at most 2 rcut + 5 cells an axis, and two for its FP32 rounding
+    const double n = 2.0 * I.rcut + 8.0;
+    const int64_t w = n < I.nx ? (int64_t)n : I.nx, h = n < I.ny ? (int64_t)n : I.ny;
+    return (int)(w * h);
+}
+
+cudaError_t launch_phi(const Inst *insts, const int4 *blist, int nb_total, const BeadTab tab[2], const PhiTab phi[2],
+                       int gparity, cudaStream_t st) {
+    if (nb_total <= 0) return cudaSuccess;
+    k_phi<<<nb_total, 256, 0, st>>>(insts, blist, tab[0], tab[1], phi[0], phi[1], gparity);
+    return cudaGetLastError();
 }
 
 }  // namespace fpd

@@ -48,7 +48,7 @@ struct Inst {
     int32_t tile_base;    // first tile of this instance in the tile-mask arrays
     int32_t mask_words;   // 32-bit words per tile mask: ceil(nb / 32), >= 1
     int32_t par_xor;      // local step parity = global step parity ^ par_xor
-    int32_t pad1_;
+    int32_t phi_cap;      // elements a bead has in PhiTab::phi (0: profiles not kept)
     double s_e, s_eps, s_q;
     float scale[9];       // FP16 storage: stored = (f_k - w_k) * scale[k]
     float inv_scale[9];
@@ -65,7 +65,8 @@ struct Inst {
     double ks_l02;
     float f_ks_l02, f_kb, f_kev, f_l0, f_inv_nx;
     // static solid layers of the sandwich Couette benchmark (Eq. 14)
-    int32_t sandwich, pad2_;
+    int32_t sandwich;
+    int32_t phi_off;      // this instance's first element in PhiTab::phi
     double sw_zl, sw_zr, half_h;
     float f_sw_zl, f_sw_zr, f_half_h;
     // periodic y without walls, and the constant external force on every
@@ -118,6 +119,21 @@ struct BeadTab {
     double *Rx, *Ry, *Vx, *Vy, *Fx, *Fy, *S, *Gx, *Gy;  // G = F / S
     float *xh, *xl, *yh, *yl, *gxf, *gyf;
 };
+// FP64 only: a bead's profile at every cell of its support box, as its bead
+// phase evaluated it for the support sum, and that box (first column and row,
+// width and height).  The next bead phase and the sweep read them instead of
+// evaluating each of the ~17 profiles a support cell meets in a step again
+// (~60 FP64 instructions each): 4096 x 1024 with 40 beads, bead phase 96 ->
+// 33 us.  Instances with Inst::phi_cap = 0 keep none.  The FP32 paths
+// evaluate: reading measured slower there (512-instance step 430 -> 518 us).
+struct PhiTab {
+    double *phi = nullptr;
+    int4 *box = nullptr;
+};
+// What a kernel of storage type S takes of it.
+struct NoPhi {};
+template <class S> struct PhiArg { using type = NoPhi; };
+template <> struct PhiArg<double> { using type = PhiTab; };
 constexpr int kTabDoubles = 9;  // per bead
 constexpr int kTabFloats = 6;
 
@@ -447,8 +463,12 @@ __device__ __forceinline__ void place_pops(S *__restrict__ A, const Inst &I, con
 // ---------------------------------------------------------------- Eq. 2
 // Minimum-image separation in x and the hard support cutoff, with every
 // rounding spelled out (no contraction), so that the cutoff decision and the
-// distance equal those of a plain IEEE evaluation.
+// distance equal those of a plain IEEE evaluation.  Clearly inside half a
+// period the rounded division gives the image 0, and d - L 0 is d itself:
+// the usual case skips the division (about 14 FP64 instructions of a
+// profile's 90).
 __device__ __forceinline__ double min_image_rn(double d, double L) {
+    if (fabs(d) < 0.49 * L) return d;
     return __dsub_rn(d, __dmul_rn(L, floor(__dadd_rn(__ddiv_rn(d, L), 0.5))));
 }
 
@@ -538,6 +558,23 @@ __device__ __forceinline__ Box support_box(const Inst &I, double Rx, double Ry) 
         b.w = (int)(xh - xl) + 1;
     }
     return b;
+}
+
+// Place of lattice cell (i, j) in a kept support box, or -1 outside it.
+__device__ __forceinline__ int box_place(const Inst &I, const int4 &bx, int i, int j) {
+    int d = i - bx.x, e = j - bx.y;
+    if (d < 0) d += I.nx;
+    if (e < 0 && I.periodic_y) e += I.ny;
+    return (d < bx.z && (unsigned)e < (unsigned)bx.w) ? e * bx.z + d : -1;
+}
+// phi_f64 of bead q (table index) at lattice cell (i, j): kept, or evaluated
+// (the same bits).
+__device__ __forceinline__ double phi_cell(const Inst &I, const BeadTab &tab, const PhiTab &pt, int q, int i, int j) {
+    if (I.phi_cap) {
+        const int at = box_place(I, pt.box[q], i, j);
+        return at >= 0 ? pt.phi[I.phi_off + (q - I.bead_off) * I.phi_cap + at] : 0.0;
+    }
+    return phi_f64(I, i + 0.5, j + 0.5, tab.Rx[q], tab.Ry[q]);
 }
 
 // FP32 variant for the reduced-precision lattice path: dx, dy relative to a

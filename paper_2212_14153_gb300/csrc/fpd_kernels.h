@@ -9,13 +9,13 @@ namespace fpd {
 
 constexpr int kTileX = 32;       // lattice tile: 32 x 8 cells, one thread each
 constexpr int kTileY = 8;
+constexpr int kSplitCtas = 304, kSplitCtas64 = 608;  // a sweep's tiles are split by rows up to this many CTAs
 constexpr int kMaxBeads = 256;   // beads per instance (shared-memory tables)
 constexpr int kBeadThreads = 128;  // per bead CTA: more beads resident at once (batched sweep +9 %)
-constexpr int kBeadThreadsFew = 256;  // per bead CTA when the beads fit on the SMs one per SM
-constexpr int kBeadLanes = 256;  // virtual lanes of the per-bead sums (any CTA size gives the same bits)
-static_assert(kBeadLanes % kBeadThreads == 0 && kBeadLanes % kBeadThreadsFew == 0 &&
-                  kBeadLanes / kBeadThreads <= 2 && kBeadLanes / kBeadThreadsFew <= 2,
-              "a bead thread holds one or two virtual lanes");
+constexpr int kBeadThreadsFew = 512;  // per bead CTA when the beads fit on the SMs one per SM
+constexpr int kBeadThreadsFew64 = 256;  // the same, FP64
+constexpr int kEarlyListTiles = 4096;  // longest sweep (tiles) whose bead phase lists its supports before waiting
+constexpr int kBeadParts = 8;    // CTAs a bead's cells are split over at most (FP64, short bead lists)
 constexpr int kGraphSteps = 32;  // time steps per captured graph chunk
 // Tile-mask buffers, used in rotation: the bead phase of step t marks buffer
 // t % kMaskBufs; the sweep of step t reads it (hot tiles) and buffer
@@ -75,12 +75,13 @@ constexpr int kLatticeVariants = 5;
 // instance creation, outside any stream capture).
 cudaError_t prepare_lattice_kernels();
 inline int lattice_vec_width(int precision) { return precision == 0 ? 2 : 4; }
-cudaError_t launch_lattice(int precision, const Inst *inst_d, const Inst &inst_h, void *pool, BeadTab tab,
+cudaError_t launch_lattice(int precision, const Inst *inst_d, const Inst &inst_h, void *pool, BeadTab tab, PhiTab phi,
                            const SweepMasks &masks, int parity, int after_beads, int variant, cudaStream_t st);
 
 // Bead phase (items (3) then (1)): one CTA per bead of any instance
-// (blist[i] = (instance slot, global bead index); NULL = instance 0, bead i;
-// every bead of an instance must be in the same launch).  With the instance's
+// (blist[i] = (2 slot + par_xor, global bead index, the instance's first bead
+// and bead count); NULL = instance 0, bead i; every bead of an instance must
+// be in the same launch).  ntiles: tiles of the sweep before it.  With the instance's
 // step parity p = gparity ^ par_xor it reads table p ^ 1 and writes table p
 // (tab0 / tab1); advance = 0 only computes S and F of table p from its own R
 // (initialisation).  Every bead ORs its bit into the mask of each lattice
@@ -105,10 +106,22 @@ struct BeadExport {
 // instance's last CTA sets kFlagFastBead (and kFlagNonFinite) when a bead
 // velocity component reaches kFastBead in magnitude (or is not finite), and
 // marks every tile of a flagged instance in mask_write; NULL: not checked.
-cudaError_t launch_beads(int precision, const Inst *inst_d, const int2 *blist, int nb_total,
-                         const void *pool, BeadTab tab0, BeadTab tab1, unsigned *mask_write, int gparity,
-                         int advance, unsigned *counters, int pdl, cudaStream_t st, BeadExport ex = BeadExport{},
+cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, int nb_total, int ntiles,
+                         const void *pool, const BeadTab tab[2], const PhiTab phi[2], unsigned *mask_write,
+                         int gparity, int advance, unsigned *counters, int pdl, cudaStream_t st, BeadExport ex = BeadExport{},
                          unsigned *status = nullptr);
+
+// An instance's profiles are kept (PhiTab) if both its tables fit in this:
+// L2-sized, and 30 times what 40 beads of a = 4 cells take.
+constexpr size_t kPhiBytes = (size_t)16 << 20;
+// Cells of the instance's largest support box (elements a bead needs in PhiTab::phi).
+int phi_cells(const Inst &inst_h);
+// FP64: fill phi and box from the positions in the table the next bead phase
+// reads (after a table was read from a checkpoint, or moved; the bead phase
+// keeps them otherwise): every bead of blist (as launch_beads) in the table
+// told of a bead phase at parity gparity.
+cudaError_t launch_phi(const Inst *insts, const int4 *blist, int nb_total, const BeadTab tab[2], const PhiTab phi[2],
+                       int gparity, cudaStream_t st);
 
 // Watchdog: sets kFlagNonFinite in status[slot] of every instance holding a
 // non-finite population at its current step.  Batch form: tiles[t] =
@@ -126,7 +139,8 @@ cudaError_t launch_watch(int precision, const Inst *insts, const Inst &inst_h, c
 // (collision 1): the sweep then runs variant 0 with both collision forms.
 // A single instance with collision 1 runs variant 0 as well.
 cudaError_t launch_lattice_batch(int precision, const Inst *insts, const int2 *tiles, int ntiles, void *pool,
-                                 BeadTab tab0, BeadTab tab1, const SweepMasks &masks, int gparity, int after_beads,
+                                 const BeadTab tab[2], const PhiTab phi[2], const SweepMasks &masks, int gparity,
+                                 int after_beads,
                                  int variant, int any_mrt, cudaStream_t st);
 
 cudaError_t launch_init(int precision, const Inst *inst_d, const Inst &inst_h, void *pool, int couette,

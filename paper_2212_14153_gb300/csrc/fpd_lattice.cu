@@ -68,8 +68,8 @@ __device__ __forceinline__ const float *stage_overlay(const Inst &I, const BeadT
 // beads marked in its tile's mask (m, W words; any = OR of the words).
 // kStaged: the FP32 overlay entries are read from sov (stage_overlay), else
 // from the table; the values and their order are the same either way.
-template <class R, bool kStaged>
-__device__ __forceinline__ void cell_overlay(const Inst &I, const BeadTab &tab, const float *__restrict__ sov,
+template <class R, bool kStaged, class P>
+__device__ __forceinline__ void cell_overlay(const Inst &I, const BeadTab &tab, const P &pt, const float *__restrict__ sov,
                                              const unsigned *__restrict__ m,
                                              const int W, const unsigned any, const int x, const int y, R &Fx,
                                              R &Fy, R &s_nu, R &s_e, R &s_eps, R &s_q) {
@@ -83,14 +83,13 @@ __device__ __forceinline__ void cell_overlay(const Inst &I, const BeadTab &tab, 
             s_q = I.fluid_rates_d[3];
             return;
         }
-        const double xc = x + 0.5, yc = y + 0.5;
-        double Phi = I.sandwich ? sandwich_phi_f64(I, yc) : 0.0;
+        double Phi = I.sandwich ? sandwich_phi_f64(I, y + 0.5) : 0.0;
         for (int w = 0; w < W && any; ++w) {
             unsigned bits = m[w];
             while (bits) {
                 const int q = I.bead_off + 32 * w + __ffs(bits) - 1;
                 bits &= bits - 1u;
-                const double ph = phi_f64(I, xc, yc, tab.Rx[q], tab.Ry[q]);
+                const double ph = phi_cell(I, tab, pt, q, x, y);
                 if (ph != 0.0) {
                     Phi += ph;
                     Fx += ph * tab.Gx[q];
@@ -222,7 +221,8 @@ template <class S> struct AdjPairs { static constexpr bool value = !std::is_same
 // into buffer Adst.  g holds the pulled populations in stored units; the
 // cells' layout is lattice_tile's (kAlongX, CY, kAdj).
 template <class S, int CY, bool kInner, bool kAlongX, int kColl, bool kStream>
-__device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, const float *__restrict__ sov,
+__device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, const typename PhiArg<S>::type &pt,
+                                             const float *__restrict__ sov,
                                              const unsigned *__restrict__ m, const int W, const unsigned any,
                                              const int x, const int (&y)[CY], const bool (&valid)[CY],
                                              const Cell (&C)[CY], typename Real<S>::type (&g)[CY][9],
@@ -253,7 +253,7 @@ __device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, 
             R Fx, Fy, s_e, s_eps, s_nu[2], s_q[2];
 #pragma unroll
             for (int k = 0; k < 2; ++k)
-                cell_overlay<R, kStream>(I, tab, sov, m, W, any, x + k * RX, y[k], Fx, Fy, s_nu[k], s_e, s_eps,
+                cell_overlay<R, kStream>(I, tab, pt, sov, m, W, any, x + k * RX, y[k], Fx, Fy, s_nu[k], s_e, s_eps,
                                          s_q[k]);
             float2 v[9];
 #pragma unroll
@@ -269,7 +269,7 @@ __device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, 
     for (int k = 0; k < CY; ++k) {
         if (!valid[k]) continue;
         R Fx, Fy, s_nu, s_e, s_eps, s_q;
-        cell_overlay<R, kStream>(I, tab, sov, m, W, any, x + k * RX, y[k], Fx, Fy, s_nu, s_e, s_eps, s_q);
+        cell_overlay<R, kStream>(I, tab, pt, sov, m, W, any, x + k * RX, y[k], Fx, Fy, s_nu, s_e, s_eps, s_q);
         collide_cell<S, R, kColl>(I, g[k], Fx, Fy, s_nu, s_e, s_eps, s_q, forced);
     }
     store();
@@ -289,6 +289,7 @@ __device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, 
 // priority (the single-lattice sweep).
 template <class S, int CY, bool kInner, bool kAlongX, int kColl, bool kStream = false>
 __device__ __forceinline__ void lattice_tile(const Inst &I, S *__restrict__ pool, const BeadTab &tab,
+                                             const typename PhiArg<S>::type &pt,
                                              const unsigned *__restrict__ mask_read,
                                              const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear,
                                              const int bx, const int by, const int parity, const int early_load,
@@ -389,7 +390,7 @@ __device__ __forceinline__ void lattice_tile(const Inst &I, S *__restrict__ pool
     const float *sov = stage_overlay<R, kStream>(I, tab, m, any);  // every thread of the CTA
     if (!valid[0]) return;  // the thread's other cells (further along its column or row) are invalid too
     if (!early_load) pull();
-    finish_cells<S, CY, kInner, kAlongX, kColl, kStream>(I, tab, sov, m, W, any, x, y, valid, C, g, Adst, cx0, pol);
+    finish_cells<S, CY, kInner, kAlongX, kColl, kStream>(I, tab, pt, sov, m, W, any, x, y, valid, C, g, Adst, cx0, pol);
 }
 
 // Tile order of a single-lattice sweep.  Every other step takes the tiles
@@ -402,15 +403,17 @@ __device__ __forceinline__ void lattice_tile(const Inst &I, S *__restrict__ pool
 // (its state is many times the L2: reversing measured no gain there).
 __device__ __forceinline__ int tile_order(int b, int n, int parity) { return (parity & 1) ? n - 1 - b : b; }
 
-template <class S, int CY, bool kAlongX, int kColl>
+// kSplit: gridDim.z CTAs share a tile's rows (row_split).
+template <class S, int CY, bool kAlongX, int kColl, bool kSplit = false>
 __global__ void __launch_bounds__(kTileX *kTileY / CY)
     k_lattice(const Inst I, S *__restrict__ pool, const BeadTab tab, const unsigned *__restrict__ mask_read,
               const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear, const int parity,
-              const int early_load, const int early_cold) {
-    lattice_tile<S, CY, true, kAlongX, kColl, true>(I, pool, tab, mask_read, mask_prev, mask_clear,
+              const int early_load, const int early_cold, const typename PhiArg<S>::type pt) {
+    lattice_tile<S, CY, true, kAlongX, kColl, true>(I, pool, tab, pt, mask_read, mask_prev, mask_clear,
                                        tile_order(blockIdx.x, gridDim.x, parity),
                                        tile_order(blockIdx.y, gridDim.y, parity), parity, early_load, early_cold,
-                                       (blockIdx.x | blockIdx.y) == 0, threadIdx.x, threadIdx.y);
+                                       (blockIdx.x | blockIdx.y | (kSplit ? blockIdx.z : 0u)) == 0, threadIdx.x,
+                                       kSplit ? threadIdx.y + blockIdx.z * blockDim.y : threadIdx.y);
 }
 
 // --------------------------------------------- staged sweep (variants 3, 4)
@@ -549,7 +552,7 @@ __global__ void __launch_bounds__(kTileX *kTileY / 2)
     if (!inner) {
         for (int s = 0; s < NS && by0 + s < I.nty; ++s) {
             if (s) __syncthreads();  // the previous tile's cells no longer read the staged overlay
-            lattice_tile<S, 2, true, true, kCollTrt, true>(I, pool, tab, mask_read, mask_prev, mask_clear, bx, by0 + s,
+            lattice_tile<S, 2, true, true, kCollTrt, true>(I, pool, tab, NoPhi{}, mask_read, mask_prev, mask_clear, bx, by0 + s,
                                                            parity, early_load, early_cold, lead, tx, ty);
         }
         return;
@@ -618,7 +621,7 @@ __global__ void __launch_bounds__(kTileX *kTileY / 2)
             Cell C[2];  // unused: inner cells
             R g[2][9];
             pull_staged<S>(rows + (r * kRowStride + xt), s_halo, r, xt, g[0], g[1]);
-            finish_cells<S, 2, true, true, kCollTrt, true>(I, tab, sov, m, W, any, x, y, valid, C, g, Adst, cx0, pol);
+            finish_cells<S, 2, true, true, kCollTrt, true>(I, tab, NoPhi{}, sov, m, W, any, x, y, valid, C, g, Adst, cx0, pol);
         }
     }
 }
@@ -643,7 +646,8 @@ __global__ void __launch_bounds__(kTileX *kTileY / CY, BatchMinBlocks<S, CY>::va
     k_lattice_batch(const Inst *__restrict__ insts, const int2 *__restrict__ tiles, S *__restrict__ pool,
                     const BeadTab tab0, const BeadTab tab1, const unsigned *__restrict__ mask_read,
                     const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear, const int gparity,
-                    const int early_load, const int early_cold) {
+                    const int early_load, const int early_cold, const typename PhiArg<S>::type phi0,
+                    const typename PhiArg<S>::type phi1) {
     __shared__ Inst sI;
     const int2 t = tiles[blockIdx.x];
     {
@@ -655,8 +659,8 @@ __global__ void __launch_bounds__(kTileX *kTileY / CY, BatchMinBlocks<S, CY>::va
     __syncthreads();
     const int parity = gparity ^ sI.par_xor;
     lattice_tile<S, CY, BatchInner<S, CY, kAlongX>::value, kAlongX, kColl>(
-        sI, pool, parity ? tab1 : tab0, mask_read, mask_prev, mask_clear, t.y & 0xffff, t.y >> 16, parity,
-        early_load, early_cold, blockIdx.x == 0, threadIdx.x, threadIdx.y);
+        sI, pool, parity ? tab1 : tab0, parity ? phi1 : phi0, mask_read, mask_prev, mask_clear, t.y & 0xffff, t.y >> 16,
+        parity, early_load, early_cold, blockIdx.x == 0, threadIdx.x, threadIdx.y);
 }
 
 // ------------------------------------------------ vectorised sweep (variant 2)
@@ -817,6 +821,7 @@ __device__ __forceinline__ void vstore_pops(S *__restrict__ A, const Inst &I, co
 // before the scatter: the shuffles need the whole warp.
 template <class S>
 __device__ __forceinline__ void lattice_tile_vec(const Inst &I, S *__restrict__ pool, const BeadTab &tab,
+                                                 const typename PhiArg<S>::type &pt,
                                                  const unsigned *__restrict__ mask_read,
                                                  const unsigned *__restrict__ mask_prev,
                                                  unsigned *__restrict__ mask_clear, const int bx, const int by,
@@ -849,7 +854,7 @@ __device__ __forceinline__ void lattice_tile_vec(const Inst &I, S *__restrict__ 
 #pragma unroll
         for (int j = 0; j < NV; ++j) {
             R Fx, Fy, s_nu, s_e, s_eps, s_q;
-            cell_overlay<R, true>(I, tab, sov, m, W, any, x0 + j, y, Fx, Fy, s_nu, s_e, s_eps, s_q);
+            cell_overlay<R, true>(I, tab, pt, sov, m, W, any, x0 + j, y, Fx, Fy, s_nu, s_e, s_eps, s_q);
             collide_cell<S, R, kCollTrt>(I, g[j], Fx, Fy, s_nu, s_e, s_eps, s_q, forced);
         }
     }
@@ -860,8 +865,8 @@ template <class S>
 __global__ void __launch_bounds__(kTileX / VecWidth<S>::value * kTileY)
     k_lattice_vec(const Inst I, S *__restrict__ pool, const BeadTab tab, const unsigned *__restrict__ mask_read,
                   const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear, const int parity,
-                  const int early_load, const int early_cold) {
-    lattice_tile_vec<S>(I, pool, tab, mask_read, mask_prev, mask_clear, tile_order(blockIdx.x, gridDim.x, parity),
+                  const int early_load, const int early_cold, const typename PhiArg<S>::type pt) {
+    lattice_tile_vec<S>(I, pool, tab, pt, mask_read, mask_prev, mask_clear, tile_order(blockIdx.x, gridDim.x, parity),
                         tile_order(blockIdx.y, gridDim.y, parity), parity, early_load, early_cold,
                         (blockIdx.x | blockIdx.y) == 0);
 }
@@ -875,7 +880,8 @@ __global__ void __launch_bounds__(kTileX / VecWidth<S>::value * kTileY, BatchVec
     k_lattice_batch_vec(const Inst *__restrict__ insts, const int2 *__restrict__ tiles, S *__restrict__ pool,
                         const BeadTab tab0, const BeadTab tab1, const unsigned *__restrict__ mask_read,
                         const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear, const int gparity,
-                        const int early_load, const int early_cold) {
+                        const int early_load, const int early_cold, const typename PhiArg<S>::type phi0,
+                        const typename PhiArg<S>::type phi1) {
     constexpr int NT = kTileX / VecWidth<S>::value * kTileY;
     __shared__ Inst sI;
     const int2 t = tiles[blockIdx.x];
@@ -891,11 +897,11 @@ __global__ void __launch_bounds__(kTileX / VecWidth<S>::value * kTileY, BatchVec
     // on the same threads: NV cells per thread along y
     constexpr int NV = VecWidth<S>::value;
     if (sI.nx % NV == 0) {
-        lattice_tile_vec<S>(sI, pool, parity ? tab1 : tab0, mask_read, mask_prev, mask_clear, t.y & 0xffff,
+        lattice_tile_vec<S>(sI, pool, parity ? tab1 : tab0, parity ? phi1 : phi0, mask_read, mask_prev, mask_clear, t.y & 0xffff,
                             t.y >> 16, parity, early_load, early_cold, blockIdx.x == 0);
     } else {
         const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-        lattice_tile<S, NV, false, false, kCollTrt>(sI, pool, parity ? tab1 : tab0, mask_read, mask_prev,
+        lattice_tile<S, NV, false, false, kCollTrt>(sI, pool, parity ? tab1 : tab0, parity ? phi1 : phi0, mask_read, mask_prev,
                                                     mask_clear, t.y & 0xffff, t.y >> 16, parity, early_load,
                                                     early_cold, blockIdx.x == 0, tid % kTileX, tid / kTileX);
     }
@@ -1143,23 +1149,39 @@ static cudaError_t launch_staged(const Inst &I, void *pool, BeadTab tab, const S
                               after_beads, ec, mk.status, mk.copy_shortfall);
 }
 
+// CTAs a tile of the single-lattice sweep is split into by rows (variants 0
+// and 1): a lattice of few tiles would leave most SMs idle.
+template <class S> static int row_split(int ntiles) {
+    int sp = 1;
+    while (sp < kTileY && 2 * sp * ntiles <= (std::is_same<S, double>::value ? kSplitCtas64 : kSplitCtas)) sp *= 2;
+    return sp;
+}
+
+template <class S> static typename PhiArg<S>::type phi_arg(const PhiTab &p) {
+    if constexpr (std::is_same<S, double>::value) return p;
+    else return NoPhi{};
+}
+
 template <class S>
-static cudaError_t lattice_v(int variant, const Inst &I, void *pool, BeadTab tab, const SweepMasks &mk, int parity,
-                             int after_beads, cudaStream_t st) {
+static cudaError_t lattice_v(int variant, const Inst &I, void *pool, BeadTab tab, const PhiTab &phi,
+                             const SweepMasks &mk, int parity, int after_beads, cudaStream_t st) {
+    const auto pt = phi_arg<S>(phi);
     cudaLaunchAttribute attr[1];
     const dim3 grid(I.ntx, I.nty);
+    const int sp = row_split<S>(I.ntx * I.nty), rows = kTileY / sp;
+    const dim3 split(I.ntx, I.nty, sp);
     const int ec = after_beads ? mk.early_cold : 0;
     // constant Lallemand-Luo rates: the moment form, one cell per thread
     if (I.collision == 1) {
-        const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX, kTileY), after_beads, st, attr);
-        return cudaLaunchKernelEx(&cfg, k_lattice<S, 1, false, kCollMrt>, I, (S *)pool, tab, mk.read, mk.prev,
-                                  mk.clear, parity, after_beads, ec);
+        const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX, rows), after_beads, st, attr);
+        return cudaLaunchKernelEx(&cfg, sp > 1 ? k_lattice<S, 1, false, kCollMrt, true> : k_lattice<S, 1, false, kCollMrt>, I, (S *)pool, tab, mk.read, mk.prev,
+                                  mk.clear, parity, after_beads, ec, pt);
     }
     if (variant == 2 && I.nx % VecWidth<S>::value == 0) {
         const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX / VecWidth<S>::value, kTileY), after_beads,
                                                     st, attr);
         return cudaLaunchKernelEx(&cfg, k_lattice_vec<S>, I, (S *)pool, tab, mk.read, mk.prev, mk.clear,
-                                  parity, after_beads, ec);
+                                  parity, after_beads, ec, pt);
     }
     if constexpr (AdjPairs<S>::value) {
         // the bulk copies need the buffers 16-byte aligned (strips and rows
@@ -1171,13 +1193,13 @@ static cudaError_t lattice_v(int variant, const Inst &I, void *pool, BeadTab tab
         }
     }
     if (variant == 1 || variant == 3 || variant == 4) {
-        const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX / 2, kTileY), after_beads, st, attr);
-        return cudaLaunchKernelEx(&cfg, k_lattice<S, 2, true, kCollTrt>, I, (S *)pool, tab, mk.read, mk.prev,
-                                  mk.clear, parity, after_beads, ec);
+        const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX / 2, rows), after_beads, st, attr);
+        return cudaLaunchKernelEx(&cfg, sp > 1 ? k_lattice<S, 2, true, kCollTrt, true> : k_lattice<S, 2, true, kCollTrt>, I, (S *)pool, tab, mk.read, mk.prev,
+                                  mk.clear, parity, after_beads, ec, pt);
     }
-    const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX, kTileY), after_beads, st, attr);
-    return cudaLaunchKernelEx(&cfg, k_lattice<S, 1, false, kCollTrt>, I, (S *)pool, tab, mk.read, mk.prev,
-                              mk.clear, parity, after_beads, ec);
+    const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX, rows), after_beads, st, attr);
+    return cudaLaunchKernelEx(&cfg, sp > 1 ? k_lattice<S, 1, false, kCollTrt, true> : k_lattice<S, 1, false, kCollTrt>, I, (S *)pool, tab, mk.read, mk.prev,
+                              mk.clear, parity, after_beads, ec, pt);
 }
 
 // The staged sweep's CTAs keep 20-46 KB of static shared memory: its
@@ -1196,20 +1218,22 @@ cudaError_t prepare_lattice_kernels() {
     return cudaSuccess;
 }
 
-cudaError_t launch_lattice(int precision, const Inst *, const Inst &inst_h, void *pool, BeadTab tab,
+cudaError_t launch_lattice(int precision, const Inst *, const Inst &inst_h, void *pool, BeadTab tab, PhiTab phi,
                            const SweepMasks &masks, int parity, int after_beads, int variant, cudaStream_t st) {
     switch (precision) {
-        case 0: return lattice_v<double>(variant, inst_h, pool, tab, masks, parity, after_beads, st);
-        case 1: return lattice_v<float>(variant, inst_h, pool, tab, masks, parity, after_beads, st);
-        case 2: return lattice_v<__half>(variant, inst_h, pool, tab, masks, parity, after_beads, st);
+        case 0: return lattice_v<double>(variant, inst_h, pool, tab, phi, masks, parity, after_beads, st);
+        case 1: return lattice_v<float>(variant, inst_h, pool, tab, phi, masks, parity, after_beads, st);
+        case 2: return lattice_v<__half>(variant, inst_h, pool, tab, phi, masks, parity, after_beads, st);
     }
     return cudaErrorInvalidValue;
 }
 
 template <class S>
 static cudaError_t lattice_batch_v(int variant, const Inst *insts, const int2 *tiles, int ntiles, void *pool,
-                                   BeadTab tab0, BeadTab tab1, const SweepMasks &mk, int gparity, int after_beads,
-                                   int any_mrt, cudaStream_t st) {
+                                   const BeadTab tab[2], const PhiTab phi[2], const SweepMasks &mk, int gparity,
+                                   int after_beads, int any_mrt, cudaStream_t st) {
+    const BeadTab &tab0 = tab[0], &tab1 = tab[1];
+    const auto phi0 = phi_arg<S>(phi[0]), phi1 = phi_arg<S>(phi[1]);
     cudaLaunchAttribute attr[1];
     const dim3 grid(ntiles);
     const int ec = after_beads ? mk.early_cold : 0;
@@ -1218,32 +1242,32 @@ static cudaError_t lattice_batch_v(int variant, const Inst *insts, const int2 *t
     if (any_mrt) {
         const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX, kTileY), after_beads, st, attr);
         return cudaLaunchKernelEx(&cfg, k_lattice_batch<S, 1, false, kCollAny>, insts, tiles, (S *)pool, tab0, tab1,
-                                  mk.read, mk.prev, mk.clear, gparity, after_beads, ec);
+                                  mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1);
     }
     if (variant == 2) {
         const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX / VecWidth<S>::value, kTileY), after_beads,
                                                     st, attr);
         return cudaLaunchKernelEx(&cfg, k_lattice_batch_vec<S>, insts, tiles, (S *)pool, tab0, tab1, mk.read,
-                                  mk.prev, mk.clear, gparity, after_beads, ec);
+                                  mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1);
     }
     if (variant == 1 || variant == 3 || variant == 4) {  // the staged blocks are single-lattice only
         const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX / 2, kTileY), after_beads, st, attr);
         return cudaLaunchKernelEx(&cfg, k_lattice_batch<S, 2, true, kCollTrt>, insts, tiles, (S *)pool, tab0, tab1,
-                                  mk.read, mk.prev, mk.clear, gparity, after_beads, ec);
+                                  mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1);
     }
     const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX, kTileY), after_beads, st, attr);
     return cudaLaunchKernelEx(&cfg, k_lattice_batch<S, 1, false, kCollTrt>, insts, tiles, (S *)pool, tab0, tab1,
-                              mk.read, mk.prev, mk.clear, gparity, after_beads, ec);
+                              mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1);
 }
 
 cudaError_t launch_lattice_batch(int precision, const Inst *insts, const int2 *tiles, int ntiles, void *pool,
-                                 BeadTab tab0, BeadTab tab1, const SweepMasks &masks, int gparity, int after_beads,
-                                 int variant, int any_mrt, cudaStream_t st) {
+                                 const BeadTab tab[2], const PhiTab phi[2], const SweepMasks &masks, int gparity,
+                                 int after_beads, int variant, int any_mrt, cudaStream_t st) {
     if (ntiles <= 0) return cudaSuccess;
     switch (precision) {
-        case 0: return lattice_batch_v<double>(variant, insts, tiles, ntiles, pool, tab0, tab1, masks, gparity, after_beads, any_mrt, st);
-        case 1: return lattice_batch_v<float>(variant, insts, tiles, ntiles, pool, tab0, tab1, masks, gparity, after_beads, any_mrt, st);
-        case 2: return lattice_batch_v<__half>(variant, insts, tiles, ntiles, pool, tab0, tab1, masks, gparity, after_beads, any_mrt, st);
+        case 0: return lattice_batch_v<double>(variant, insts, tiles, ntiles, pool, tab, phi, masks, gparity, after_beads, any_mrt, st);
+        case 1: return lattice_batch_v<float>(variant, insts, tiles, ntiles, pool, tab, phi, masks, gparity, after_beads, any_mrt, st);
+        case 2: return lattice_batch_v<__half>(variant, insts, tiles, ntiles, pool, tab, phi, masks, gparity, after_beads, any_mrt, st);
     }
     return cudaErrorInvalidValue;
 }

@@ -21,6 +21,7 @@ struct fpd_sim {
     size_t pool_bytes = 0, tab_bytes = 0, mask_bytes = 0;  // sizes of pool, both tables, all masks
     double *tabmem = nullptr;       // two bead tables
     fpd::BeadTab tab[2]{};
+    fpd::PhiTab phi[2]{};           // FP64: profiles kept beside the tables
     unsigned *counters = nullptr;   // one per instance (bead-phase last-block)
     unsigned *status = nullptr;     // sticky FPD_FLAG_* bits of the instance (device word)
     unsigned *masks[fpd::kMaskBufs] = {};  // per-tile bead masks, in rotation by step (t % kMaskBufs)

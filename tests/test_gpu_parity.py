@@ -826,3 +826,80 @@ def test_staged_blocks_periodic_y_forced_and_sandwich(precision, variant):
         assert np.array_equal(pa, pb)
         for x, y in zip(a.beads(), b.beads()):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("precision,tol", [(0, 1e-12), (1, 2e-5)])
+@pytest.mark.parametrize("shape", ["wide support", "many beads", "edge of the list"])
+def test_bead_phase_shapes_vs_oracle(precision, tol, shape):
+    # the forms the bead phase takes: supports of more cells than one list
+    # holds (in FP64 also too large to keep the profiles of), more beads than
+    # a warp screens at once, a box of just over 1024 and 1280 cells
+    rng = np.random.default_rng(31)
+    if shape == "wide support":
+        cfg = wl.random_fiber(rng, 130, 131, n_beads=32, a=1.0, xi=8.0, n_fibers=2, precision=precision)
+    elif shape == "many beads":
+        cfg = wl.random_fiber(rng, 260, 90, n_beads=14, a=2.0, xi=0.5, n_fibers=5, precision=precision)
+    else:
+        cfg = wl.random_fiber(rng, 100, 80, n_beads=3, a=4.0, xi=1.45 if precision else 1.25, precision=precision)
+    steps = 3 if shape == "wide support" else 40
+    sim = gpu_sim(cfg)
+    sim.step(steps)
+    ux, uy, _ = sim.fields()
+    R, V = sim.beads()[:2]
+    sim.close()
+    ref = orc_sim(cfg)
+    ref.step(steps)
+    rx, ry, _ = ref.fields()
+    rR, rV = ref.beads()[:2]
+    eu = np.sqrt(np.sum((ux - rx) ** 2 + (uy - ry) ** 2) / np.sum(rx ** 2 + ry ** 2))
+    ev = np.linalg.norm(V - rV) / np.linalg.norm(rV)
+    print(f"{shape}, precision {precision}: u {eu:.1e}, V {ev:.1e}, R {np.abs(R - rR).max():.1e}")
+    assert eu < tol and ev < 10 * tol and np.abs(R - rR).max() < 10 * tol
+
+
+def test_bead_velocity_beyond_the_first_sum_range_vs_oracle():
+    # velocity terms of one cell per step and more do not fit the range the
+    # fixed-point sum tries first: with a bead pushed hard enough for that the
+    # first bead phase repeats it with more room (later steps amplify
+    # rounding: the flow is far outside the method's range)
+    rng = np.random.default_rng(5)
+    cfg = wl.random_fiber(rng, 64, 48, n_beads=1, a=2.0, xi=1.0, periodic_y=1, bead_fx=120.0,
+                          nu_f=0.5, stiffness_K=0.0)
+    sim, ref = gpu_sim(cfg), orc_sim(cfg)
+    sim.step(2)
+    ref.step(1)
+    assert np.abs(ref.fields()[0]).max() > 1.0
+    ref.step(1)
+    for x, y in zip(sim.beads()[:2], ref.beads()[:2]):
+        np.testing.assert_allclose(x, y, rtol=1e-12)
+    sim.close()
+
+
+def test_fp64_checkpoint_and_batch_rebuild_restore_the_kept_profiles(tmp_path):
+    # the FP64 bead phase reads profiles kept by the previous one: they are
+    # made again after a checkpoint is read, and when a batch moves them
+    rng = np.random.default_rng(8)
+    cfg = wl.random_fiber(rng, 90, 50, n_beads=6, a=2.0, xi=1.0)
+    whole = gpu_sim(cfg)
+    whole.step(45)
+    a = gpu_sim(cfg)
+    a.step(20)
+    a.save(str(tmp_path / "c"))
+    b = gpu_sim(cfg)
+    b.load(str(tmp_path / "c"))
+    b.step(25)
+    other = wl.random_fiber(rng, 60, 40, n_beads=4, a=2.0, xi=1.0)
+    from paper_2212_14153_gb300 import fpd
+    bat = fpd.Batch(0, 4, 32 << 20, 64)
+    gone, slot = bat.add(other, 7), bat.add(cfg, 45)
+    bat.run(7)
+    bat.remove(gone)
+    bat.run(10)
+    bat.add(other, 9)
+    while bat.run(100):
+        pass
+    want = whole.populations(), whole.beads()
+    for got in ((b.populations(), b.beads()), (bat.populations(slot), bat.beads(slot))):
+        assert np.array_equal(got[0], want[0])
+        for x, y in zip(got[1], want[1]):
+            assert np.array_equal(x, y)
