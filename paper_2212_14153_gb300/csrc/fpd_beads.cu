@@ -56,6 +56,8 @@ namespace {
 // hundred roundings of a sum averaging out, below the sum's above 1e-6.  A
 // caller that meets a larger term (mag) repeats the sum with a larger ex.
 constexpr int kVelBits = 0;
+constexpr float kEarlyMove = 0.499f;
+static_assert(kEarlyMove < kFastBead, "faster beads are judged by their FP64 velocity");
 template <class R> struct Fix;
 template <> struct Fix<float> {
     using T = long long;
@@ -408,6 +410,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     using T = typename F::T;
     constexpr int NW = NT / 32;
     constexpr int kCap = ListCap<R>::value;
+    constexpr int kPer = kCap / NT > 3 ? 3 : (kCap + NT - 1) / NT;  // box cells a thread lists at a time
     constexpr size_t kBuf = sizeof(SupportCell<R>) * kCap > sizeof(ForceShared<R>) ? sizeof(SupportCell<R>) * kCap
                                                                                    : sizeof(ForceShared<R>);
     __shared__ Inst sI;
@@ -417,9 +420,11 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     __shared__ int4 s_nbox[kF64 ? kMaxBeads : 1];  // a neighbour's kept box, and where its profile starts
     __shared__ int s_noff[kF64 ? kMaxBeads : 1];
     __shared__ SumShared<T, NW> s_sum;
-    __shared__ double s_R[2], s_unit;
+    __shared__ double s_R[2], s_S, s_unit;
     __shared__ Support s_sup;
-    __shared__ int s_n, s_redo;
+    __shared__ unsigned s_cnt[2][NW];
+    __shared__ int s_state;
+    __shared__ float s_unit_f;
     __shared__ unsigned s_seen;
     SupportCell<R> *list = reinterpret_cast<SupportCell<R> *>(s_buf);
 
@@ -442,19 +447,26 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         pdl_trigger();
     }
     {
-        // cooperative copy of the instance record (one 32-bit word a thread)
-        static_assert(sizeof(Inst) % 4 == 0, "Inst is copied as 32-bit words");
-        const unsigned *src = (const unsigned *)(insts + ii);
-        unsigned *dst = (unsigned *)&sI;
-        for (int wd = tid; wd < (int)(sizeof(Inst) / 4); wd += NT) dst[wd] = src[wd];
+        // asynchronous copy of the instance record, 8 bytes a thread (a plain
+        // copy's stores would hold back the loads below until it arrived)
+        static_assert(sizeof(Inst) % 8 == 0 && alignof(Inst) == 8, "Inst is copied 8 bytes at a time");
+        for (int wd = tid; wd < (int)(sizeof(Inst) / 8); wd += NT)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                             static_cast<unsigned>(__cvta_generic_to_shared((uint64_t *)&sI + wd))),
+                         "l"((const uint64_t *)(insts + ii) + wd)
+                         : "memory");
     }
+    auto record_here = []() {
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncthreads();
+    };
     // Up to pdl_wait() only the records and the old table are read: the
     // preceding launch, a sweep, may still be running, but it was released
     // after the bead phase that wrote this table had completed (its lead CTA
     // waits for it).  Table reads go to L2 (an SM's L1 may hold lines of an
     // earlier step).
     int any_close = 0;  // some bead may come within the excluded volume's reach of this one
-    double Rx = 0.0, Ry = 0.0;  // the bead's old position
+    double Rx = 0.0, Ry = 0.0, S_old = 1.0;  // the bead's old position, support sum
     float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f;
     if (advance) {
         xh = __ldcg(told.xh + b);
@@ -463,7 +475,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         yl = __ldcg(told.yl + b);
         Rx = __ldcg(told.Rx + b);
         Ry = __ldcg(told.Ry + b);
-        if (tid == NT - 1) s_unit = 1.0 / __ldcg(told.S + b);
+        if (tid == NT - 1) S_old = __ldcg(told.S + b);
     }
     // the lattice cell of row cj, column ci of a support box
     auto cell_of = [](const Inst &I, const Support &bx, int ci, int cj, int &i, int &j) {
@@ -502,7 +514,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
                     nbr.gy = __ldcg(told.gyf + gq);
                 }
             }
-            if (q0 == 0) __syncthreads();  // the record is in place
+            if (q0 == 0) record_here();
             // nearest image of the bead from bead q: the high parts' image
             // shift is a whole number of cells, removed exactly
             const float fnx = (float)I.nx, fny = (float)I.ny;
@@ -533,7 +545,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             }
             nn += __popc(m);
         }
-        if constexpr (kF64) __syncthreads();  // the neighbours are in place (FP32: make_list's barrier)
+        if constexpr (kF64) __syncthreads();  // the neighbours are in place (FP32: make_list's first barrier)
         // populations are pulled from the current buffer
         const S *A = pop_buffer(pool, I, parity);
         const bool kept = kF64 && I.phi_cap != 0;
@@ -550,40 +562,52 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         const float inv_w = inv_width(bx);
         // List the support cells (phi_b != 0) among box cells [c0, c1),
         // c1 - c0 <= kCap, with the force density of the previous table.
-        // Their order differs from run to run; the sums do not depend on it.
         auto make_list = [&](int c0, int c1) -> int {
-            if (tid == 0) s_n = 0;
-            __syncthreads();
+            int n = 0;
 #pragma unroll 1
-            for (int cb = c0 + 32 * w; cb < c1; cb += NT) {
-                const int c = cb + lane;
-                R ph = (R)0;
-                if (c < c1) {
-                    int ci, cj;
-                    cell_rc(bx, inv_w, c, ci, cj);
-                    if constexpr (kF64) {
-                        if (kept) {
-                            ph = __ldcg(pold.phi + s_noff[self] + c);
+            for (int r0 = c0, buf = 0; r0 < c1; r0 += kPer * NT, buf ^= 1) {
+                // kPer cells a thread: independent evaluations in flight
+                R ph[kPer];
+                unsigned m[kPer], cnt = 0u;
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    const int c = r0 + k * NT + tid;
+                    ph[k] = (R)0;
+                    if (c < c1) {
+                        int ci, cj;
+                        cell_rc(bx, inv_w, c, ci, cj);
+                        if constexpr (kF64) {
+                            if (kept) {
+                                ph[k] = __ldcg(pold.phi + s_noff[self] + c);
+                            } else {
+                                int i, j;
+                                cell_of(I, bx, ci, cj, i, j);
+                                ph[k] = phi_f64(I, i + 0.5, j + 0.5, Rx, Ry);
+                            }
                         } else {
-                            int i, j;
-                            cell_of(I, bx, ci, cj, i, j);
-                            ph = phi_f64(I, i + 0.5, j + 0.5, Rx, Ry);
+                            ph[k] = phi_f32(bx.rel[0] + (float)ci, bx.rel[1] + (float)cj, I.f_a, I.f_inv_xi, I.f_rcut2);
                         }
-                    } else {
-                        ph = phi_f32(bx.rel[0] + (float)ci, bx.rel[1] + (float)cj, I.f_a, I.f_inv_xi, I.f_rcut2);
                     }
+                    m[k] = __ballot_sync(0xffffffffu, ph[k] != (R)0);
+                    cnt += __popc(m[k]);
                 }
-                const unsigned m = __ballot_sync(0xffffffffu, ph != (R)0);
-                int at = 0;
-                if (lane == 0) at = atomicAdd(&s_n, __popc(m));
-                at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
-                if (ph != (R)0) {
-                    list[at].phi = ph;
-                    list[at].o = c;
+                // places: after the cells of the warps before this one
+                if (lane == 0) s_cnt[buf][w] = cnt;
+                __syncthreads();
+                const unsigned of = lane < NW ? s_cnt[buf][lane] : 0u;
+                int at = n + (int)__reduce_add_sync(0xffffffffu, lane < w ? of : 0u);
+                n += (int)__reduce_add_sync(0xffffffffu, of);
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    if (ph[k] != (R)0) {
+                        SupportCell<R> &sc = list[at + __popc(m[k] & ((1u << lane) - 1u))];
+                        sc.phi = ph[k];
+                        sc.o = r0 + k * NT + tid;
+                    }
+                    at += __popc(m[k]);
                 }
             }
             __syncthreads();
-            const int n = s_n;
             // entries tid, tid + NT, ... are read back by this thread only
 #pragma unroll 1
             for (int e = tid; e < n; e += NT) {
@@ -639,7 +663,10 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         };
         const int ncell = bx.n[0] * bx.n[1], share = (ncell + parts - 1) / parts;
         const int c_lo = min(part * share, ncell), c_hi = min(c_lo + share, ncell);
-        if (tid == NT - 1) s_unit *= pow2(-(F::kTop - kVelBits - bit_length(ncell)));
+        if (tid == NT - 1) {
+            s_unit = 1.0 / S_old * pow2(-(F::kTop - kVelBits - bit_length(ncell)));
+            s_unit_f = (float)s_unit;
+        }
         int n = make_list(c_lo, min(c_lo + kCap, c_hi));
         // wait for the preceding sweep (the populations read below), then let
         // the next sweep launch at once: its tiles that no bead marked start
@@ -693,47 +720,68 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
                 n = make_list(c0, min(c0 + kCap, c_hi));
             }
             total<R, NT, 2>(ax, ay, mx, s_sum, uses);
+            // FP32 paths: the new support box from the old place and V in FP32,
+            // a few instructions, so that the support sum need not wait for
+            // the FP64 chain of the move (FP64 instructions cost a warp 64
+            // cycles or more each): V clearly below kFastBead, whose rounding
+            // (2^-25) is far below the box offsets' own
             if (w == 0) {
                 const int need = F::need(mx);
-                const bool redo = need > bound && F::finite(mx);
-                if (!redo) {
-                    // lane 0: x, the others: y
-                    const double t = (double)(lane == 0 ? ax : ay);
-                    const double unit = s_unit * pow2(bound - kVelBits);
-                    const double v = F::finite(mx) ? t * unit : __longlong_as_double(0x7ff8000000000000ll);
-                    const double r = (lane == 0 ? Rx : Ry) + v;
+                int state = need > bound && F::finite(mx) ? need : -1;  // > 0: once more with this bound
+                if constexpr (!kF64) {
+                    const float vx = (float)ax * s_unit_f, vy = (float)ay * s_unit_f;
+                    if (state < 0 && bound == kVelBits && F::finite(mx) && fabsf(vx) < kEarlyMove && fabsf(vy) < kEarlyMove &&
+                        !far_off(xh, yh)) {
+                        state = 0;
+                        if (lane < 2)
+                            support_axis(I, lane, lane ? yh : xh, lane ? yl + vy : xl + vx, false, 0.0, 0.0,
+                                         s_sup.lo[lane], s_sup.n[lane], s_sup.rel[lane]);
+                    }
+                }
+                if (lane == 0) s_state = state;
+            }
+            __syncthreads();
+            const int state = s_state;
+            if (state > 0) {
+                // a term of magnitude 2^kVelBits or more (a diverging run): once
+                // more with room for it
+                bound = state;
+                n = make_list(c_lo, min(c_lo + kCap, c_hi));
+                continue;
+            }
+            if (w == 0) {
+                // the move; lane 0: x, the others: y
+                double unit = s_unit;
+                if (bound != kVelBits) unit *= pow2(bound - kVelBits);
+                double v = (double)(lane == 0 ? ax : ay) * unit;
+                if (!F::finite(mx)) v = __longlong_as_double(0x7ff8000000000000ll);
+                const double r = (lane == 0 ? Rx : Ry) + v;
+                if (part == 0 && lane < 2) {
+                    (lane ? tnew.Ry : tnew.Rx)[b] = r;
+                    (lane ? tnew.Vy : tnew.Vx)[b] = v;
+                }
+                if (lane < 2) s_R[lane] = r;
+                if (state < 0) {
                     const float h = (float)r, l = (float)(r - (double)h);
                     const double rx = __shfl_sync(0xffffffffu, r, 0), ry = __shfl_sync(0xffffffffu, r, 1);
                     const bool far = far_off(__shfl_sync(0xffffffffu, h, 0), __shfl_sync(0xffffffffu, h, 1));
-                    if (lane < 2) {
-                        support_axis(I, lane, h, l, far, rx, ry, s_sup.lo[lane], s_sup.n[lane], s_sup.rel[lane]);
-                        s_R[lane] = r;
-                    }
+                    if (lane < 2) support_axis(I, lane, h, l, far, rx, ry, s_sup.lo[lane], s_sup.n[lane], s_sup.rel[lane]);
                     // fast-bead guard (below): this bead's bits, |v| >=
                     // kFastBead or not finite by the high word
                     const unsigned hv = (unsigned)__double2hiint(v) & 0x7fffffffu;
                     const bool fast = hv >= (unsigned)__double2hiint(kFastBead);
                     any_close |= __any_sync(0xffffffffu, fast);
-                    if (part == 0 && lane < 2) {
-                        (lane ? tnew.Ry : tnew.Rx)[b] = r;
-                        (lane ? tnew.Vy : tnew.Vx)[b] = v;
-                        if (status && fast)
-                            atomicOr(status + ii, kFlagFastBead | (hv >= 0x7ff00000u ? kFlagNonFinite : 0u));
-                    }
+                    if (part == 0 && lane < 2 && status && fast)
+                        atomicOr(status + ii, kFlagFastBead | (hv >= 0x7ff00000u ? kFlagNonFinite : 0u));
                 }
-                if (lane == 0) s_redo = redo ? need : 0;
             }
-            __syncthreads();
-            if (s_redo == 0) break;
-            // a term of magnitude 2^kVelBits or more (a diverging run): once
-            // more with room for it
-            bound = s_redo;
-            n = make_list(c_lo, min(c_lo + kCap, c_hi));
+            if (state < 0) __syncthreads();
+            break;
         }
     } else {
         pdl_wait();
         pdl_trigger();
-        __syncthreads();  // the record is in place
+        record_here();
         any_close = 1;
         if (tid < 2) {
             const double rx = tnew.Rx[b], ry = tnew.Ry[b], r = tid ? ry : rx;
@@ -754,7 +802,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     const int c_lo = min(part * share, ncell), c_hi = min(c_lo + share, ncell);
     const int s_shift = F::kTop - 1 - bit_length(ncell);  // phi < 2
 #pragma unroll 1
-    for (int c = c_lo + tid; c < c_hi; c += NT) {
+    for (int c = c_lo + (tid + NT - 32) % NT; c < c_hi; c += NT) {  // warp 0, busy with the move, comes last
         R ph;
         int ci, cj;
         cell_rc(bx, inv_w, c, ci, cj);
@@ -781,9 +829,12 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     // warp 0 hands in the bead (R, V and S) while the others mark tiles.  An
     // arrival counts 1, and 2^16 if the excluded volume may act on the bead.
     if (w == 0) {
-        if (lane == 0) tnew.S[b] = (double)acc * pow2(-s_shift);
+        if (lane == 0) s_S = tnew.S[b] = (double)acc * pow2(-s_shift);
         __syncwarp();  // lane 1's R and V before lane 0's release
-        if (lane == 0) s_seen = arrive_acq_rel(&counters[ii], any_close ? 0x10001u : 1u) | (any_close ? 0x10000u : 0u);
+        if (lane == 0) {
+            s_seen = 0u;
+            if (nb > 1) s_seen = arrive_acq_rel(&counters[ii], any_close ? 0x10001u : 1u) | (any_close ? 0x10000u : 0u);
+        }
     } else {
         // FP32 overlay table: x (and y when periodic) wrapped into the
         // lattice, split into hi + lo
@@ -832,8 +883,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     const int items = 2 * nb, N = I.n_beads;
     const float inv_n = 1.0f / (float)N;
     for (int k = tid; k < items; k += NT) {
-        fs.r[k] = __ldcg(((k & 1) ? tnew.Ry : tnew.Rx) + first + (k >> 1));
-        if (!(k & 1)) fs.S[k >> 1] = __ldcg(tnew.S + first + (k >> 1));
+        fs.r[k] = nb == 1 ? s_R[k] : __ldcg(((k & 1) ? tnew.Ry : tnew.Rx) + first + (k >> 1));
+        if (!(k & 1)) fs.S[k >> 1] = nb == 1 ? s_S : __ldcg(tnew.S + first + (k >> 1));
     }
     __syncthreads();
     // fast-bead guard: the early update of unmarked tiles assumes a bead
