@@ -699,11 +699,22 @@ int fpd_get_tuning(const fpd_sim *s, int32_t *variant, int32_t *n_variants) {
 
 int fpd_sync(fpd_sim *s) {
     if (!s) return fail(nullptr, FPD_EINVAL, "fpd_sync: NULL handle");
-    cudaError_t e = cudaStreamSynchronize(s->stream);
-    if (e != cudaSuccess) return cuda_fail(s, e, "stream synchronize");
     unsigned flags = 0;
-    e = cudaMemcpy(&flags, s->status, sizeof flags, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(s, e, "read status");
+    cudaError_t e;
+    if (s->host_stage) {
+        // the status word follows the queued work into page-locked memory:
+        // one wait instead of two (a synchronous copy after it took 8.6 us)
+        unsigned *word = (unsigned *)(s->host_stage + 7 * (size_t)s->inst.nb);
+        e = cudaMemcpyAsync(word, s->status, sizeof flags, cudaMemcpyDeviceToHost, s->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+        if (e != cudaSuccess) return cuda_fail(s, e, "stream synchronize");
+        flags = *word;
+    } else {
+        e = cudaStreamSynchronize(s->stream);
+        if (e != cudaSuccess) return cuda_fail(s, e, "stream synchronize");
+        e = cudaMemcpy(&flags, s->status, sizeof flags, cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return cuda_fail(s, e, "read status");
+    }
     if (flags & fpd::kFlagNonFinite)
         return fail(s, FPD_ENAN, "non-finite state found by step %lld (FPD_FLAG_NONFINITE)", (long long)s->nstep);
     if (flags & fpd::kFlagCopyTimeout)
@@ -768,7 +779,7 @@ int fpd_read_beads(fpd_sim *s, double *pos, double *vel, double *force, double *
     // R, V, F, S of a table are seven consecutive arrays of nb doubles: one
     // copy into pinned staging memory, ordered after the queued steps
     if (!s->host_stage) {
-        cudaError_t e = cudaMallocHost(&s->host_stage, 7 * (size_t)nb * sizeof(double));
+        cudaError_t e = cudaMallocHost(&s->host_stage, (7 * (size_t)nb + 1) * sizeof(double));
         if (e != cudaSuccess) {
             s->host_stage = nullptr;
             return cuda_fail(s, e, "pinned staging for bead reads");

@@ -124,6 +124,8 @@ struct fpd_batch {
     cudaStream_t cap_stream = nullptr;
     double *phi_mem = nullptr;  // FP64: both tables' kept profiles (PhiTab::phi)
     int64_t phi_len = 0;        // doubles in phi_mem
+    double *host_stage = nullptr;  // pinned staging for bead reads (7 doubles a bead of the largest read so far)
+    int host_beads = 0;
     double *scratch = nullptr;
     size_t scratch_bytes = 0;
     std::string err;
@@ -171,6 +173,7 @@ void free_batch(fpd_batch *b) {
     cudaFree(b->beads_all_d);
     cudaFree(b->beads_old_d);
     cudaFree(b->beads_fresh_d);
+    if (b->host_stage) cudaFreeHost(b->host_stage);
     cudaFree(b->phi_mem);
     for (auto &p : b->phi) cudaFree(p.box);
     cudaFree(b->scratch);
@@ -724,31 +727,42 @@ int fpd_batch_read_populations(fpd_batch *b, int32_t slot, double *f) {
 int fpd_batch_read_beads(fpd_batch *b, int32_t slot, double *pos, double *vel, double *force, double *support) {
     int rc = slot_ok(b, slot);
     if (rc) return rc;
-    if ((rc = fpd_batch_sync(b))) return rc;
     const Slot &sl = b->slots[slot];
     const int nb = sl.inst.nb, off = sl.inst.bead_off;
-    if (nb == 0) return FPD_OK;
+    if (nb == 0) return fpd_batch_sync(b);
+    if (nb > b->host_beads) {
+        if (b->host_stage) cudaFreeHost(b->host_stage);
+        b->host_stage = nullptr;
+        b->host_beads = 0;
+        const cudaError_t e = cudaMallocHost(&b->host_stage, 7 * (size_t)nb * sizeof(double));
+        if (e != cudaSuccess) {
+            b->host_stage = nullptr;
+            return bcuda(b, e, "pinned staging for bead reads");
+        }
+        b->host_beads = nb;
+    }
+    // R, V, F, S of a table are seven consecutive arrays of max_beads
+    // doubles: one strided copy into pinned memory, ordered after the queued
+    // steps, instead of seven synchronous ones (59 us a slot)
     const int64_t l = sl.steps_done;
     const fpd::BeadTab &t = b->tab[l == 0 ? 0 : (int)((l - 1) & 1)];
-    std::vector<double> a(nb), c(nb);
-    auto pair = [&](double *dst, const double *dx, const double *dy) -> int {
-        if (!dst) return FPD_OK;
-        cudaError_t e = cudaMemcpy(a.data(), dx + off, nb * sizeof(double), cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess) e = cudaMemcpy(c.data(), dy + off, nb * sizeof(double), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return bcuda(b, e, "copy beads");
+    const size_t row = nb * sizeof(double), pitch = (size_t)(b->max_beads > 0 ? b->max_beads : 1) * sizeof(double);
+    cudaError_t e = cudaMemcpy2DAsync(b->host_stage, row, t.Rx + off, pitch, row, 7, cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return bcuda(b, e, "copy beads");
+    const double *h = b->host_stage;
+    auto pair = [&](double *dst, int k) {
+        if (!dst) return;
+        const double *x = h + (size_t)k * nb, *y = x + nb;
         for (int i = 0; i < nb; ++i) {
-            dst[2 * i] = a[i];
-            dst[2 * i + 1] = c[i];
+            dst[2 * i] = x[i];
+            dst[2 * i + 1] = y[i];
         }
-        return FPD_OK;
     };
-    if ((rc = pair(pos, t.Rx, t.Ry))) return rc;
-    if ((rc = pair(vel, t.Vx, t.Vy))) return rc;
-    if ((rc = pair(force, t.Fx, t.Fy))) return rc;
-    if (support) {
-        cudaError_t e = cudaMemcpy(support, t.S + off, nb * sizeof(double), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return bcuda(b, e, "copy support sums");
-    }
+    pair(pos, 0);
+    pair(vel, 2);
+    pair(force, 4);
+    if (support) std::copy(h + 6 * (size_t)nb, h + 7 * (size_t)nb, support);
     return FPD_OK;
 }
 

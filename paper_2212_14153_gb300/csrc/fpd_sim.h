@@ -42,7 +42,7 @@ struct fpd_sim {
     double launches[2] = {0, 0};
     // captured step chunks, one per starting parity (see fpd_step)
     bool use_graphs = true;
-    double *host_stage = nullptr;  // pinned staging for bead reads (7 nb doubles)
+    double *host_stage = nullptr;  // pinned staging for bead reads (7 nb doubles) and the status word
     // completion events of stream-ordered bead reads, by ticket % kReadTickets
     static constexpr int kReadTickets = 8;
     cudaEvent_t read_ev[kReadTickets] = {};
