@@ -350,7 +350,8 @@ int enqueue_step(fpd_sim *s, cudaStream_t st, int64_t t, bool profiled) {
     // from step 1 on, the previous bead phase (or the initial marks) is in
     // the previous buffer
     const fpd::SweepMasks mk{s->masks[t % M], s->masks[(t + M - 1) % M], s->masks[(t + 1) % M],
-                             (t >= 1 && s->early_cold) ? 1 : 0, s->status, s->copy_shortfall};
+                             (t >= 1 && s->early_cold) ? 1 : 0, s->status, (I.nb == 0 && !profiled) ? 1 : 0,
+                             s->copy_shortfall};
     e = fpd::launch_lattice(s->precision, s->inst_d, I, s->pool, s->tab[parity], s->phi[parity], mk, parity,
                             after_beads, s->variant, st);
     if (e != cudaSuccess) return cuda_fail(s, e, "lattice kernel launch");

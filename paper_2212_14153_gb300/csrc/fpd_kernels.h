@@ -35,6 +35,10 @@ struct SweepMasks {
     unsigned *clear;       // zeroed for the next bead phase
     int early_cold;
     unsigned *status = nullptr;  // the instance's status word (staged sweep)
+    // 1: launch the sweep as a programmatic dependent of the previous launch
+    // although no bead phase precedes it (a chain without beads): its CTAs
+    // are in place when that one ends, and wait for it before they read
+    int chained = 0;
     unsigned copy_shortfall = 0;  // test only: extra bytes the staged copies expect (their waits run out)
 };
 

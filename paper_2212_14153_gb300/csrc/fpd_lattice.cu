@@ -89,7 +89,7 @@ __device__ __forceinline__ void cell_overlay(const Inst &I, const BeadTab &tab, 
             while (bits) {
                 const int q = I.bead_off + 32 * w + __ffs(bits) - 1;
                 bits &= bits - 1u;
-                const double ph = phi_cell(I, tab, pt, q, x, y);
+                const double ph = phi_cell(I, tab, pt.phi, q, x, y);
                 if (ph != 0.0) {
                     Phi += ph;
                     Fx += ph * tab.Gx[q];
@@ -166,8 +166,8 @@ constexpr int kCollTrt = 0, kCollMrt = 1, kCollAny = 2;
 template <int kColl> __device__ __forceinline__ bool moment_form(const Inst &I, bool forced) {
     return kColl == kCollMrt || (kColl == kCollAny && I.collision == 1) || forced;
 }
-template <class S, class R, int kColl>
-__device__ __forceinline__ void collide_cell(const Inst &I, R g[9], R Fx, R Fy, R s_nu, R s_e, R s_eps, R s_q,
+template <class S, class R, int kColl, class P>
+__device__ __forceinline__ void collide_cell(const Inst &I, const P &pt, R g[9], R Fx, R Fy, R s_nu, R s_e, R s_eps, R s_q,
                                              bool forced) {
     constexpr bool kScaled = Store<S>::kScaled;
     if (moment_form<kColl>(I, forced)) {
@@ -180,6 +180,9 @@ __device__ __forceinline__ void collide_cell(const Inst &I, R g[9], R Fx, R Fy, 
 #pragma unroll
             for (int k = 0; k < 9; ++k) g[k] *= (R)I.scale[k];
         }
+    } else if constexpr (std::is_same<S, double>::value) {
+        if (!I.sandwich) collide_trt(g, pt.fluid);
+        else collide_trt(g, trt_rates(s_nu, s_q));
     } else {
         collide_trt<R, kScaled>(g, s_nu, s_q, I);
     }
@@ -221,7 +224,7 @@ template <class S> struct AdjPairs { static constexpr bool value = !std::is_same
 // into buffer Adst.  g holds the pulled populations in stored units; the
 // cells' layout is lattice_tile's (kAlongX, CY, kAdj).
 template <class S, int CY, bool kInner, bool kAlongX, int kColl, bool kStream>
-__device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, const typename PhiArg<S>::type &pt,
+__device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, const typename SweepArg<S>::type &pt,
                                              const float *__restrict__ sov,
                                              const unsigned *__restrict__ m, const int W, const unsigned any,
                                              const int x, const int (&y)[CY], const bool (&valid)[CY],
@@ -270,7 +273,7 @@ __device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, 
         if (!valid[k]) continue;
         R Fx, Fy, s_nu, s_e, s_eps, s_q;
         cell_overlay<R, kStream>(I, tab, pt, sov, m, W, any, x + k * RX, y[k], Fx, Fy, s_nu, s_e, s_eps, s_q);
-        collide_cell<S, R, kColl>(I, g[k], Fx, Fy, s_nu, s_e, s_eps, s_q, forced);
+        collide_cell<S, R, kColl>(I, pt, g[k], Fx, Fy, s_nu, s_e, s_eps, s_q, forced);
     }
     store();
 }
@@ -289,7 +292,7 @@ __device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, 
 // priority (the single-lattice sweep).
 template <class S, int CY, bool kInner, bool kAlongX, int kColl, bool kStream = false>
 __device__ __forceinline__ void lattice_tile(const Inst &I, S *__restrict__ pool, const BeadTab &tab,
-                                             const typename PhiArg<S>::type &pt,
+                                             const typename SweepArg<S>::type &pt,
                                              const unsigned *__restrict__ mask_read,
                                              const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear,
                                              const int bx, const int by, const int parity, const int early_load,
@@ -408,7 +411,7 @@ template <class S, int CY, bool kAlongX, int kColl, bool kSplit = false>
 __global__ void __launch_bounds__(kTileX *kTileY / CY)
     k_lattice(const Inst I, S *__restrict__ pool, const BeadTab tab, const unsigned *__restrict__ mask_read,
               const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear, const int parity,
-              const int early_load, const int early_cold, const typename PhiArg<S>::type pt) {
+              const int early_load, const int early_cold, const typename SweepArg<S>::type pt) {
     lattice_tile<S, CY, true, kAlongX, kColl, true>(I, pool, tab, pt, mask_read, mask_prev, mask_clear,
                                        tile_order(blockIdx.x, gridDim.x, parity),
                                        tile_order(blockIdx.y, gridDim.y, parity), parity, early_load, early_cold,
@@ -626,6 +629,19 @@ __global__ void __launch_bounds__(kTileX *kTileY / 2)
     }
 }
 
+// The FP64 sweep's argument of one instance of a batch (every thread calls it).
+template <class S>
+__device__ __forceinline__ void batch_arg(typename SweepArg<S>::type &arg, const Inst &I,
+                                          const typename PhiArg<S>::type &phi) {
+    if constexpr (std::is_same<S, double>::value) {
+        if (threadIdx.x == 0 && threadIdx.y == 0) {
+            arg.phi = phi;
+            arg.fluid = trt_rates(I.fluid_rates_d[0], I.fluid_rates_d[3]);
+        }
+        __syncthreads();
+    }
+}
+
 // Batched sweep over a packed tile list: tiles[t] = (instance slot,
 // by << 16 | bx).  Each instance reads table and layout of its own parity
 // (global parity ^ par_xor); the record is copied to shared memory per CTA.
@@ -658,9 +674,11 @@ __global__ void __launch_bounds__(kTileX *kTileY / CY, BatchMinBlocks<S, CY>::va
     }
     __syncthreads();
     const int parity = gparity ^ sI.par_xor;
+    __shared__ typename SweepArg<S>::type arg;
+    batch_arg<S>(arg, sI, parity ? phi1 : phi0);
     lattice_tile<S, CY, BatchInner<S, CY, kAlongX>::value, kAlongX, kColl>(
-        sI, pool, parity ? tab1 : tab0, parity ? phi1 : phi0, mask_read, mask_prev, mask_clear, t.y & 0xffff, t.y >> 16,
-        parity, early_load, early_cold, blockIdx.x == 0, threadIdx.x, threadIdx.y);
+        sI, pool, parity ? tab1 : tab0, arg, mask_read, mask_prev, mask_clear, t.y & 0xffff, t.y >> 16, parity,
+        early_load, early_cold, blockIdx.x == 0, threadIdx.x, threadIdx.y);
 }
 
 // ------------------------------------------------ vectorised sweep (variant 2)
@@ -821,7 +839,7 @@ __device__ __forceinline__ void vstore_pops(S *__restrict__ A, const Inst &I, co
 // before the scatter: the shuffles need the whole warp.
 template <class S>
 __device__ __forceinline__ void lattice_tile_vec(const Inst &I, S *__restrict__ pool, const BeadTab &tab,
-                                                 const typename PhiArg<S>::type &pt,
+                                                 const typename SweepArg<S>::type &pt,
                                                  const unsigned *__restrict__ mask_read,
                                                  const unsigned *__restrict__ mask_prev,
                                                  unsigned *__restrict__ mask_clear, const int bx, const int by,
@@ -855,7 +873,7 @@ __device__ __forceinline__ void lattice_tile_vec(const Inst &I, S *__restrict__ 
         for (int j = 0; j < NV; ++j) {
             R Fx, Fy, s_nu, s_e, s_eps, s_q;
             cell_overlay<R, true>(I, tab, pt, sov, m, W, any, x0 + j, y, Fx, Fy, s_nu, s_e, s_eps, s_q);
-            collide_cell<S, R, kCollTrt>(I, g[j], Fx, Fy, s_nu, s_e, s_eps, s_q, forced);
+            collide_cell<S, R, kCollTrt>(I, pt, g[j], Fx, Fy, s_nu, s_e, s_eps, s_q, forced);
         }
     }
     vstore_pops<S, NV>(Adst, I, C, g);
@@ -865,7 +883,7 @@ template <class S>
 __global__ void __launch_bounds__(kTileX / VecWidth<S>::value * kTileY)
     k_lattice_vec(const Inst I, S *__restrict__ pool, const BeadTab tab, const unsigned *__restrict__ mask_read,
                   const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear, const int parity,
-                  const int early_load, const int early_cold, const typename PhiArg<S>::type pt) {
+                  const int early_load, const int early_cold, const typename SweepArg<S>::type pt) {
     lattice_tile_vec<S>(I, pool, tab, pt, mask_read, mask_prev, mask_clear, tile_order(blockIdx.x, gridDim.x, parity),
                         tile_order(blockIdx.y, gridDim.y, parity), parity, early_load, early_cold,
                         (blockIdx.x | blockIdx.y) == 0);
@@ -893,15 +911,17 @@ __global__ void __launch_bounds__(kTileX / VecWidth<S>::value * kTileY, BatchVec
     }
     __syncthreads();
     const int parity = gparity ^ sI.par_xor;
+    __shared__ typename SweepArg<S>::type arg;
+    batch_arg<S>(arg, sI, parity ? phi1 : phi0);
     // an instance whose width is not a multiple of NV runs the column form
     // on the same threads: NV cells per thread along y
     constexpr int NV = VecWidth<S>::value;
     if (sI.nx % NV == 0) {
-        lattice_tile_vec<S>(sI, pool, parity ? tab1 : tab0, parity ? phi1 : phi0, mask_read, mask_prev, mask_clear, t.y & 0xffff,
+        lattice_tile_vec<S>(sI, pool, parity ? tab1 : tab0, arg, mask_read, mask_prev, mask_clear, t.y & 0xffff,
                             t.y >> 16, parity, early_load, early_cold, blockIdx.x == 0);
     } else {
         const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-        lattice_tile<S, NV, false, false, kCollTrt>(sI, pool, parity ? tab1 : tab0, parity ? phi1 : phi0, mask_read, mask_prev,
+        lattice_tile<S, NV, false, false, kCollTrt>(sI, pool, parity ? tab1 : tab0, arg, mask_read, mask_prev,
                                                     mask_clear, t.y & 0xffff, t.y >> 16, parity, early_load,
                                                     early_cold, blockIdx.x == 0, tid % kTileX, tid / kTileX);
     }
@@ -1124,7 +1144,7 @@ __global__ void __launch_bounds__(kTileX *kTileY)
 }  // namespace
 
 // ---------------------------------------------------------------- launchers
-static cudaLaunchConfig_t sweep_config(dim3 grid, dim3 block, int after_beads, cudaStream_t st,
+static cudaLaunchConfig_t sweep_config(dim3 grid, dim3 block, int dependent, cudaStream_t st,
                                        cudaLaunchAttribute *attr) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -1133,7 +1153,7 @@ static cudaLaunchConfig_t sweep_config(dim3 grid, dim3 block, int after_beads, c
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = after_beads ? 1 : 0;
+    cfg.numAttrs = dependent ? 1 : 0;
     return cfg;
 }
 
@@ -1161,11 +1181,16 @@ template <class S> static typename PhiArg<S>::type phi_arg(const PhiTab &p) {
     if constexpr (std::is_same<S, double>::value) return p;
     else return NoPhi{};
 }
+template <class S> static typename SweepArg<S>::type sweep_arg(const PhiTab &p, const Inst &I) {
+    if constexpr (std::is_same<S, double>::value)
+        return SweepF64{p, trt_rates(I.fluid_rates_d[0], I.fluid_rates_d[3])};
+    else return NoPhi{};
+}
 
 template <class S>
 static cudaError_t lattice_v(int variant, const Inst &I, void *pool, BeadTab tab, const PhiTab &phi,
                              const SweepMasks &mk, int parity, int after_beads, cudaStream_t st) {
-    const auto pt = phi_arg<S>(phi);
+    const auto pt = sweep_arg<S>(phi, I);
     cudaLaunchAttribute attr[1];
     const dim3 grid(I.ntx, I.nty);
     const int sp = row_split<S>(I.ntx * I.nty), rows = kTileY / sp;
@@ -1173,13 +1198,13 @@ static cudaError_t lattice_v(int variant, const Inst &I, void *pool, BeadTab tab
     const int ec = after_beads ? mk.early_cold : 0;
     // constant Lallemand-Luo rates: the moment form, one cell per thread
     if (I.collision == 1) {
-        const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX, rows), after_beads, st, attr);
+        const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX, rows), after_beads | mk.chained, st, attr);
         return cudaLaunchKernelEx(&cfg, sp > 1 ? k_lattice<S, 1, false, kCollMrt, true> : k_lattice<S, 1, false, kCollMrt>, I, (S *)pool, tab, mk.read, mk.prev,
                                   mk.clear, parity, after_beads, ec, pt);
     }
     if (variant == 2 && I.nx % VecWidth<S>::value == 0) {
-        const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX / VecWidth<S>::value, kTileY), after_beads,
-                                                    st, attr);
+        const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX / VecWidth<S>::value, kTileY),
+                                                    after_beads | mk.chained, st, attr);
         return cudaLaunchKernelEx(&cfg, k_lattice_vec<S>, I, (S *)pool, tab, mk.read, mk.prev, mk.clear,
                                   parity, after_beads, ec, pt);
     }
@@ -1193,11 +1218,11 @@ static cudaError_t lattice_v(int variant, const Inst &I, void *pool, BeadTab tab
         }
     }
     if (variant == 1 || variant == 3 || variant == 4) {
-        const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX / 2, rows), after_beads, st, attr);
+        const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX / 2, rows), after_beads | mk.chained, st, attr);
         return cudaLaunchKernelEx(&cfg, sp > 1 ? k_lattice<S, 2, true, kCollTrt, true> : k_lattice<S, 2, true, kCollTrt>, I, (S *)pool, tab, mk.read, mk.prev,
                                   mk.clear, parity, after_beads, ec, pt);
     }
-    const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX, rows), after_beads, st, attr);
+    const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX, rows), after_beads | mk.chained, st, attr);
     return cudaLaunchKernelEx(&cfg, sp > 1 ? k_lattice<S, 1, false, kCollTrt, true> : k_lattice<S, 1, false, kCollTrt>, I, (S *)pool, tab, mk.read, mk.prev,
                               mk.clear, parity, after_beads, ec, pt);
 }
