@@ -106,6 +106,7 @@ struct fpd_batch {
     unsigned *status = nullptr;  // sticky FPD_FLAG_* bits per slot (device)
     int64_t watch_next = fpd::kWatchSteps;  // global step of the next watchdog pass
     int2 *tiles_d = nullptr;
+    fpd::TileRec *recs_d = nullptr;  // FP32 and FP16 storage: the tiles' records
     int tiles_cap = 0, ntiles = 0;
     unsigned *masks = nullptr;  // kMaskBufs * tiles_cap * mask_words, in rotation by global step
     int4 *beads_all_d = nullptr, *beads_old_d = nullptr, *beads_fresh_d = nullptr;  // as launch_beads takes them
@@ -169,6 +170,7 @@ void free_batch(fpd_batch *b) {
     cudaFree(b->counters);
     cudaFree(b->status);
     cudaFree(b->tiles_d);
+    cudaFree(b->recs_d);
     cudaFree(b->masks);
     cudaFree(b->beads_all_d);
     cudaFree(b->beads_old_d);
@@ -260,11 +262,15 @@ int rebuild(fpd_batch *b) {
         if (sl.state == kActive && sl.inst.collision == 1) b->any_mrt = 1;
     if (b->ntiles > b->tiles_cap || !b->masks) {
         cudaFree(b->tiles_d);
+        cudaFree(b->recs_d);
         cudaFree(b->masks);
         b->tiles_d = nullptr;
+        b->recs_d = nullptr;
         b->masks = nullptr;
         const int cap = std::max(std::max(b->ntiles, 1), 2 * b->tiles_cap);
         if ((e = cudaMalloc(&b->tiles_d, cap * sizeof(int2))) != cudaSuccess) return bcuda(b, e, "cudaMalloc tiles");
+        if (b->precision != 0 && (e = cudaMalloc(&b->recs_d, cap * sizeof(fpd::TileRec))) != cudaSuccess)
+            return bcuda(b, e, "cudaMalloc tile records");
         if ((e = cudaMalloc(&b->masks, fpd::kMaskBufs * (size_t)cap * b->mask_words * sizeof(unsigned))) !=
             cudaSuccess)
             return bcuda(b, e, "cudaMalloc masks");
@@ -277,6 +283,8 @@ int rebuild(fpd_batch *b) {
     if ((e = cudaMemcpyAsync(b->insts_d, b->insts_h.data(), b->insts_h.size() * sizeof(fpd::Inst),
                              cudaMemcpyHostToDevice, b->stream)) != cudaSuccess)
         return bcuda(b, e, "copy instance records");
+    if (b->recs_d && (e = fpd::launch_tile_recs(b->insts_d, b->tiles_d, b->ntiles, b->recs_d, b->stream)) != cudaSuccess)
+        return bcuda(b, e, "tile records");
     if (b->tiles_cap > 0 &&
         (e = cudaMemsetAsync(b->masks, 0, fpd::kMaskBufs * (size_t)b->tiles_cap * b->mask_words * sizeof(unsigned),
                              b->stream)) !=
@@ -483,8 +491,8 @@ int enqueue_bstep(fpd_batch *b, cudaStream_t st, int64_t gstep, bool any_first) 
                               b->counters, 1, st, fpd::BeadExport{}, b->status);
         if (e != cudaSuccess) return bcuda(b, e, "batched bead phase");
     }
-    e = fpd::launch_lattice_batch(b->precision, b->insts_d, b->tiles_d, b->ntiles, b->pool, b->tab, b->phi, mk,
-                                  gp, nbl > 0 ? 1 : 0, b->variant, b->any_mrt, st);
+    e = fpd::launch_lattice_batch(b->precision, b->insts_d, b->tiles_d, b->ntiles, b->pool, b->tab, b->phi,
+                                  b->recs_d, b->mask_words, mk, gp, nbl > 0 ? 1 : 0, b->variant, b->any_mrt, st);
     if (e != cudaSuccess) return bcuda(b, e, "batched lattice sweep");
     return FPD_OK;
 }

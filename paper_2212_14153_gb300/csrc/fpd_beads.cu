@@ -850,20 +850,24 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             (lane ? tnew.yl : tnew.xl)[b] = (float)(v - (double)hi);
         }
         // mark bead b in the mask of every lattice tile its support box, widened
-        // by one cell, reaches: one atomicOr per tile row and tile column the
-        // box starts in; the widening covers the bead's move in the next step, so
-        // the next sweep may update unmarked tiles before its bead phase ends
+        // by one cell, reaches (the part before a periodic edge, then the part
+        // after it; a tile reached twice is marked twice); the widening covers
+        // the bead's move in the next step, so the next sweep may update
+        // unmarked tiles before its bead phase ends
         const Support wb = widen(I, bx);
-        const float inv_wb = inv_width(wb);
         const int lb = b - first;
         const unsigned bit = 1u << (lb & 31);
+        const int c0 = wb.lo[0] / kTileX, c1 = (min(wb.lo[0] + wb.n[0], I.nx) - 1) / kTileX;
+        const int r0 = wb.lo[1] / kTileY, r1 = (min(wb.lo[1] + wb.n[1], I.ny) - 1) / kTileY;
+        const int over_x = wb.lo[0] + wb.n[0] - I.nx, over_y = wb.lo[1] + wb.n[1] - I.ny;
+        const int nc = c1 - c0 + 1, cols = nc + (over_x > 0 ? (over_x - 1) / kTileX + 1 : 0);
+        const int nr = r1 - r0 + 1, rows = nr + (over_y > 0 ? (over_y - 1) / kTileY + 1 : 0);
+        const int marks = wb.n[0] > 0 && wb.n[1] > 0 ? rows * cols : 0;
 #pragma unroll 1
-        for (int t = tid - 32; t < wb.n[0] * wb.n[1]; t += NT - 32) {
-            int ci, cj, col, row;
-            cell_rc(wb, inv_wb, t, ci, cj);
-            cell_of(I, wb, ci, cj, col, row);
-            if ((cj != 0 && (row % kTileY) != 0) || (ci != 0 && (col % kTileX) != 0)) continue;
-            const int tile = I.tile_base + (row / kTileY) * I.ntx + col / kTileX;
+        for (int t = tid - 32; t < marks; t += NT - 32) {
+            const int tr = t / cols, tc = t - tr * cols;
+            const int row = tr < nr ? r0 + tr : tr - nr, col = tc < nc ? c0 + tc : tc - nc;
+            const int tile = I.tile_base + row * I.ntx + col;
             atomicOr(mask_write + tile * I.mask_words + (lb >> 5), bit);
         }
     }

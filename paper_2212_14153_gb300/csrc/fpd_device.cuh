@@ -83,6 +83,23 @@ struct Inst {
     float trt_sw[3], trt_k45[3], trt_k3[3];
 };
 
+// One tile of a batch's sweep (FP32 and FP16 storage) with what its update
+// needs of the instance's record while no bead marks it.
+struct alignas(16) TileRec {
+    // where its populations are (one 16-byte load prefetches a tile):
+    int64_t tile;          // element offset of its first cell in buffer 0
+    int32_t buffer;        // elements of one buffer (9 planes)
+    int32_t rows_par;      // rows of the tile in the lattice << 1 | par_xor
+    int32_t at, nx, ny, strip;  // tile (by << 16 | bx), lattice, elements of a strip
+    int32_t slot;
+    int32_t plain;         // magic or BGK rates, no body force, no sandwich layers
+    int32_t periodic_y;
+    float s_nu, s_q;       // the fluid's rates
+    float wall_b, wall_t;  // bounce-back terms (stored units) of k = 5 (bottom), k = 8 (top); k = 6, 7 minus that
+    int32_t pad_;
+};
+static_assert(sizeof(TileRec) == 64, "four 16-byte loads");
+
 // Element offset of column x (>= 0) within its row of plane 0.
 static_assert(kStripW == 32, "col_off, strip_left and strip_right shift by 5");
 __device__ __forceinline__ int col_off(const Inst &I, int x) { return (x >> 5) * I.strip + (x & 31); }
@@ -161,6 +178,17 @@ template <> struct Store<double> {
     static __device__ __forceinline__ double ld_stream(const double *p, uint64_t) { return *p; }
     static __device__ __forceinline__ void st_stream(double *p, double v, uint64_t) { *p = v; }
 };
+// Read-only 16 bytes kept in L2 before other lines (a batch streams many
+// times the L2 every step; its tile records are read once a step).
+__device__ __forceinline__ int4 ld_keep(const int4 *p) {
+    uint64_t pol;
+    asm("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(pol));
+    int4 v;
+    asm volatile("ld.global.L2::cache_hint.v4.s32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(p), "l"(pol));
+    return v;
+}
 // L2 eviction priority of the population stream of a single-lattice sweep
 // (createpolicy, applied per access through .L2::cache_hint).  Each element
 // is read once and written once per step and one sweep moves more than the
@@ -796,7 +824,7 @@ __device__ __forceinline__ void collide_trt(V x[9], V sp, V sm, const Inst &I) {
 // sweep): rho (c.u)^2 is formed as (c.j)(c.u), so the quadratic terms of all
 // four pairs come from jx ux, jy uy and jx uy, and every product with a rate
 // is one of these constants.  57 FP64 instructions a cell instead of about 80
-// (4096 x 1024 without beads: 571 -> 453 us).
+// (4096 x 1024 without beads: 571 -> 473 us).
 struct TrtRates {
     double m0, c1, c2;      // 1 - sp, (1 - sp) / 2, (1 - sm) / 2
     double k0, k1, k3;      // sp w of the rest, axis and diagonal links

@@ -142,9 +142,12 @@ cudaError_t launch_watch(int precision, const Inst *insts, const Inst &inst_h, c
 // any_mrt = 1 when some instance uses constant Lallemand-Luo rates
 // (collision 1): the sweep then runs variant 0 with both collision forms.
 // A single instance with collision 1 runs variant 0 as well.
+// recs: the tiles' records (FP32 and FP16 storage; launch_tile_recs), mask_words: words per
+// tile mask.
+cudaError_t launch_tile_recs(const Inst *insts, const int2 *tiles, int ntiles, TileRec *recs, cudaStream_t st);
 cudaError_t launch_lattice_batch(int precision, const Inst *insts, const int2 *tiles, int ntiles, void *pool,
-                                 const BeadTab tab[2], const PhiTab phi[2], const SweepMasks &masks, int gparity,
-                                 int after_beads,
+                                 const BeadTab tab[2], const PhiTab phi[2], const TileRec *recs, int mask_words,
+                                 const SweepMasks &masks, int gparity, int after_beads,
                                  int variant, int any_mrt, cudaStream_t st);
 
 cudaError_t launch_init(int precision, const Inst *inst_d, const Inst &inst_h, void *pool, int couette,

@@ -657,14 +657,135 @@ template <class S, int CY, bool kAlongX> struct BatchInner {
     static constexpr bool value = (CY == 1 || kAlongX) && !std::is_same<S, double>::value;
 };
 
+// A batch's sweep in FP32 or FP16 storage reads a tile record first (TileRec)
+// and updates a tile that no bead marked, of an instance without body force or
+// sandwich layers, from it: no copy of the instance's record to shared memory,
+// no barrier.  The sweep is bound by memory latency (ncu, 128 instances:
+// long-scoreboard stalls first, DRAM at 63 %, the same with 20 % fewer
+// instructions), so
+// - each CTA has the populations of the tile kAhead CTAs on brought to L2 by
+//   one bulk prefetch (a tile's rows are contiguous in its strip): with that
+//   the bytes in flight do not depend on registers.  kAhead is one wave of
+//   resident CTAs; 512 instances, us a step, at 304, 760, 1216, 1672, 2128 and
+//   3648 CTAs ahead: 376, 363, 363, 367, 378, 456; none: 392.  After the
+//   tile's own loads instead (it then spills): 373;
+// - records are kept in L2 (ld_keep) and prefetched two such distances ahead,
+//   masks with them: 409 -> 392 us a step.
+// The same pulls and the same one-cell update as lattice_tile's, so the same
+// bits.  A warp owns one row of the tile, so that rows next to a wall or a
+// periodic edge branch off as a whole.
+constexpr unsigned kAhead = 1216;
+__device__ __forceinline__ TileRec tile_rec(const TileRec *__restrict__ recs) {
+    TileRec r;
+    const int4 *q = reinterpret_cast<const int4 *>(recs);
+    int4 *d = reinterpret_cast<int4 *>(&r);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) d[i] = ld_keep(q + i);
+    return r;
+}
+// By one thread of the CTA.
+template <class S>
+__device__ __forceinline__ void prefetch_tiles(const S *__restrict__ pool, const TileRec *__restrict__ recs,
+                                               const unsigned *__restrict__ mask_prev, const int mask_words,
+                                               const int gparity) {
+    const unsigned far = blockIdx.x + 4 * kAhead, next = blockIdx.x + kAhead;
+    if (far < gridDim.x) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(recs + far));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(mask_prev + (size_t)far * mask_words));
+    }
+    if (next < gridDim.x) {
+        const int4 q = ld_keep(reinterpret_cast<const int4 *>(recs + next));
+        const int64_t tile = (int64_t)(unsigned)q.x | (int64_t)q.y << 32;
+        const S *p = pool + tile + (((gparity ^ q.w) & 1) ? q.z : 0);
+        // 16-byte aligned, a multiple of 16 bytes: planes start at 256 bytes, rows hold 9 * 32 elements
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"((q.w >> 1) * kRowStride * (int)sizeof(S)));
+    }
+}
+template <int k, class S>
+__device__ __forceinline__ void pull_rec_one(const S *__restrict__ p, int shl, int shr, int dn, int up, bool bot,
+                                             bool top, float wb, float wt, float g[9]) {
+    constexpr int cx = Q<k>::cx, cy = Q<k>::cy;
+    if ((cy > 0 && bot) || (cy < 0 && top)) {
+        g[k] = Store<S>::ld_raw(p + Q<k>::opp * kPlaneStride) + (cy > 0 ? (float)cx * wb : (float)cx * wt);
+    } else {
+        const int off = PullOff<k>::value + (cx > 0 ? shl : (cx < 0 ? shr : 0)) + (cy > 0 ? dn : (cy < 0 ? up : 0));
+        g[k] = Store<S>::ld_raw(p + off);
+    }
+}
+template <class S>
+__device__ __forceinline__ void tile_from_rec(const TileRec &r, S *__restrict__ pool, const Inst *__restrict__ insts,
+                                              const int gparity) {
+    const int tx = threadIdx.x, x = (r.at & 0xffff) * kTileX + tx, y = (r.at >> 16) * kTileY + threadIdx.y;
+    if (x >= r.nx || y >= r.ny) return;
+    const Inst &I = insts[r.slot];  // read by FP16 storage only (its scales)
+    const int parity = (gparity ^ r.rows_par) & 1;
+    const int cx = (x >> 5) * r.strip + tx, last = ((r.nx - 1) >> 5) * r.strip + ((r.nx - 1) & 31);
+    const int shl = x == 0 ? last + 1 : (tx == 0 ? kStripW - r.strip : 0);
+    const int shr = x == r.nx - 1 ? -cx - 1 : (tx == 31 ? r.strip - kStripW : 0);
+    S *const base = pool + r.tile + ((int)threadIdx.y * kRowStride + tx);
+    const S *const p = base + (parity ? r.buffer : 0);
+    float g[9];
+    if (y > 0 && y < r.ny - 1) {
+        pull_inner<S, float, true, false>(p, shl, shr, I, g);
+    } else {
+        const bool b0 = y == 0, bn = y == r.ny - 1, bot = b0 && !r.periodic_y, top = bn && !r.periodic_y;
+        const int dn = b0 ? r.ny * kRowStride : 0, up = bn ? -r.ny * kRowStride : 0;
+        pull_rec_one<0>(p, shl, shr, dn, up, bot, top, r.wall_b, r.wall_t, g);
+        pull_rec_one<1>(p, shl, shr, dn, up, bot, top, r.wall_b, r.wall_t, g);
+        pull_rec_one<2>(p, shl, shr, dn, up, bot, top, r.wall_b, r.wall_t, g);
+        pull_rec_one<3>(p, shl, shr, dn, up, bot, top, r.wall_b, r.wall_t, g);
+        pull_rec_one<4>(p, shl, shr, dn, up, bot, top, r.wall_b, r.wall_t, g);
+        pull_rec_one<5>(p, shl, shr, dn, up, bot, top, r.wall_b, r.wall_t, g);
+        pull_rec_one<6>(p, shl, shr, dn, up, bot, top, r.wall_b, r.wall_t, g);
+        pull_rec_one<7>(p, shl, shr, dn, up, bot, top, r.wall_b, r.wall_t, g);
+        pull_rec_one<8>(p, shl, shr, dn, up, bot, top, r.wall_b, r.wall_t, g);
+    }
+    collide_trt<float, Store<S>::kScaled>(g, r.s_nu, r.s_q, I);
+    put_at<S, float, true, false>(base + (parity ? 0 : r.buffer), I, g);
+}
+__global__ void k_tile_recs(const Inst *__restrict__ insts, const int2 *__restrict__ tiles, int ntiles,
+                            TileRec *__restrict__ recs) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= ntiles) return;
+    const Inst &I = insts[tiles[t].x];
+    TileRec r{};
+    const int bx = tiles[t].y & 0xffff, y0 = (tiles[t].y >> 16) * kTileY;
+    r.tile = I.pop_off + (y0 * kRowStride + bx * I.strip);
+    r.rows_par = min(kTileY, I.ny - y0) << 1 | I.par_xor;
+    r.buffer = (int)(9 * I.plane);
+    r.strip = I.strip;
+    r.nx = I.nx;
+    r.ny = I.ny;
+    r.at = tiles[t].y;
+    r.slot = tiles[t].x;
+    r.plain = I.collision != 1 && !I.sandwich && !body_forced<float>(I);
+    r.periodic_y = I.periodic_y;
+    r.s_nu = I.fluid_rates_f[0];
+    r.s_q = I.fluid_rates_f[3];
+    r.wall_b = I.bbs[0][5];
+    r.wall_t = I.bbs[1][8];
+    recs[t] = r;
+}
+
 template <class S, int CY, bool kAlongX, int kColl>
 __global__ void __launch_bounds__(kTileX *kTileY / CY, BatchMinBlocks<S, CY>::value)
     k_lattice_batch(const Inst *__restrict__ insts, const int2 *__restrict__ tiles, S *__restrict__ pool,
                     const BeadTab tab0, const BeadTab tab1, const unsigned *__restrict__ mask_read,
                     const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear, const int gparity,
                     const int early_load, const int early_cold, const typename PhiArg<S>::type phi0,
-                    const typename PhiArg<S>::type phi1) {
+                    const typename PhiArg<S>::type phi1, const TileRec *__restrict__ recs, const int mask_words) {
     __shared__ Inst sI;
+    if constexpr (CY == 1 && !std::is_same<S, double>::value) {
+        const TileRec r = tile_rec(recs + blockIdx.x);
+        if (threadIdx.x == 0 && threadIdx.y == kTileY - 1) prefetch_tiles<S>(pool, recs, mask_prev, mask_words, gparity);
+        if (r.plain && tile_cold_early(mask_prev + blockIdx.x * mask_words, mask_words, early_cold, blockIdx.x == 0)) {
+            pdl_trigger();
+            if (threadIdx.x == 0 && threadIdx.y == 0)
+                for (int w = 0; w < mask_words; ++w) mask_clear[blockIdx.x * mask_words + w] = 0u;
+            tile_from_rec<S>(r, pool, insts, gparity);
+            return;
+        }
+    }
     const int2 t = tiles[blockIdx.x];
     {
         const unsigned *src = (const unsigned *)(insts + t.x);
@@ -1253,10 +1374,16 @@ cudaError_t launch_lattice(int precision, const Inst *, const Inst &inst_h, void
     return cudaErrorInvalidValue;
 }
 
+cudaError_t launch_tile_recs(const Inst *insts, const int2 *tiles, int ntiles, TileRec *recs, cudaStream_t st) {
+    if (ntiles <= 0) return cudaSuccess;
+    k_tile_recs<<<(ntiles + 255) / 256, 256, 0, st>>>(insts, tiles, ntiles, recs);
+    return cudaGetLastError();
+}
+
 template <class S>
 static cudaError_t lattice_batch_v(int variant, const Inst *insts, const int2 *tiles, int ntiles, void *pool,
-                                   const BeadTab tab[2], const PhiTab phi[2], const SweepMasks &mk, int gparity,
-                                   int after_beads, int any_mrt, cudaStream_t st) {
+                                   const BeadTab tab[2], const PhiTab phi[2], const TileRec *recs, int mask_words,
+                                   const SweepMasks &mk, int gparity, int after_beads, int any_mrt, cudaStream_t st) {
     const BeadTab &tab0 = tab[0], &tab1 = tab[1];
     const auto phi0 = phi_arg<S>(phi[0]), phi1 = phi_arg<S>(phi[1]);
     cudaLaunchAttribute attr[1];
@@ -1267,7 +1394,7 @@ static cudaError_t lattice_batch_v(int variant, const Inst *insts, const int2 *t
     if (any_mrt) {
         const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX, kTileY), after_beads, st, attr);
         return cudaLaunchKernelEx(&cfg, k_lattice_batch<S, 1, false, kCollAny>, insts, tiles, (S *)pool, tab0, tab1,
-                                  mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1);
+                                  mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1, recs, mask_words);
     }
     if (variant == 2) {
         const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX / VecWidth<S>::value, kTileY), after_beads,
@@ -1278,21 +1405,21 @@ static cudaError_t lattice_batch_v(int variant, const Inst *insts, const int2 *t
     if (variant == 1 || variant == 3 || variant == 4) {  // the staged blocks are single-lattice only
         const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX / 2, kTileY), after_beads, st, attr);
         return cudaLaunchKernelEx(&cfg, k_lattice_batch<S, 2, true, kCollTrt>, insts, tiles, (S *)pool, tab0, tab1,
-                                  mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1);
+                                  mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1, recs, mask_words);
     }
     const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX, kTileY), after_beads, st, attr);
     return cudaLaunchKernelEx(&cfg, k_lattice_batch<S, 1, false, kCollTrt>, insts, tiles, (S *)pool, tab0, tab1,
-                              mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1);
+                              mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1, recs, mask_words);
 }
 
 cudaError_t launch_lattice_batch(int precision, const Inst *insts, const int2 *tiles, int ntiles, void *pool,
-                                 const BeadTab tab[2], const PhiTab phi[2], const SweepMasks &masks, int gparity,
-                                 int after_beads, int variant, int any_mrt, cudaStream_t st) {
+                                 const BeadTab tab[2], const PhiTab phi[2], const TileRec *recs, int mask_words,
+                                 const SweepMasks &masks, int gparity, int after_beads, int variant, int any_mrt, cudaStream_t st) {
     if (ntiles <= 0) return cudaSuccess;
     switch (precision) {
-        case 0: return lattice_batch_v<double>(variant, insts, tiles, ntiles, pool, tab, phi, masks, gparity, after_beads, any_mrt, st);
-        case 1: return lattice_batch_v<float>(variant, insts, tiles, ntiles, pool, tab, phi, masks, gparity, after_beads, any_mrt, st);
-        case 2: return lattice_batch_v<__half>(variant, insts, tiles, ntiles, pool, tab, phi, masks, gparity, after_beads, any_mrt, st);
+        case 0: return lattice_batch_v<double>(variant, insts, tiles, ntiles, pool, tab, phi, recs, mask_words, masks, gparity, after_beads, any_mrt, st);
+        case 1: return lattice_batch_v<float>(variant, insts, tiles, ntiles, pool, tab, phi, recs, mask_words, masks, gparity, after_beads, any_mrt, st);
+        case 2: return lattice_batch_v<__half>(variant, insts, tiles, ntiles, pool, tab, phi, recs, mask_words, masks, gparity, after_beads, any_mrt, st);
     }
     return cudaErrorInvalidValue;
 }

@@ -283,3 +283,28 @@ def test_periodic_driven_instances_in_a_batch(fpd):
         for c, s in zip(mixed, slots):
             _same((b.populations(s), b.beads(s)), _alone(fpd, c, 120))
         b.close()
+
+
+@pytest.mark.parametrize("precision", [1, 2])
+def test_batch_tiles_updated_from_their_records_equal_alone(fpd, precision):
+    # unmarked tiles of a batch are updated from tile records: rows at walls
+    # and at both periodic edges, ragged widths and heights, one column of
+    # tiles, body force and sandwich layers (which take the general path), and
+    # enough tiles that each CTA prefetches another one's populations
+    rng = np.random.default_rng(60 + precision)
+    cases = [
+        wl.random_fiber(rng, 45, 9000, n_beads=3, a=2.0, xi=0.5, precision=precision),
+        wl.random_fiber(rng, 31, 7, n_beads=1, a=1.0, xi=0.25, precision=precision, periodic_y=1, bead_fx=0.01),
+        wl.random_fiber(rng, 96, 41, n_beads=4, a=2.0, xi=0.5, precision=precision, periodic_y=1),
+        wl.couette_only(33, 8, u=0.01, nu=0.2, init_couette=0, precision=precision),
+        dict(wl.couette_only(64, 24, u=0.01, nu=0.2, precision=precision), gx=1e-5),
+        dict(wl.couette_only(50, 40, u=0.01, nu=0.1, precision=precision), sandwich_zl=8.0, sandwich_zr=32.0),
+        dict(wl.couette_only(1, 5, u=0.01, nu=0.2, precision=precision), collision=2),
+    ]
+    b = fpd.Batch(precision, len(cases), 256 << 20, 64)
+    slots = [b.add(c, 40) for c in cases]
+    while b.run(1000):
+        pass
+    for c, s in zip(cases, slots):
+        _same((b.populations(s), b.beads(s)), _alone(fpd, c, 40))
+    b.close()
