@@ -224,6 +224,59 @@ __device__ __forceinline__ float min_image_yf(const Inst &I, float d) {
     return I.periodic_y ? d - (float)I.ny * rintf(d * I.f_inv_ny) : d;
 }
 
+// A double as a pair of floats, h + l equal to it within 2^-48 of its size,
+// from its bits: the conversions and subtractions are FP64 instructions, a
+// chain of which took the last CTA about a microsecond.  Sizes outside
+// [2^-74, 2^127) do not occur for positions in use: 0 below, NaN above.
+__device__ __forceinline__ float2 split(double x) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const int e = (int)(u >> 52) & 0x7ff;
+    const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
+    if (e < 949) return make_float2(0.f, 0.f);
+    if (e >= 1150) return make_float2(__int_as_float(0x7fc00000), 0.f);
+    const float h = __uint_as_float(sign | (unsigned)(e - 896) << 23 | ((unsigned)(u >> 29) & 0x7fffffu));
+    const float l = (float)((unsigned)u & 0x1fffffffu) * __uint_as_float(sign | (unsigned)(e - 948) << 23);
+    return make_float2(h, l);
+}
+// Error-free sum (Knuth): s + e == a + b exactly.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+    s = __fadd_rn(a, b);
+    const float bb = __fsub_rn(s, a);
+    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+// (a + a')^2 as p + e, a' the low part of a
+__device__ __forceinline__ void square2(float a, float al, float &p, float &e) {
+    p = __fmul_rn(a, a);
+    e = __fmaf_rn(2.0f * a, al, __fmaf_rn(a, a, -p));
+}
+
+// Length, tangent component and stretch of the segment from A to B on this
+// thread's axis; the other axis' thread is the lane next to it (xor 1).
+__device__ __forceinline__ void segment_axis(const Inst &I, double A, double B, double &L, double &t, double &str) {
+    const double d = B - A, d2 = d * d;
+    L = sqrt(d2 + __shfl_xor_sync(0xffffffffu, d2, 1));
+    t = d * (1.0 / L);
+    str = L - I.l0;
+}
+// FP32 paths: differences and squares in pairs of floats (2^-46), as the
+// stretch L - l0 = (|d|^2 - l0^2) / (L + l0) of a stiff spring is small
+// against them and must not cancel away.
+__device__ __forceinline__ void segment_axis(const Inst &I, float2 A, float2 B, float &L, float &t, float &str) {
+    float dh, dl, p, pe, s, se, q, qe;
+    two_sum(B.x, -A.x, dh, dl);
+    dl += B.y - A.y;
+    const float d = dh + dl;
+    dl -= d - dh;
+    square2(d, dl, p, pe);
+    two_sum(p, __shfl_xor_sync(0xffffffffu, p, 1), s, se);
+    se += pe + __shfl_xor_sync(0xffffffffu, pe, 1);
+    const float2 l0 = split(I.l0);
+    square2(l0.x, l0.y, q, qe);
+    L = sqrtf(s + se);
+    t = d / L;
+    str = ((s - q) + (se - qe)) / (L + I.f_l0);
+}
+
 // Excluded-volume candidates of every bead of the instance into cand: beads
 // that share no spring with it, nearer than l0 by an FP32 distance test with
 // 1% margin.  Xf, Yf: positions relative to bead 0 of the instance.  Warp w
@@ -252,17 +305,18 @@ __device__ __forceinline__ void screen_close(const Inst &I, const float *Xf, con
     }
 }
 
+__device__ __forceinline__ double place(double r) { return r; }
+__device__ __forceinline__ double place(float2 r) { return (double)r.x + (double)r.y; }
 // Excluded volume on bead q along axis ax (0 x, 1 y) from the beads in its
-// candidate words, in bead order; r: interleaved x, y positions.
-template <class R>
-__device__ __forceinline__ R close_force(const Inst &I, const double *r, const unsigned *cand, int q, int ax) {
-    const int nw = (I.nb + 31) / 32;
+// nw candidate words, in bead order; r: interleaved x, y positions.
+template <class R, class Place>
+__device__ __forceinline__ R close_force(const Inst &I, const Place *r, const unsigned *cand, int nw, int q, int ax) {
     R f = (R)0;
     for (int c = 0; c < nw; ++c)
-        for (unsigned bits = cand[q * nw + c]; bits; bits &= bits - 1u) {
+        for (unsigned bits = cand[c]; bits; bits &= bits - 1u) {
             const int p = 32 * c + __ffs(bits) - 1;
-            const double dx = min_image(r[2 * q] - r[2 * p], I.nx, I.f_inv_nx);
-            const double dy = min_image_y(I, r[2 * q + 1] - r[2 * p + 1]);
+            const double dx = min_image(place(r[2 * q]) - place(r[2 * p]), I.nx, I.f_inv_nx);
+            const double dy = min_image_y(I, place(r[2 * q + 1]) - place(r[2 * p + 1]));
             if constexpr (std::is_same<R, double>::value) {
                 const double d = sqrt(dx * dx + dy * dy);
                 if (d < I.l0 && d > 0.0) f += I.k_ev * (I.l0 - d) / d * (ax ? dy : dx);
@@ -292,15 +346,18 @@ template <class R> struct alignas(4 * sizeof(R)) Neighbour {
     R x, y, gx, gy;
 };
 // Box cells listed at a time (a support box of the usual beads fits at once:
-// 29 x 29 cells for a = 4, xi = 1).
-template <class R> struct ListCap { static constexpr int value = std::is_same<R, double>::value ? 1024 : 1280; };
+// 29 x 29 cells for a = 4, xi = 1; with a CTA to an SM 45 x 45).
+template <class R, int NT> struct ListCap {
+    static constexpr int value = std::is_same<R, double>::value ? 1000 : NT >= 512 ? 2048 : 1280;
+};
 
 // The last CTA's view of its instance, in the shared memory the list took;
 // x and y of a bead or segment side by side.
 template <class R> struct ForceShared {
-    double r[2 * kMaxBeads], S[kMaxBeads];
+    using Place = typename std::conditional<std::is_same<R, double>::value, double, float2>::type;  // FP32 paths: split
+    Place r[2 * kMaxBeads];
+    R S[kMaxBeads], t[2 * kMaxBeads], pull[2 * kMaxBeads], len[kMaxBeads], str[kMaxBeads];
     float xf[kMaxBeads], yf[kMaxBeads];
-    R t[2 * kMaxBeads], pull[2 * kMaxBeads], len[kMaxBeads], str[kMaxBeads];
     unsigned cand[kMaxBeads * (kMaxBeads / 32)];
 };
 
@@ -409,8 +466,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     using F = Fix<R>;
     using T = typename F::T;
     constexpr int NW = NT / 32;
-    constexpr int kCap = ListCap<R>::value;
-    constexpr int kPer = kCap / NT > 3 ? 3 : (kCap + NT - 1) / NT;  // box cells a thread lists at a time
+    constexpr int kCap = ListCap<R, NT>::value;
+    constexpr int kPer = NT >= 512 ? 2 : 3;  // box cells a thread lists at a time
     constexpr size_t kBuf = sizeof(SupportCell<R>) * kCap > sizeof(ForceShared<R>) ? sizeof(SupportCell<R>) * kCap
                                                                                    : sizeof(ForceShared<R>);
     __shared__ Inst sI;
@@ -882,13 +939,15 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     const unsigned st_now = (status && advance) ? __ldcg(status + ii) : 0u;
     // The instance's new positions and support sums (written by every CTA;
     // the L2-coherent loads see them), then every segment, then every bead;
-    // a thread works on one axis (ax) of item q: FP64 instructions cost a
-    // warp 64 cycles each whatever its lanes do, so x and y share them
+    // a thread works on one axis (ax) of item q (FP64 instructions cost a
+    // warp 64 cycles each whatever its lanes do, so x and y share them)
     const int items = 2 * nb, N = I.n_beads;
     const float inv_n = 1.0f / (float)N;
     for (int k = tid; k < items; k += NT) {
-        fs.r[k] = nb == 1 ? s_R[k] : __ldcg(((k & 1) ? tnew.Ry : tnew.Rx) + first + (k >> 1));
-        if (!(k & 1)) fs.S[k >> 1] = nb == 1 ? s_S : __ldcg(tnew.S + first + (k >> 1));
+        const double x = nb == 1 ? s_R[k] : __ldcg(((k & 1) ? tnew.Ry : tnew.Rx) + first + (k >> 1));
+        if constexpr (kF64) fs.r[k] = x;
+        else fs.r[k] = split(x);
+        if (!(k & 1)) fs.S[k >> 1] = (R)(nb == 1 ? s_S : __ldcg(tnew.S + first + (k >> 1)));
     }
     __syncthreads();
     // fast-bead guard: the early update of unmarked tiles assumes a bead
@@ -904,21 +963,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     for (int k0 = 0; k0 < items; k0 += NT) {
         const int k = k0 + tid, q = k >> 1;
         const bool seg = k < items && in_fiber(q) < N - 1;
-        const double d = seg ? fs.r[k + 2] - fs.r[k] : 1.0;
-        const double d2 = d * d, s = d2 + __shfl_xor_sync(0xffffffffu, d2, 1);
         R L, t, str;
-        if constexpr (kF64) {
-            L = sqrt(s);
-            t = d * (1.0 / L);
-            str = L - I.l0;
-        } else {
-            // positions stay FP64; the stretch L - l0 = (|d|^2 - l0^2) /
-            // (L + l0) is formed from the FP64 |d|^2 so that the small strain
-            // of a stiff spring does not cancel away in FP32
-            L = sqrtf((float)s);
-            t = (float)d / L;
-            str = (float)(s - I.l0 * I.l0) / (L + I.f_l0);
-        }
+        segment_axis(I, fs.r[seg ? k : 0], fs.r[seg ? k + 2 : 1], L, t, str);
         if (seg) {
             fs.t[k] = t;
             if (!(k & 1)) {
@@ -929,8 +975,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     }
     if (crowd) {
         for (int q = tid; q < nb; q += NT) {
-            fs.xf[q] = (float)(fs.r[2 * q] - fs.r[0]);
-            fs.yf[q] = (float)(fs.r[2 * q + 1] - fs.r[1]);
+            fs.xf[q] = (float)(place(fs.r[2 * q]) - place(fs.r[0]));
+            fs.yf[q] = (float)(place(fs.r[2 * q + 1]) - place(fs.r[1]));
         }
         __syncthreads();
         screen_close<NW>(I, fs.xf, fs.yf, fs.cand);
@@ -960,23 +1006,22 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         R f = (R)0;
         if (i0 > 0) f -= fs.pull[k - 2];
         if (i0 < N - 1) f += fs.pull[k];
-        if (crowd) f += close_force<R>(I, fs.r, fs.cand, q, ax);
+        if (crowd) f += close_force<R>(I, fs.r, fs.cand + q * ((nb + 31) / 32), (nb + 31) / 32, q, ax);
         // constant external force F_0 (driven particle, Sec. 3.2)
         if constexpr (kF64) f += ax ? I.ext_fy : I.ext_fx;
         else f += ax ? I.f_ext_fy : I.f_ext_fx;
         R g;
-        if constexpr (kF64) g = f * (1.0 / fs.S[q]);
-        else g = f * (1.0f / (float)fs.S[q]);
+        g = f * ((R)1 / fs.S[q]);
         (ax ? tnew.gyf : tnew.gxf)[gq] = (float)g;
         (ax ? tnew.Gy : tnew.Gx)[gq] = g;
         (ax ? tnew.Fy : tnew.Fx)[gq] = f;
         if (ex.ring) {
             // export: R, V, F, S of bead q into the ring slot of this phase
             double *d = ex.ring + (size_t)(ex_k % (unsigned long long)ex.slots) * ex.stride + kExportHeader;
-            d[ax * nb + q] = fs.r[k];
+            d[ax * nb + q] = __ldcg((ax ? tnew.Ry : tnew.Rx) + gq);
             d[(2 + ax) * nb + q] = __ldcg((ax ? tnew.Vy : tnew.Vx) + gq);
             d[(4 + ax) * nb + q] = f;
-            if (!ax) d[6 * nb + q] = fs.S[q];
+            if (!ax) d[6 * nb + q] = __ldcg(tnew.S + gq);
         }
     }
     if (ex.ring) {
