@@ -111,6 +111,7 @@ struct fpd_batch {
     unsigned *masks = nullptr;  // kMaskBufs * tiles_cap * mask_words, in rotation by global step
     int4 *beads_all_d = nullptr, *beads_old_d = nullptr, *beads_fresh_d = nullptr;  // as launch_beads takes them
     int n_all = 0, n_old = 0, n_fresh = 0;
+    int each = 0;  // beads of every resident instance that has any (0: not all the same)
     std::vector<Slot> slots;
     std::vector<fpd::Inst> insts_h;
     int64_t gstep = 0;
@@ -257,6 +258,14 @@ int rebuild(fpd_batch *b) {
         b->insts_h[s] = I;
     }
     b->ntiles = (int)tiles.size();
+    b->each = 0;
+    bool uneven = false;
+    for (auto &sl : b->slots)
+        if (sl.state == kActive && sl.inst.nb > 0) {
+            uneven |= b->each != 0 && b->each != sl.inst.nb;
+            b->each = sl.inst.nb;
+        }
+    if (uneven) b->each = 0;
     b->any_mrt = 0;
     for (auto &sl : b->slots)
         if (sl.state == kActive && sl.inst.collision == 1) b->any_mrt = 1;
@@ -323,7 +332,7 @@ int rebuild(fpd_batch *b) {
     }
     // initial bead tables of new instances (local parity 0 -> table 0)
     if (b->n_fresh > 0) {
-        e = fpd::launch_beads(b->precision, b->insts_d, b->beads_fresh_d, b->n_fresh, b->ntiles, b->pool, b->tab, b->phi,
+        e = fpd::launch_beads(b->precision, b->insts_d, b->beads_fresh_d, b->n_fresh, 0, b->ntiles, b->pool, b->tab, b->phi,
                               b->masks + (size_t)(b->gstep % fpd::kMaskBufs) * b->tiles_cap * b->mask_words, gp, 0,
                               b->counters, 0, b->stream);
         if (e != cudaSuccess) return bcuda(b, e, "initial bead tables");
@@ -386,6 +395,7 @@ int fpd_batch_create(int32_t precision, int32_t max_slots, int64_t pool_bytes, i
                                  d + 5 * nbm, d + 6 * nbm, d + 7 * nbm, d + 8 * nbm, f,
                                  f + nbm,     f + 2 * nbm, f + 3 * nbm, f + 4 * nbm, f + 5 * nbm};
     }
+    fpd::prepare_bead_kernels();
     if ((e = cudaStreamSynchronize(b->stream)) != cudaSuccess) {
         free_batch(b);
         delete b;
@@ -487,7 +497,7 @@ int enqueue_bstep(fpd_batch *b, cudaStream_t st, int64_t gstep, bool any_first) 
                              b->masks + (size_t)((gstep + 1) % M) * mstride, gstep > b->rebuild_gstep ? 1 : 0};
     cudaError_t e;
     if (nbl > 0) {
-        e = fpd::launch_beads(b->precision, b->insts_d, blist, nbl, b->ntiles, b->pool, b->tab, b->phi, mw, gp, 1,
+        e = fpd::launch_beads(b->precision, b->insts_d, blist, nbl, b->each, b->ntiles, b->pool, b->tab, b->phi, mw, gp, 1,
                               b->counters, 1, st, fpd::BeadExport{}, b->status);
         if (e != cudaSuccess) return bcuda(b, e, "batched bead phase");
     }

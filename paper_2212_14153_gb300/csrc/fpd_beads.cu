@@ -277,6 +277,19 @@ __device__ __forceinline__ void segment_axis(const Inst &I, float2 A, float2 B, 
     str = ((s - q) + (se - qe)) / (L + I.f_l0);
 }
 
+// What a segment pulls its first bead with along one axis (and its second the
+// other way): Eq. 11's spring, and Eq. 12's bending, k_b (t_{q+1} + t_{q-1}).
+// (I - t_q t_q) / L with the tangents of missing segments zero (v their sum,
+// vt = v.t).  Every rounding spelled out: two kernels share it.
+__device__ __forceinline__ double segment_pull(const Inst &I, double v, double vt, double t, double str, double L) {
+    const double bend = __ddiv_rn(__dmul_rn(I.k_b, __fma_rn(-vt, t, v)), L);
+    return __fma_rn(__dmul_rn(I.ks_l02, str), t, -bend);
+}
+__device__ __forceinline__ float segment_pull(const Inst &I, float v, float vt, float t, float str, float L) {
+    const float bend = __fdiv_rn(__fmul_rn(I.f_kb, __fmaf_rn(-vt, t, v)), L);
+    return __fmaf_rn(__fmul_rn(I.f_ks_l02, str), t, -bend);
+}
+
 // Excluded-volume candidates of every bead of the instance into cand: beads
 // that share no spring with it, nearer than l0 by an FP32 distance test with
 // 1% margin.  Xf, Yf: positions relative to bead 0 of the instance.  Warp w
@@ -307,10 +320,20 @@ __device__ __forceinline__ void screen_close(const Inst &I, const float *Xf, con
 
 __device__ __forceinline__ double place(double r) { return r; }
 __device__ __forceinline__ double place(float2 r) { return (double)r.x + (double)r.y; }
+// The same for bead q of at most 32, lane p holding bead p's place.
+__device__ __forceinline__ unsigned close_beads(const Inst &I, float x, float y, int q) {
+    const int N = I.n_beads, p = threadIdx.x & 31, lo = q / N * N;
+    float fx = __shfl_sync(0xffffffffu, x, q) - x;
+    fx -= (float)I.nx * rintf(fx * I.f_inv_nx);
+    const float fy = min_image_yf(I, __shfl_sync(0xffffffffu, y, q) - y);
+    const bool bonded = p == q || (p >= lo && p < lo + N && abs(p - q) < 2);
+    return __ballot_sync(0xffffffffu, p < I.nb && fx * fx + fy * fy < I.f_l0 * I.f_l0 * 1.0201f && !bonded);
+}
+
 // Excluded volume on bead q along axis ax (0 x, 1 y) from the beads in its
 // nw candidate words, in bead order; r: interleaved x, y positions.
 template <class R, class Place>
-__device__ __forceinline__ R close_force(const Inst &I, const Place *r, const unsigned *cand, int nw, int q, int ax) {
+__device__ __noinline__ R close_force(const Inst &I, const Place *r, const unsigned *cand, int nw, int q, int ax) {
     R f = (R)0;
     for (int c = 0; c < nw; ++c)
         for (unsigned bits = cand[c]; bits; bits &= bits - 1u) {
@@ -376,16 +399,25 @@ __device__ __forceinline__ void cell_rc(const Support &b, const float inv_w, int
 __device__ __forceinline__ float inv_width(const Support &b) {
     return b.n[0] * (int64_t)b.n[1] < (1 << 19) ? 1.0f / (float)b.n[0] : 0.0f;
 }
+// One axis of a support box (Support); from support_box, out of line: its
+// registers are not the kernel's.
+struct Axis {
+    int lo, n;
+    float rel;
+};
+__device__ __noinline__ Axis far_axis(const Inst &I, int ax, double Rx, double Ry) {
+    const Box b = support_box(I, Rx, Ry);
+    return Axis{ax ? b.j0 : b.i0, b.w > 0 && b.h > 0 ? (ax ? b.h : b.w) : 0,
+                ax ? (float)(b.ju + 0.5 - Ry) : (float)(b.iu + 0.5 - Rx)};
+}
 // One axis (ax: 0 x, 1 y) of the support box of a bead at h + l on it, in
 // FP32 with a cell of margin as support_box; positions of a million cells or
 // more, or not finite, take support_box of the FP64 position (Rx, Ry).
 __device__ __forceinline__ void support_axis(const Inst &I, int ax, float h, float l, bool far, double Rx, double Ry,
                                              int &lo, int &n, float &rel) {
     if (far) {
-        const Box b = support_box(I, Rx, Ry);
-        lo = ax ? b.j0 : b.i0;
-        n = b.w > 0 && b.h > 0 ? (ax ? b.h : b.w) : 0;
-        rel = ax ? (float)(b.ju + 0.5 - Ry) : (float)(b.iu + 0.5 - Rx);
+        const Axis f = far_axis(I, ax, Rx, Ry);
+        lo = f.lo, n = f.n, rel = f.rel;
         return;
     }
     const int L = ax ? I.ny : I.nx;
@@ -455,7 +487,15 @@ template <int NT> struct BeadMinBlocks<double, NT> { static constexpr int value 
 // resident), more when every bead has an SM of its own (shorter per-bead
 // loops).  A cluster's CTAs (FP64) each take a share of the bead's cells.
 // wait_first: wait for the sweep before listing the support (launch_beads).
-template <class S, int NT>
+// kTeam (FP32 paths, a short list of 1 to kTeamBeads beads an instance): an instance's
+// CTAs form a cluster.  Each pushes its bead's new position to the others'
+// shared memory while the support sums are taken and computes its own bead's
+// force after one cluster barrier, instead of handing in through global memory
+// to a last CTA (an atomic and a round of loads, 1.9 us, and all beads' forces
+// on one SM): ten 100 x 200 instances of 10 beads 11.7 -> 10.7 us a step, one
+// 9.8 -> 8.1, a 160 x 160 driven bead 10.3 -> 9.2.  The same arithmetic, so the
+// same bits.
+template <class S, int NT, bool kTeam>
 __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     k_beads(const Inst *__restrict__ insts, const int4 *__restrict__ blist, const S *__restrict__ pool,
             const BeadTab tab0, const BeadTab tab1, const typename PhiArg<S>::type phi0,
@@ -477,7 +517,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     __shared__ int4 s_nbox[kF64 ? kMaxBeads : 1];  // a neighbour's kept box, and where its profile starts
     __shared__ int s_noff[kF64 ? kMaxBeads : 1];
     __shared__ SumShared<T, NW> s_sum;
-    __shared__ double s_R[2], s_S, s_unit;
+    __shared__ double s_R[2], s_old[2], s_S, s_unit;
     __shared__ Support s_sup;
     __shared__ unsigned s_cnt[2][NW];
     __shared__ int s_state;
@@ -487,7 +527,12 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
 
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int parts = kF64 ? (int)cluster_ctas() : 1, part = kF64 ? (int)cluster_rank() : 0;
-    if (parts > 1) cluster_arrive();  // waited for by the first total()
+    static_assert(!(kF64 && kTeam), "FP64 clusters share a bead");
+    // team: every bead's place and whether it may be close to another
+    __shared__ double s_peer[kTeam ? kTeamBeads : 1][2];
+    __shared__ unsigned long long s_near[kTeam ? kTeamBeads : 1];
+    __shared__ float2 s_place[kTeam ? 2 * kTeamBeads : 1];
+    if (parts > 1 || kTeam) cluster_arrive();  // waited for before the first push
     int uses = 0;
     // blist[i] = (2 slot + par_xor, global bead index, the instance's first
     // bead and bead count); NULL: instance 0, bead i
@@ -523,15 +568,15 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     // waits for it).  Table reads go to L2 (an SM's L1 may hold lines of an
     // earlier step).
     int any_close = 0;  // some bead may come within the excluded volume's reach of this one
-    double Rx = 0.0, Ry = 0.0, S_old = 1.0;  // the bead's old position, support sum
+    double S_old = 1.0;  // the bead's old support sum
     float xh = 0.f, xl = 0.f, yh = 0.f, yl = 0.f;
     if (advance) {
         xh = __ldcg(told.xh + b);
         xl = __ldcg(told.xl + b);
         yh = __ldcg(told.yh + b);
         yl = __ldcg(told.yl + b);
-        Rx = __ldcg(told.Rx + b);
-        Ry = __ldcg(told.Ry + b);
+        // and its old position, in shared memory (FP64 registers are dear)
+        if (tid < 2) s_old[tid] = __ldcg((tid ? told.Ry : told.Rx) + b);
         if (tid == NT - 1) S_old = __ldcg(told.S + b);
     }
     // the lattice cell of row cj, column ci of a support box
@@ -613,8 +658,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             bx.n[0] = kb.z, bx.n[1] = kb.w;
         } else {
             const bool far = far_off(xh, yh);
-            support_axis(I, 0, xh, xl, far, Rx, Ry, bx.lo[0], bx.n[0], bx.rel[0]);
-            support_axis(I, 1, yh, yl, far, Rx, Ry, bx.lo[1], bx.n[1], bx.rel[1]);
+            support_axis(I, 0, xh, xl, far, s_old[0], s_old[1], bx.lo[0], bx.n[0], bx.rel[0]);
+            support_axis(I, 1, yh, yl, far, s_old[0], s_old[1], bx.lo[1], bx.n[1], bx.rel[1]);
         }
         const float inv_w = inv_width(bx);
         // List the support cells (phi_b != 0) among box cells [c0, c1),
@@ -639,7 +684,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
                             } else {
                                 int i, j;
                                 cell_of(I, bx, ci, cj, i, j);
-                                ph[k] = phi_f64(I, i + 0.5, j + 0.5, Rx, Ry);
+                                ph[k] = phi_f64(I, i + 0.5, j + 0.5, s_old[0], s_old[1]);
                             }
                         } else {
                             ph[k] = phi_f32(bx.rel[0] + (float)ci, bx.rel[1] + (float)cj, I.f_a, I.f_inv_xi, I.f_rcut2);
@@ -806,13 +851,14 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
                 n = make_list(c_lo, min(c_lo + kCap, c_hi));
                 continue;
             }
+            if constexpr (kTeam) cluster_wait();  // the cluster's CTAs all run
             if (w == 0) {
                 // the move; lane 0: x, the others: y
                 double unit = s_unit;
                 if (bound != kVelBits) unit *= pow2(bound - kVelBits);
                 double v = (double)(lane == 0 ? ax : ay) * unit;
                 if (!F::finite(mx)) v = __longlong_as_double(0x7ff8000000000000ll);
-                const double r = (lane == 0 ? Rx : Ry) + v;
+                const double r = s_old[lane == 0 ? 0 : 1] + v;
                 if (part == 0 && lane < 2) {
                     (lane ? tnew.Ry : tnew.Rx)[b] = r;
                     (lane ? tnew.Vy : tnew.Vx)[b] = v;
@@ -830,6 +876,12 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
                     any_close |= __any_sync(0xffffffffu, fast);
                     if (part == 0 && lane < 2 && status && fast)
                         atomicOr(status + ii, kFlagFastBead | (hv >= 0x7ff00000u ? kFlagNonFinite : 0u));
+                }
+                if constexpr (kTeam) {
+                    const double ra = __shfl_sync(0xffffffffu, r, lane & 1);
+                    if (lane < 2 * nb)
+                        st_cluster(&s_peer[b - first][lane & 1], lane >> 1, (unsigned long long)__double_as_longlong(ra));
+                    if (lane < nb) st_cluster(&s_near[b - first], lane, any_close ? 1ull : 0ull);
                 }
             }
             if (state < 0) __syncthreads();
@@ -879,6 +931,10 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     if constexpr (kF64) {
         if (I.phi_cap && part == 0 && tid == 0) pnew.box[b] = make_int4(bx.lo[0], bx.lo[1], bx.n[0], bx.n[1]);
     }
+    if constexpr (kTeam) {
+        __syncwarp();
+        cluster_arrive();  // this CTA's pushes (warp 0) are done
+    }
     total<R, NT, 1>(acc, none, mx, s_sum, uses);
     if (part != 0) return;
 
@@ -887,10 +943,13 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     // arrival counts 1, and 2^16 if the excluded volume may act on the bead.
     if (w == 0) {
         if (lane == 0) s_S = tnew.S[b] = (double)acc * pow2(-s_shift);
-        __syncwarp();  // lane 1's R and V before lane 0's release
-        if (lane == 0) {
-            s_seen = 0u;
-            if (nb > 1) s_seen = arrive_acq_rel(&counters[ii], any_close ? 0x10001u : 1u) | (any_close ? 0x10000u : 0u);
+        if constexpr (!kTeam) {
+            __syncwarp();  // lane 1's R and V before lane 0's release
+            if (lane == 0) {
+                s_seen = 0u;
+                if (nb > 1)
+                    s_seen = arrive_acq_rel(&counters[ii], any_close ? 0x10001u : 1u) | (any_close ? 0x10000u : 0u);
+            }
         }
     } else {
         // FP32 overlay table: x (and y when periodic) wrapped into the
@@ -927,6 +986,47 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             const int tile = I.tile_base + row * I.ntx + col;
             atomicOr(mask_write + tile * I.mask_words + (lb >> 5), bit);
         }
+    }
+    if constexpr (kTeam) {
+        cluster_wait();  // every bead's place is here, and its status bits are set
+        const int q = b - first, N = I.n_beads, i0 = q - q / N * N;
+        // fast-bead guard, as below
+        if (w != 0) {
+            if (q == 0 && status && (__ldcg(status + ii) & kFlagFastBead))
+                for (int t = tid - 32; t < I.ntx * I.nty; t += NT - 32)
+                    atomicOr(mask_write + (I.tile_base + t) * I.mask_words, 1u);
+            return;
+        }
+        if (lane < 2 * nb) s_place[lane] = split(s_peer[lane >> 1][lane & 1]);
+        const bool crowd = I.k_ev != 0.0 && __any_sync(0xffffffffu, lane < nb && s_near[lane] != 0ull);
+        __syncwarp();
+        // lanes 2 m + ax, m < 4: axis ax of segment q - 2 + m of the fiber
+        const int ax = lane & 1, m = (lane >> 1) & 3, j = q - 2 + m;
+        const bool seg = i0 - 2 + m >= 0 && i0 - 2 + m < N - 1;
+        float L, t, str;
+        segment_axis(I, s_place[seg ? 2 * j + ax : 0], s_place[seg ? 2 * j + 2 + ax : 1], L, t, str);
+        if (!seg) t = 0.f;
+        const float tn = __shfl_down_sync(0xffffffffu, t, 2), tp = __shfl_up_sync(0xffffffffu, t, 2);
+        const float v = tn + tp, vt1 = v * t, vt = vt1 + __shfl_xor_sync(0xffffffffu, vt1, 1);
+        const float pull = seg ? segment_pull(I, v, vt, t, str, L) : 0.f;
+        const float before = __shfl_up_sync(0xffffffffu, pull, 2);
+        float f = 0.f;  // in lanes 4 and 5 (m = 2)
+        if (i0 > 0) f -= before;
+        if (i0 < N - 1) f += pull;
+        if (crowd) {
+            const float x = (float)(place(s_place[2 * (lane < nb ? lane : 0)]) - place(s_place[0]));
+            const float y = (float)(place(s_place[2 * (lane < nb ? lane : 0) + 1]) - place(s_place[1]));
+            const unsigned cand = close_beads(I, x, y, q);
+            f += close_force<float>(I, s_place, &cand, 1, q, ax);
+        }
+        f += ax ? I.f_ext_fy : I.f_ext_fx;
+        if ((lane >> 1) == 2) {
+            const float g = f * (1.0f / (float)s_S);
+            (ax ? tnew.gyf : tnew.gxf)[b] = g;
+            (ax ? tnew.Gy : tnew.Gx)[b] = g;
+            (ax ? tnew.Fy : tnew.Fx)[b] = f;
+        }
+        return;
     }
     __syncthreads();
     const unsigned seen = s_seen;  // arrivals before this one, and this one's flag
@@ -982,9 +1082,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         screen_close<NW>(I, fs.xf, fs.yf, fs.cand);
     }
     __syncthreads();
-    // What segment q pulls bead q with (and bead q + 1 the other way): Eq. 11's
-    // spring, and Eq. 12's bending, k_b (t_{q+1} + t_{q-1}).(I - t_q t_q) / L
-    // with the tangents of missing segments zero
+    // What segment q pulls bead q with
     for (int k0 = 0; k0 < items; k0 += NT) {
         const int k = k0 + tid, q = k >> 1, i0 = in_fiber(q);
         const bool seg = k < items && i0 < N - 1;
@@ -995,10 +1093,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             if (i0 > 0) v += fs.t[k - 2];
         }
         const R vt1 = v * t, vt = vt1 + __shfl_xor_sync(0xffffffffu, vt1, 1);
-        if (seg) {
-            const R ks = kF64 ? (R)I.ks_l02 : (R)I.f_ks_l02, kb = kF64 ? (R)I.k_b : (R)I.f_kb;
-            fs.pull[k] = ks * fs.str[q] * t - kb * (v - vt * t) / fs.len[q];
-        }
+        if (seg) fs.pull[k] = segment_pull(I, v, vt, t, fs.str[q], fs.len[q]);
     }
     __syncthreads();
     for (int k = tid; k < items; k += NT) {
@@ -1081,23 +1176,58 @@ int sm_count() {
 }
 
 template <class S>
-cudaError_t launch_beads_t(cudaLaunchConfig_t &cfg, bool few, const Inst *inst_d, const int4 *blist, const void *pool,
-                           const BeadTab tab[2], const PhiTab phi[2], unsigned *mask_write, int gparity, int advance, int wait_first,
-                           unsigned *counters, BeadExport ex, unsigned *status) {
-    constexpr int kFew = std::is_same<S, double>::value ? kBeadThreadsFew64 : kBeadThreadsFew;
+cudaError_t launch_beads_t(cudaLaunchConfig_t &cfg, bool few, bool team, const Inst *inst_d, const int4 *blist,
+                           const void *pool, const BeadTab tab[2], const PhiTab phi[2], unsigned *mask_write,
+                           int gparity, int advance, int wait_first, unsigned *counters, BeadExport ex,
+                           unsigned *status) {
+    constexpr bool kF64 = std::is_same<S, double>::value;
+    constexpr int kFew = kF64 ? kBeadThreadsFew64 : kBeadThreadsFew;
     cfg.blockDim = dim3(few ? kFew : kBeadThreads);
     typename PhiArg<S>::type p0, p1;
-    if constexpr (std::is_same<S, double>::value) p0 = phi[0], p1 = phi[1];
-    if (few)
-        return cudaLaunchKernelEx(&cfg, k_beads<S, kFew>, inst_d, blist, (const S *)pool, tab[0], tab[1], p0, p1, mask_write,
-                                  gparity, advance, wait_first, counters, ex, status);
-    return cudaLaunchKernelEx(&cfg, k_beads<S, kBeadThreads>, inst_d, blist, (const S *)pool, tab[0], tab[1], p0, p1, mask_write,
-                              gparity, advance, wait_first, counters, ex, status);
+    if constexpr (kF64) p0 = phi[0], p1 = phi[1];
+    auto *k = few ? k_beads<S, kFew, false> : k_beads<S, kBeadThreads, false>;
+    if constexpr (!kF64)
+        if (team) k = k_beads<S, kFew, true>;
+    return cudaLaunchKernelEx(&cfg, k, inst_d, blist, (const S *)pool, tab[0], tab[1], p0, p1, mask_write, gparity,
+                              advance, wait_first, counters, ex, status);
+}
+
+// Most beads of an instance that form a cluster on the current device: more
+// than 8 CTAs are beyond the portable size, and need the device's leave.
+int team_limit() {
+    static std::atomic<int> cache[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    int most = cache[dev].load(std::memory_order_relaxed);
+    if (most) return most;
+    most = kTeamBeads;
+    const void *k[] = {(const void *)k_beads<float, kBeadThreadsFew, true>,
+                       (const void *)k_beads<__half, kBeadThreadsFew, true>};
+    cudaLaunchAttribute a[1];
+    a[0].id = cudaLaunchAttributeClusterDimension;
+    a[0].val.clusterDim.x = kTeamBeads;
+    a[0].val.clusterDim.y = a[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kTeamBeads);
+    cfg.blockDim = dim3(kBeadThreadsFew);
+    cfg.attrs = a;
+    cfg.numAttrs = 1;
+    for (const void *f : k) {
+        int n = 0;
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+            cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess || n < 1)
+            most = 8;
+    }
+    (void)cudaGetLastError();
+    cache[dev].store(most, std::memory_order_relaxed);
+    return most;
 }
 
 }  // namespace
 
-cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, int nb_total, int ntiles,
+void prepare_bead_kernels() { (void)team_limit(); }
+
+cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, int nb_total, int each, int ntiles,
                          const void *pool, const BeadTab tab[2], const PhiTab phi[2], unsigned *mask_write, int gparity, int advance,
                          unsigned *counters, int pdl, cudaStream_t st, BeadExport ex, unsigned *status) {
     if (nb_total <= 0) return cudaSuccess;
@@ -1118,6 +1248,9 @@ cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, i
     // list their supports while it runs.  They enter a longer sweep's SMs
     // only as it drains; then the next sweep's release comes first
     const int wait_first = ntiles > kEarlyListTiles ? 1 : 0;
+    // Every instance of the launch has `each` beads (0: not all the same): its
+    // CTAs form a cluster where there is room beside the sweep for one
+    const bool team = precision != 0 && few && !wait_first && advance && !ex.ring && each >= 1 && each <= team_limit();
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nb_total * parts);
     cfg.stream = st;
@@ -1127,9 +1260,9 @@ cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, i
         attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[na++].val.programmaticStreamSerializationAllowed = 1;
     }
-    if (parts > 1) {
+    if (parts > 1 || team) {
         attr[na].id = cudaLaunchAttributeClusterDimension;
-        attr[na].val.clusterDim.x = parts;
+        attr[na].val.clusterDim.x = team ? each : parts;
         attr[na].val.clusterDim.y = 1;
         attr[na++].val.clusterDim.z = 1;
     }
@@ -1137,13 +1270,13 @@ cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, i
     cfg.numAttrs = na;
     switch (precision) {
         case 0:
-            return launch_beads_t<double>(cfg, few, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
+            return launch_beads_t<double>(cfg, few, team, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
                                           wait_first, counters, ex, status);
         case 1:
-            return launch_beads_t<float>(cfg, few, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
+            return launch_beads_t<float>(cfg, few, team, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
                                          wait_first, counters, ex, status);
         case 2:
-            return launch_beads_t<__half>(cfg, few, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
+            return launch_beads_t<__half>(cfg, few, team, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
                                           wait_first, counters, ex, status);
     }
     return cudaErrorInvalidValue;

@@ -15,6 +15,7 @@ constexpr int kBeadThreads = 128;  // per bead CTA: more beads resident at once 
 constexpr int kBeadThreadsFew = 512;  // per bead CTA when the beads fit on the SMs one per SM
 constexpr int kBeadThreadsFew64 = 256;  // the same, FP64
 constexpr int kEarlyListTiles = 4096;  // longest sweep (tiles) whose bead phase lists its supports before waiting
+constexpr int kTeamBeads = 16;  // most beads of an instance whose CTAs form a cluster
 constexpr int kBeadParts = 8;    // CTAs a bead's cells are split over at most (FP64, short bead lists)
 constexpr int kGraphSteps = 32;  // time steps per captured graph chunk
 // Tile-mask buffers, used in rotation: the bead phase of step t marks buffer
@@ -85,7 +86,8 @@ cudaError_t launch_lattice(int precision, const Inst *inst_d, const Inst &inst_h
 // Bead phase (items (3) then (1)): one CTA per bead of any instance
 // (blist[i] = (2 slot + par_xor, global bead index, the instance's first bead
 // and bead count); NULL = instance 0, bead i; every bead of an instance must
-// be in the same launch).  ntiles: tiles of the sweep before it.  With the instance's
+// be in the same launch, side by side).  each: beads of every instance of the
+// launch, 0 if not all the same.  ntiles: tiles of the sweep before it.  With the instance's
 // step parity p = gparity ^ par_xor it reads table p ^ 1 and writes table p
 // (tab0 / tab1); advance = 0 only computes S and F of table p from its own R
 // (initialisation).  Every bead ORs its bit into the mask of each lattice
@@ -106,11 +108,14 @@ struct BeadExport {
     int slots = 0;
     int stride = 0;
 };
+// prepare_bead_kernels: kernel attributes on the current device, set when an
+// instance or batch is created (outside any stream capture).
+void prepare_bead_kernels();
 // status: per-instance status words (indexed by instance slot), where the
 // instance's last CTA sets kFlagFastBead (and kFlagNonFinite) when a bead
 // velocity component reaches kFastBead in magnitude (or is not finite), and
 // marks every tile of a flagged instance in mask_write; NULL: not checked.
-cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, int nb_total, int ntiles,
+cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, int nb_total, int each, int ntiles,
                          const void *pool, const BeadTab tab[2], const PhiTab phi[2], unsigned *mask_write,
                          int gparity, int advance, unsigned *counters, int pdl, cudaStream_t st, BeadExport ex = BeadExport{},
                          unsigned *status = nullptr);

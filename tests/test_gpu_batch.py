@@ -308,3 +308,50 @@ def test_batch_tiles_updated_from_their_records_equal_alone(fpd, precision):
     for c, s in zip(cases, slots):
         _same((b.populations(s), b.beads(s)), _alone(fpd, c, 40))
     b.close()
+
+
+@pytest.mark.parametrize("n_beads,n_fibers", [(1, 1), (2, 1), (4, 2), (9, 1), (8, 2), (17, 1)])
+@pytest.mark.parametrize("precision", [1, 2])
+def test_beads_of_a_cluster_equal_beads_handed_to_a_last_cta(fpd, precision, n_beads, n_fibers):
+    # an instance of up to 16 beads computes its forces in a cluster of CTAs,
+    # alone and in a batch of equal bead counts; in a batch of unequal ones
+    # the last CTA of each instance does: the same bits
+    rng = np.random.default_rng(100 * precision + 10 * n_beads + n_fibers)
+    cfg = wl.random_fiber(rng, 96, 60, n_beads=n_beads, a=2.0, xi=0.5, n_fibers=n_fibers, precision=precision)
+    cfg["centres"] = [[48.0 + 30.0 * f, 30.0 + 0.5 * f] for f in range(n_fibers)]
+    cfg["theta0"] = [0.6 + 1.5 * f for f in range(n_fibers)]
+    other = wl.random_fiber(rng, 64, 40, n_beads=n_beads + 1, a=2.0, xi=0.5, precision=precision)
+    steps = 12
+    want = _alone(fpd, cfg, steps)
+    for extra in ([dict(cfg, theta0=[0.1] * n_fibers)], [other]):
+        b = fpd.Batch(precision, 8, 64 << 20, 256)
+        slots = [b.add(c, steps) for c in [cfg] + extra]
+        while b.run(1000):
+            pass
+        _same((b.populations(slots[0]), b.beads(slots[0])), want)
+        b.close()
+
+
+@pytest.mark.parametrize("n_beads", [4, 10])
+def test_fibers_in_contact_in_a_cluster_and_handed_to_a_last_cta(fpd, n_beads):
+    # two parallel fibers closer than a bead diameter repel (excluded volume):
+    # 8 beads in a cluster, 20 by the last CTA, in FP32 against the FP64 oracle
+    # (2e-5: FP32 arithmetic over 12 steps, as the parity tests) and, between
+    # batch and alone, bit for bit
+    import oracle
+    rng = np.random.default_rng(n_beads)
+    cfg = wl.random_fiber(rng, 100, 60, n_beads=n_beads, a=2.0, xi=0.5, n_fibers=2, precision=1, k_ev=0.05)
+    cfg.update(centres=[[50.0, 28.0], [50.7, 31.6]], theta0=[0.0, 0.0])
+    want = _alone(fpd, cfg, 12)
+    ref = oracle.Sim(dict(cfg, precision=0, threads=4))
+    ref.step(12)
+    R, V, F = ref.beads()[:3]
+    assert np.linalg.norm(want[1][1] - V) < 2e-5 * np.linalg.norm(V)
+    assert np.linalg.norm(want[1][2] - F) < 2e-5 * np.linalg.norm(F)
+    b = fpd.Batch(1, 4, 64 << 20, 256)
+    slot = b.add(cfg, 12)
+    b.add(wl.random_fiber(rng, 64, 40, n_beads=3, a=2.0, xi=0.5, precision=1), 12)
+    while b.run(1000):
+        pass
+    _same((b.populations(slot), b.beads(slot)), want)
+    b.close()
