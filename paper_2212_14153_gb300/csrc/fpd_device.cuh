@@ -527,7 +527,11 @@ __device__ __forceinline__ double phi_f64(const Inst &I, double xc, double yc, d
     const double r2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
     if (!(r2 < I.rcut2)) return 0.0;
     const double r = sqrt(r2);
-    return 0.5 * (tanh((I.a - r) / I.xi) + 1.0);
+    // dividing by a power of two and multiplying by its inverse round alike;
+    // the division is about ten FP64 instructions
+    const unsigned long long xi = (unsigned long long)__double_as_longlong(I.xi);
+    const double z = (xi << 12) == 0ull ? (I.a - r) * I.inv_xi : (I.a - r) / I.xi;
+    return 0.5 * (tanh(z) + 1.0);
 }
 
 // Cells whose centre may lie within the cutoff of (Rx, Ry): a box that wraps
@@ -613,16 +617,6 @@ __device__ __forceinline__ int box_place(const Inst &I, const int4 &bx, int i, i
     if (e < 0 && I.periodic_y) e += I.ny;
     return (d < bx.z && (unsigned)e < (unsigned)bx.w) ? e * bx.z + d : -1;
 }
-// phi_f64 of bead q (table index) at lattice cell (i, j): kept, or evaluated
-// (the same bits).
-__device__ __forceinline__ double phi_cell(const Inst &I, const BeadTab &tab, const PhiTab &pt, int q, int i, int j) {
-    if (I.phi_cap) {
-        const int at = box_place(I, pt.box[q], i, j);
-        return at >= 0 ? pt.phi[I.phi_off + (q - I.bead_off) * I.phi_cap + at] : 0.0;
-    }
-    return phi_f64(I, i + 0.5, j + 0.5, tab.Rx[q], tab.Ry[q]);
-}
-
 // FP32 variant for the reduced-precision lattice path: dx, dy relative to a
 // tile origin already reduced to small numbers by the caller.  Evaluated as
 // the logistic function, phi = 1 / (1 + exp(2 (r - a) / xi)), with r - a =

@@ -68,7 +68,7 @@ __device__ __forceinline__ const float *stage_overlay(const Inst &I, const BeadT
 // beads marked in its tile's mask (m, W words; any = OR of the words).
 // kStaged: the FP32 overlay entries are read from sov (stage_overlay), else
 // from the table; the values and their order are the same either way.
-template <class R, bool kStaged, class P>
+template <class R, bool kStaged, int kOver, class P>
 __device__ __forceinline__ void cell_overlay(const Inst &I, const BeadTab &tab, const P &pt, const float *__restrict__ sov,
                                              const unsigned *__restrict__ m,
                                              const int W, const unsigned any, const int x, const int y, R &Fx,
@@ -84,17 +84,43 @@ __device__ __forceinline__ void cell_overlay(const Inst &I, const BeadTab &tab, 
             return;
         }
         double Phi = I.sandwich ? sandwich_phi_f64(I, y + 0.5) : 0.0;
+        // kept profiles (PhiTab), kOver beads at a time: their boxes, then their
+        // profiles, are asked for together (one after the other they cost two
+        // memory round trips a bead, which set the time of a lattice of few
+        // tiles); otherwise evaluated
         for (int w = 0; w < W && any; ++w) {
             unsigned bits = m[w];
             while (bits) {
-                const int q = I.bead_off + 32 * w + __ffs(bits) - 1;
-                bits &= bits - 1u;
-                const double ph = phi_cell(I, tab, pt.phi, q, x, y);
-                if (ph != 0.0) {
-                    Phi += ph;
-                    Fx += ph * tab.Gx[q];
-                    Fy += ph * tab.Gy[q];
+                int q[kOver];
+                double ph[kOver];
+                const int first = I.bead_off + 32 * w - 1;
+                if (I.phi_cap) {
+                    int4 bx[kOver];
+#pragma unroll
+                    for (int k = 0; k < kOver; ++k) {
+                        q[k] = bits ? first + __ffs(bits) : -1;
+                        bits &= bits - 1u;
+                        if (q[k] >= 0) bx[k] = pt.phi.box[q[k]];
+                    }
+#pragma unroll
+                    for (int k = 0; k < kOver; ++k) {
+                        const int at = q[k] >= 0 ? box_place(I, bx[k], x, y) : -1;
+                        ph[k] = at >= 0 ? pt.phi.phi[I.phi_off + (q[k] - I.bead_off) * I.phi_cap + at] : 0.0;
+                    }
+                } else {
+                    q[0] = first + __ffs(bits);
+                    bits &= bits - 1u;
+                    ph[0] = phi_f64(I, x + 0.5, y + 0.5, tab.Rx[q[0]], tab.Ry[q[0]]);
+#pragma unroll
+                    for (int k = 1; k < kOver; ++k) ph[k] = 0.0;
                 }
+#pragma unroll
+                for (int k = 0; k < kOver; ++k)
+                    if (ph[k] != 0.0) {
+                        Phi += ph[k];
+                        Fx += ph[k] * tab.Gx[q[k]];
+                        Fy += ph[k] * tab.Gy[q[k]];
+                    }
             }
         }
         const double nu = I.nu_f * (1.0 + (I.visc_ratio - 1.0) * Phi);
@@ -223,7 +249,7 @@ template <class S> struct AdjPairs { static constexpr bool value = !std::is_same
 // two unforced cells in packed FP32 pairs, else cell by cell) and the stores
 // into buffer Adst.  g holds the pulled populations in stored units; the
 // cells' layout is lattice_tile's (kAlongX, CY, kAdj).
-template <class S, int CY, bool kInner, bool kAlongX, int kColl, bool kStream>
+template <class S, int CY, bool kInner, bool kAlongX, int kColl, bool kStream, int kOver = 1>
 __device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, const typename SweepArg<S>::type &pt,
                                              const float *__restrict__ sov,
                                              const unsigned *__restrict__ m, const int W, const unsigned any,
@@ -256,7 +282,7 @@ __device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, 
             R Fx, Fy, s_e, s_eps, s_nu[2], s_q[2];
 #pragma unroll
             for (int k = 0; k < 2; ++k)
-                cell_overlay<R, kStream>(I, tab, pt, sov, m, W, any, x + k * RX, y[k], Fx, Fy, s_nu[k], s_e, s_eps,
+                cell_overlay<R, kStream, kOver>(I, tab, pt, sov, m, W, any, x + k * RX, y[k], Fx, Fy, s_nu[k], s_e, s_eps,
                                          s_q[k]);
             float2 v[9];
 #pragma unroll
@@ -272,7 +298,7 @@ __device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, 
     for (int k = 0; k < CY; ++k) {
         if (!valid[k]) continue;
         R Fx, Fy, s_nu, s_e, s_eps, s_q;
-        cell_overlay<R, kStream>(I, tab, pt, sov, m, W, any, x + k * RX, y[k], Fx, Fy, s_nu, s_e, s_eps, s_q);
+        cell_overlay<R, kStream, kOver>(I, tab, pt, sov, m, W, any, x + k * RX, y[k], Fx, Fy, s_nu, s_e, s_eps, s_q);
         collide_cell<S, R, kColl>(I, pt, g[k], Fx, Fy, s_nu, s_e, s_eps, s_q, forced);
     }
     store();
@@ -290,7 +316,7 @@ __device__ __forceinline__ void finish_cells(const Inst &I, const BeadTab &tab, 
 // tiles away from walls and periodic edges use the in-strip pull offsets.
 // kStream: the population loads and stores carry the L2 evict-first
 // priority (the single-lattice sweep).
-template <class S, int CY, bool kInner, bool kAlongX, int kColl, bool kStream = false>
+template <class S, int CY, bool kInner, bool kAlongX, int kColl, bool kStream = false, int kOver = 1>
 __device__ __forceinline__ void lattice_tile(const Inst &I, S *__restrict__ pool, const BeadTab &tab,
                                              const typename SweepArg<S>::type &pt,
                                              const unsigned *__restrict__ mask_read,
@@ -393,7 +419,7 @@ __device__ __forceinline__ void lattice_tile(const Inst &I, S *__restrict__ pool
     const float *sov = stage_overlay<R, kStream>(I, tab, m, any);  // every thread of the CTA
     if (!valid[0]) return;  // the thread's other cells (further along its column or row) are invalid too
     if (!early_load) pull();
-    finish_cells<S, CY, kInner, kAlongX, kColl, kStream>(I, tab, pt, sov, m, W, any, x, y, valid, C, g, Adst, cx0, pol);
+    finish_cells<S, CY, kInner, kAlongX, kColl, kStream, kOver>(I, tab, pt, sov, m, W, any, x, y, valid, C, g, Adst, cx0, pol);
 }
 
 // Tile order of a single-lattice sweep.  Every other step takes the tiles
@@ -412,7 +438,7 @@ __global__ void __launch_bounds__(kTileX *kTileY / CY)
     k_lattice(const Inst I, S *__restrict__ pool, const BeadTab tab, const unsigned *__restrict__ mask_read,
               const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear, const int parity,
               const int early_load, const int early_cold, const typename SweepArg<S>::type pt) {
-    lattice_tile<S, CY, true, kAlongX, kColl, true>(I, pool, tab, pt, mask_read, mask_prev, mask_clear,
+    lattice_tile<S, CY, true, kAlongX, kColl, true, kSplit ? 4 : 1>(I, pool, tab, pt, mask_read, mask_prev, mask_clear,
                                        tile_order(blockIdx.x, gridDim.x, parity),
                                        tile_order(blockIdx.y, gridDim.y, parity), parity, early_load, early_cold,
                                        (blockIdx.x | blockIdx.y | (kSplit ? blockIdx.z : 0u)) == 0, threadIdx.x,
@@ -993,7 +1019,7 @@ __device__ __forceinline__ void lattice_tile_vec(const Inst &I, S *__restrict__ 
 #pragma unroll
         for (int j = 0; j < NV; ++j) {
             R Fx, Fy, s_nu, s_e, s_eps, s_q;
-            cell_overlay<R, true>(I, tab, pt, sov, m, W, any, x0 + j, y, Fx, Fy, s_nu, s_e, s_eps, s_q);
+            cell_overlay<R, true, 1>(I, tab, pt, sov, m, W, any, x0 + j, y, Fx, Fy, s_nu, s_e, s_eps, s_q);
             collide_cell<S, R, kCollTrt>(I, pt, g[j], Fx, Fy, s_nu, s_e, s_eps, s_q, forced);
         }
     }
