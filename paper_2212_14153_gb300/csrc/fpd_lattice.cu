@@ -432,12 +432,32 @@ __device__ __forceinline__ void lattice_tile(const Inst &I, S *__restrict__ pool
 // (its state is many times the L2: reversing measured no gain there).
 __device__ __forceinline__ int tile_order(int b, int n, int parity) { return (parity & 1) ? n - 1 - b : b; }
 
+// A lattice about as large as L2 or larger has its sweep bound by the bytes
+// that a CTA's registers keep in flight: each CTA has the populations of the
+// tile kAheadOne CTAs on brought to L2 by one bulk prefetch (its rows are
+// contiguous in its strip).  2048 x 2048, FP16, variant 1: 29.7 -> 27.2 us a
+// step (DRAM 5.08 -> 5.55 TB/s of the bytes it cannot do without).  1368 CTAs
+// on: the same; 684: 26.9 against 26.5 where these two take 26.5.  By one
+// thread.
+constexpr unsigned kAheadOne = 2736;
+template <class S>
+__device__ __forceinline__ void prefetch_ahead(const Inst &I, const S *__restrict__ pool, const int parity) {
+    const unsigned c = blockIdx.y * gridDim.x + blockIdx.x + kAheadOne;
+    if (c >= gridDim.x * gridDim.y) return;
+    const int y0 = tile_order(c / gridDim.x, gridDim.y, parity) * kTileY, rows = min(kTileY, I.ny - y0);
+    const S *p = pop_buffer(pool, I, parity) + (y0 * kRowStride + tile_order(c % gridDim.x, gridDim.x, parity) * I.strip);
+    // 16-byte aligned, a multiple of 16 bytes: prefetch_one, rows of 9 * 32 elements
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(rows * kRowStride * (int)sizeof(S)));
+}
+
 // kSplit: gridDim.z CTAs share a tile's rows (row_split).
 template <class S, int CY, bool kAlongX, int kColl, bool kSplit = false>
 __global__ void __launch_bounds__(kTileX *kTileY / CY)
     k_lattice(const Inst I, S *__restrict__ pool, const BeadTab tab, const unsigned *__restrict__ mask_read,
               const unsigned *__restrict__ mask_prev, unsigned *__restrict__ mask_clear, const int parity,
-              const int early_load, const int early_cold, const typename SweepArg<S>::type pt) {
+              const int early_load, const int early_cold, const int ahead,
+              const typename SweepArg<S>::type pt) {
+    if (!kSplit && ahead && threadIdx.x == 0 && threadIdx.y == kTileY - 1) prefetch_ahead(I, pool, parity);
     lattice_tile<S, CY, true, kAlongX, kColl, true, kSplit ? 4 : 1>(I, pool, tab, pt, mask_read, mask_prev, mask_clear,
                                        tile_order(blockIdx.x, gridDim.x, parity),
                                        tile_order(blockIdx.y, gridDim.y, parity), parity, early_load, early_cold,
@@ -1324,6 +1344,26 @@ template <class S> static int row_split(int ntiles) {
     return sp;
 }
 
+// Whether a single-lattice sweep prefetches (prefetch_ahead), from the bytes
+// of its two population buffers.  us a step of the better of variants 0 and
+// 1, without -> with:
+//   FP16:  75 MB 17.98 -> 18.06,  94 MB 18.77 -> 18.74, 113 MB 22.07 -> 20.89,
+//         151 MB 29.72 -> 27.24, 302 MB 58.3 -> 54.3, 604 MB 115.6 -> 106.1
+//   FP32: 113 MB 17.82 -> 17.50, 142 MB 21.43 -> 20.10, 226 MB 32.71 -> 32.17,
+//         264 MB 38.38 -> 38.09, 302 MB 43.55 -> 44.40, 604 MB 87.96 -> 92.63
+//   FP64: 604 MB 486.5 -> 486.6 (bound by its FP64 instructions)
+// Below 100 MB both buffers stay in L2.  Large FP32 lattices have enough bytes
+// in flight by themselves; there the reversed order of every other sweep
+// (tile_order) finds less in L2 with the prefetches in the way.
+constexpr int64_t kPrefetchMin = 100000000, kPrefetchMax32 = 280000000;
+template <class S> static int prefetch_one(const Inst &I, const void *pool) {
+    if (std::is_same<S, double>::value) return 0;
+    // the bulk prefetch needs the buffers 16-byte aligned
+    if ((reinterpret_cast<uintptr_t>((const S *)pool + I.pop_off) & 15u) != 0) return 0;
+    const int64_t bytes = 2 * 9 * (int64_t)sizeof(S) * I.nx * I.ny;
+    return bytes >= kPrefetchMin && (sizeof(S) == 2 || bytes <= kPrefetchMax32);
+}
+
 template <class S> static typename PhiArg<S>::type phi_arg(const PhiTab &p) {
     if constexpr (std::is_same<S, double>::value) return p;
     else return NoPhi{};
@@ -1343,11 +1383,12 @@ static cudaError_t lattice_v(int variant, const Inst &I, void *pool, BeadTab tab
     const int sp = row_split<S>(I.ntx * I.nty), rows = kTileY / sp;
     const dim3 split(I.ntx, I.nty, sp);
     const int ec = after_beads ? mk.early_cold : 0;
+    const int ahead = prefetch_one<S>(I, pool);
     // constant Lallemand-Luo rates: the moment form, one cell per thread
     if (I.collision == 1) {
         const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX, rows), after_beads | mk.chained, st, attr);
         return cudaLaunchKernelEx(&cfg, sp > 1 ? k_lattice<S, 1, false, kCollMrt, true> : k_lattice<S, 1, false, kCollMrt>, I, (S *)pool, tab, mk.read, mk.prev,
-                                  mk.clear, parity, after_beads, ec, pt);
+                                  mk.clear, parity, after_beads, ec, ahead, pt);
     }
     if (variant == 2 && I.nx % VecWidth<S>::value == 0) {
         const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX / VecWidth<S>::value, kTileY),
@@ -1367,11 +1408,11 @@ static cudaError_t lattice_v(int variant, const Inst &I, void *pool, BeadTab tab
     if (variant == 1 || variant == 3 || variant == 4) {
         const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX / 2, rows), after_beads | mk.chained, st, attr);
         return cudaLaunchKernelEx(&cfg, sp > 1 ? k_lattice<S, 2, true, kCollTrt, true> : k_lattice<S, 2, true, kCollTrt>, I, (S *)pool, tab, mk.read, mk.prev,
-                                  mk.clear, parity, after_beads, ec, pt);
+                                  mk.clear, parity, after_beads, ec, ahead, pt);
     }
     const cudaLaunchConfig_t cfg = sweep_config(split, dim3(kTileX, rows), after_beads | mk.chained, st, attr);
     return cudaLaunchKernelEx(&cfg, sp > 1 ? k_lattice<S, 1, false, kCollTrt, true> : k_lattice<S, 1, false, kCollTrt>, I, (S *)pool, tab, mk.read, mk.prev,
-                              mk.clear, parity, after_beads, ec, pt);
+                              mk.clear, parity, after_beads, ec, ahead, pt);
 }
 
 // The staged sweep's CTAs keep 20-46 KB of static shared memory: its

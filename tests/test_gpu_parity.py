@@ -903,3 +903,27 @@ def test_fp64_checkpoint_and_batch_rebuild_restore_the_kept_profiles(tmp_path):
         assert np.array_equal(got[0], want[0])
         for x, y in zip(got[1], want[1]):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("nx,ny,precision", [
+    (1747, 1733, 2),  # ragged last strip and tile row
+    (1251, 1233, 1),
+    (70003, 40, 2),   # five tile rows of 2188 tiles
+])
+def test_sweep_that_prefetches_against_the_staged_one(nx, ny, precision):
+    # a lattice about as large as L2 prefetches later tiles to L2 in variant
+    # 1; the staged sweep does not, and gives the same bits
+    rng = np.random.default_rng(nx)
+    cfg = wl.random_fiber(rng, nx, ny, n_beads=8, a=2.5, xi=1.0, precision=precision)
+    got = []
+    for variant in (1, 3):
+        s = gpu_sim(cfg)
+        s.set_tuning(variant)
+        for n in (1, 32, 2):
+            s.step(n)
+        assert s.flags() == 0
+        got.append((s.populations(), s.beads()))
+        s.close()
+    assert np.array_equal(got[0][0], got[1][0])
+    for x, y in zip(got[0][1], got[1][1]):
+        assert np.array_equal(x, y)
