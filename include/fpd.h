@@ -140,7 +140,9 @@ int fpd_workspace_bytes(const fpd_params *p, uint64_t *bytes);
  * 256-byte aligned address; e.g. the data of a torch tensor), which the
  * caller keeps valid until fpd_destroy and frees afterwards: the library
  * never frees it.  Buffers for reads (fpd_read_*, fpd_internal_flow) and
- * host staging are still allocated by the library on first use.  The paper
+ * host staging are still allocated by the library on first use, and FP64
+ * instances have up to 16 MB of bead profiles allocated when they are created
+ * (they run without, slower, where that fails).  The paper
  * has no counterpart: this serves applications that own device memory.
  * FPD_EINVAL for a NULL or short or misaligned workspace. */
 int fpd_create_ex(const fpd_params *p, void *stream, void *workspace, uint64_t workspace_bytes, fpd_sim **out);

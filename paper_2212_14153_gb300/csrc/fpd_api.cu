@@ -262,6 +262,8 @@ void free_all(fpd_sim *s) {
         cudaEventDestroy(r.a);
         cudaEventDestroy(r.b);
     }
+    cudaFree(s->phimem);
+    s->phimem = nullptr;
     s->pool = s->tabmem = s->scratch = nullptr;
 }
 
@@ -476,8 +478,7 @@ namespace {
 // counter and the instance record.
 constexpr size_t kStateAlign = 256;
 struct StateLayout {
-    size_t pool, tab, masks, counters, inst, phi, box, total;  // offsets; total = block size
-    size_t phi_one;  // bytes of one table's kept profiles (0: not kept)
+    size_t pool, tab, masks, counters, inst, total;  // offsets; total = block size
     size_t pool_bytes, tab_bytes, tab_one, mask_bytes, mask_words;
 };
 size_t up(size_t v) { return (v + kStateAlign - 1) / kStateAlign * kStateAlign; }
@@ -496,14 +497,28 @@ StateLayout state_layout(const fpd::Inst &I, size_t elem) {
     L.counters = up(L.masks + L.mask_bytes);
     // last-block counter, the 64-bit export counter at +8, the status word at +16
     L.inst = up(L.counters + 32);
-    // FP64: the beads' profiles over their support boxes (PhiTab), unless
-    // their supports are so wide that the two tables would outgrow kPhiBytes
-    L.phi = up(L.inst + sizeof(fpd::Inst));
-    L.phi_one = elem == 8 ? (size_t)I.nb * fpd::phi_cells(I) * sizeof(double) : 0;
-    if (2 * L.phi_one > fpd::kPhiBytes) L.phi_one = 0;
-    L.box = up(L.phi + 2 * L.phi_one);
-    L.total = up(L.box + (L.phi_one ? 2 * nbm * sizeof(int4) : 0));
+    L.total = up(L.inst + sizeof(fpd::Inst));
     return L;
+}
+
+// FP64: room for the beads' profiles over their support boxes (PhiTab), beside
+// the state block, unless the supports are so wide that the two tables would
+// outgrow kPhiBytes.  Without it (no memory left) the instance evaluates them.
+void alloc_profiles(fpd_sim *s) {
+    const fpd::Inst &I = s->inst;
+    if (s->elem != 8 || I.nb <= 0) return;
+    const size_t one = (size_t)I.nb * fpd::phi_cells(I), bytes = 2 * one * sizeof(double);
+    const size_t box = 2 * (size_t)I.nb * sizeof(int4);
+    if (bytes > fpd::kPhiBytes) return;
+    if (cudaMalloc(&s->phimem, bytes + box) != cudaSuccess) {
+        s->phimem = nullptr;
+        (void)cudaGetLastError();
+        return;
+    }
+    int4 *b = (int4 *)s->phimem;
+    double *f = (double *)(b + 2 * I.nb);
+    for (int t = 0; t < 2; ++t) s->phi[t] = fpd::PhiTab{f + t * one, b + t * I.nb};
+    s->inst.phi_cap = fpd::phi_cells(I);
 }
 
 int create_impl(const fpd_params *p, void *stream, void *workspace, uint64_t workspace_bytes, fpd_sim **out);
@@ -570,7 +585,6 @@ int create_impl(const fpd_params *p, void *stream, void *workspace, uint64_t wor
     FPD_TRY(fpd::prepare_lattice_kernels(), "sweep kernel attributes");
     fpd::prepare_bead_kernels();
     const StateLayout L = state_layout(I, s->elem);
-    s->inst.phi_cap = L.phi_one ? fpd::phi_cells(I) : 0;
     if (workspace) {
         if (workspace_bytes < L.total || ((uintptr_t)workspace % kStateAlign) != 0) {
             fail(nullptr, FPD_EINVAL, "workspace must hold %llu bytes at a %zu-byte aligned address",
@@ -596,11 +610,11 @@ int create_impl(const fpd_params *p, void *stream, void *workspace, uint64_t wor
         s->tab[t] = fpd::BeadTab{b,           b + nbm,     b + 2 * nbm, b + 3 * nbm, b + 4 * nbm,
                                  b + 5 * nbm, b + 6 * nbm, b + 7 * nbm, b + 8 * nbm, f,
                                  f + nbm,     f + 2 * nbm, f + 3 * nbm, f + 4 * nbm, f + 5 * nbm};
-        if (L.phi_one) {
-            s->phi[t].phi = (double *)(base + L.phi + t * L.phi_one);
-            s->phi[t].box = (int4 *)(base + L.box) + t * nbm;
-        }
     }
+    alloc_profiles(s);
+    if (s->phimem)
+        FPD_TRY(cudaMemsetAsync(s->phimem, 0, 2 * (size_t)nb * (sizeof(int4) + I.phi_cap * sizeof(double)), s->stream),
+                "cudaMemset kept profiles");
     // tile masks, one buffer per step of the rotation (zeroed with the block)
     s->masks[0] = (unsigned *)(base + L.masks);
     for (int m = 1; m < fpd::kMaskBufs; ++m) s->masks[m] = s->masks[0] + m * L.mask_words;

@@ -128,6 +128,22 @@ def test_workspace_bytes_without_a_device(lib):
     assert e.value.code == fpd.FPD_EINVAL
 
 
+def test_workspace_holds_the_state_only(lib):
+    # the profiles that FP64 bead phases keep lie beside the workspace: an
+    # instance's bytes differ between precisions by its populations alone
+    from paper_2212_14153_gb300 import fpd
+    import numpy as np
+    p = fpd.fpd_default_params()
+    p.nx, p.ny, p.n_beads, p.n_fibers = 96, 64, 8, 1
+    cen = np.array([48.0, 32.0]); th = np.array([0.5])
+    p.centre_xy = cen.ctypes.data_as(fpd._DP)
+    p.theta0 = th.ctypes.data_as(fpd._DP)
+    n = []
+    for p.precision in (0, 1):
+        n.append(fpd.fpd_workspace_bytes(p))
+    assert n[0] - n[1] == 2 * 9 * 96 * 64 * 4
+
+
 def test_async_bead_reads_reject_a_null_handle(lib):
     # host-only argument checks of the stream-ordered bead read
     t = ctypes.c_uint64(0)

@@ -927,3 +927,17 @@ def test_sweep_that_prefetches_against_the_staged_one(nx, ny, precision):
     assert np.array_equal(got[0][0], got[1][0])
     for x, y in zip(got[0][1], got[1][1]):
         assert np.array_equal(x, y)
+
+
+def test_fp64_in_a_caller_workspace_keeps_profiles_too():
+    import torch
+    from paper_2212_14153_gb300 import fpd
+    cfg = wl.random_fiber(np.random.default_rng(58), 70, 37, n_beads=5, a=2.0, xi=1.0)
+    ws = torch.empty(fpd.workspace_bytes(cfg), dtype=torch.uint8, device="cuda")
+    a, b = gpu_sim(cfg), fpd.Simulation(cfg, workspace=ws)
+    a.step(77)
+    b.step(77)
+    assert np.array_equal(a.populations(), b.populations())
+    for x, y in zip(a.beads(), b.beads()):
+        assert np.array_equal(x, y)
+    b.close()
