@@ -22,6 +22,7 @@
 #include <cstdio>
 #include <map>
 #include <string>
+#include <mutex>
 #include <vector>
 
 #include "fpd_sim.h"
@@ -126,6 +127,7 @@ struct fpd_batch {
     cudaStream_t cap_stream = nullptr;
     double *phi_mem = nullptr;  // FP64: both tables' kept profiles (PhiTab::phi)
     int64_t phi_len = 0;        // doubles in phi_mem
+    std::mutex stage_lock;         // of the next two
     double *host_stage = nullptr;  // pinned staging for bead reads (7 doubles a bead of the largest read so far)
     int host_beads = 0;
     double *scratch = nullptr;
@@ -748,27 +750,32 @@ int fpd_batch_read_beads(fpd_batch *b, int32_t slot, double *pos, double *vel, d
     const Slot &sl = b->slots[slot];
     const int nb = sl.inst.nb, off = sl.inst.bead_off;
     if (nb == 0) return fpd_batch_sync(b);
+    // one read at a time uses the staging, threads reading different slots wait
+    std::lock_guard<std::mutex> own(b->stage_lock);
+    std::vector<double> plain;
     if (nb > b->host_beads) {
         if (b->host_stage) cudaFreeHost(b->host_stage);
         b->host_stage = nullptr;
         b->host_beads = 0;
-        const cudaError_t e = cudaMallocHost(&b->host_stage, 7 * (size_t)nb * sizeof(double));
-        if (e != cudaSuccess) {
+        if (cudaMallocHost(&b->host_stage, 7 * (size_t)nb * sizeof(double)) == cudaSuccess) {
+            b->host_beads = nb;
+        } else {  // no page-locked memory left: pageable, slower
             b->host_stage = nullptr;
-            return bcuda(b, e, "pinned staging for bead reads");
+            (void)cudaGetLastError();
+            plain.resize(7 * (size_t)nb);
         }
-        b->host_beads = nb;
     }
+    double *const stage = b->host_stage ? b->host_stage : plain.data();
     // R, V, F, S of a table are seven consecutive arrays of max_beads
     // doubles: one strided copy into pinned memory, ordered after the queued
     // steps, instead of seven synchronous ones (59 us a slot)
     const int64_t l = sl.steps_done;
     const fpd::BeadTab &t = b->tab[l == 0 ? 0 : (int)((l - 1) & 1)];
     const size_t row = nb * sizeof(double), pitch = (size_t)(b->max_beads > 0 ? b->max_beads : 1) * sizeof(double);
-    cudaError_t e = cudaMemcpy2DAsync(b->host_stage, row, t.Rx + off, pitch, row, 7, cudaMemcpyDeviceToHost, b->stream);
+    cudaError_t e = cudaMemcpy2DAsync(stage, row, t.Rx + off, pitch, row, 7, cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(b, e, "copy beads");
-    const double *h = b->host_stage;
+    const double *h = stage;
     auto pair = [&](double *dst, int k) {
         if (!dst) return;
         const double *x = h + (size_t)k * nb, *y = x + nb;
