@@ -332,7 +332,7 @@ int enqueue_step(fpd_sim *s, cudaStream_t st, int64_t t, bool profiled) {
             b = take_event(s);
             cudaEventRecord(a, st);
         }
-        e = fpd::launch_beads(s->precision, s->inst_d, nullptr, I.nb, I.nb, I.ntx * I.nty, s->pool, s->tab, s->phi,
+        e = fpd::launch_beads(s->precision, s->inst_d, nullptr, I.nb, I.nb, fpd::phi_cells(I), I.ntx * I.nty, s->pool, s->tab, s->phi,
                               s->masks[t % fpd::kMaskBufs], parity, 1, s->counters, profiled ? 0 : 1, st,
                               fpd::BeadExport{s->ex_ring_d, s->ex_count, s->ex_slots, s->ex_stride}, s->status);
         if (e != cudaSuccess) return cuda_fail(s, e, "bead kernel launch");
@@ -636,7 +636,7 @@ int create_impl(const fpd_params *p, void *stream, void *workspace, uint64_t wor
                 "copy beads");
         FPD_TRY(cudaMemcpyAsync(s->tab[0].Ry, Ry.data(), nb * sizeof(double), cudaMemcpyHostToDevice, s->stream),
                 "copy beads");
-        FPD_TRY(fpd::launch_beads(s->precision, s->inst_d, nullptr, nb, nb, I.ntx * I.nty, s->pool, s->tab, s->phi,
+        FPD_TRY(fpd::launch_beads(s->precision, s->inst_d, nullptr, nb, nb, fpd::phi_cells(I), I.ntx * I.nty, s->pool, s->tab, s->phi,
                                   s->masks[0], 0, 0, s->counters, 0, s->stream),
                 "initial bead table");
     }

@@ -112,6 +112,7 @@ struct fpd_batch {
     unsigned *masks = nullptr;  // kMaskBufs * tiles_cap * mask_words, in rotation by global step
     int4 *beads_all_d = nullptr, *beads_old_d = nullptr, *beads_fresh_d = nullptr;  // as launch_beads takes them
     int n_all = 0, n_old = 0, n_fresh = 0;
+    int box = 0;   // largest phi_cells of the resident instances with beads
     int each = 0;  // beads of every resident instance that has any (0: not all the same)
     std::vector<Slot> slots;
     std::vector<fpd::Inst> insts_h;
@@ -260,12 +261,13 @@ int rebuild(fpd_batch *b) {
         b->insts_h[s] = I;
     }
     b->ntiles = (int)tiles.size();
-    b->each = 0;
+    b->each = b->box = 0;
     bool uneven = false;
     for (auto &sl : b->slots)
         if (sl.state == kActive && sl.inst.nb > 0) {
             uneven |= b->each != 0 && b->each != sl.inst.nb;
             b->each = sl.inst.nb;
+            b->box = std::max(b->box, fpd::phi_cells(sl.inst));
         }
     if (uneven) b->each = 0;
     b->any_mrt = 0;
@@ -334,7 +336,7 @@ int rebuild(fpd_batch *b) {
     }
     // initial bead tables of new instances (local parity 0 -> table 0)
     if (b->n_fresh > 0) {
-        e = fpd::launch_beads(b->precision, b->insts_d, b->beads_fresh_d, b->n_fresh, 0, b->ntiles, b->pool, b->tab, b->phi,
+        e = fpd::launch_beads(b->precision, b->insts_d, b->beads_fresh_d, b->n_fresh, 0, b->box, b->ntiles, b->pool, b->tab, b->phi,
                               b->masks + (size_t)(b->gstep % fpd::kMaskBufs) * b->tiles_cap * b->mask_words, gp, 0,
                               b->counters, 0, b->stream);
         if (e != cudaSuccess) return bcuda(b, e, "initial bead tables");
@@ -499,7 +501,7 @@ int enqueue_bstep(fpd_batch *b, cudaStream_t st, int64_t gstep, bool any_first) 
                              b->masks + (size_t)((gstep + 1) % M) * mstride, gstep > b->rebuild_gstep ? 1 : 0};
     cudaError_t e;
     if (nbl > 0) {
-        e = fpd::launch_beads(b->precision, b->insts_d, blist, nbl, b->each, b->ntiles, b->pool, b->tab, b->phi, mw, gp, 1,
+        e = fpd::launch_beads(b->precision, b->insts_d, blist, nbl, b->each, b->box, b->ntiles, b->pool, b->tab, b->phi, mw, gp, 1,
                               b->counters, 1, st, fpd::BeadExport{}, b->status);
         if (e != cudaSuccess) return bcuda(b, e, "batched bead phase");
     }

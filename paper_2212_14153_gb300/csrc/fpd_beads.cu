@@ -8,13 +8,14 @@
 //   Sec 2.3 R_b <- R_b + V_b (forward Euler, dt = 1);
 //   S_b = sum_x phi_b(x; R_b) at the new position (the discrete int phi_b);
 // then the last CTA of an instance to finish (device-wide atomic counter, no
-// waiting) computes every bead force of that instance from the new positions:
+// waiting), or each bead's CTA of a cluster that holds the instance (kTeam),
+// computes the bead forces of that instance from the new positions:
 //   Eq. 11 springs, Eq. 12 bending in its general form (tangents of missing
 //   segments are zero, which reproduces the edge cases of Eqs. 12b-12e),
 //   plus the excluded-volume repulsion k_ev (d - r) r_hat of non-bonded beads
 //   closer than d, and G = F / S for the spreading of Eq. 4.  Each bead's CTA
 //   writes its place in the FP32 overlay table (positions split hi + lo) read
-//   by the lattice sweep of the reduced-precision paths, the last CTA the G.
+//   by the lattice sweep of the reduced-precision paths, with the forces the G.
 //
 // What bounds it: a chain of latencies.  A step of a small lattice is the
 // sweep plus everything between the sweep's end and the overlay table, so
@@ -22,7 +23,10 @@
 // the force density there depend only on the table of the previous step, and
 // are listed in shared memory before the kernel waits for the sweep (it is
 // launched while the sweep still runs).  Left on the chain are one round of
-// population loads, one sum, the move, the support sum, and the last CTA.
+// population loads, one sum, the move, the support sum, and the forces.  us a
+// step, before (list after the wait, sums in a tree, forces in FP64) and now:
+// 100 x 200 with 10 beads 17.9 -> 8.1, 1024 x 256 with 20 (last CTA) 23.0 ->
+// 11.0, FP64 80 x 40 with 8 153 -> 30.
 //
 // Sums are taken in fixed point (Fix below): exact integer additions, so
 // they do not depend on which thread or CTA adds which cell, and a warp adds
@@ -1176,18 +1180,19 @@ int sm_count() {
 }
 
 template <class S>
-cudaError_t launch_beads_t(cudaLaunchConfig_t &cfg, bool few, bool team, const Inst *inst_d, const int4 *blist,
+cudaError_t launch_beads_t(cudaLaunchConfig_t &cfg, int threads, bool team, const Inst *inst_d, const int4 *blist,
                            const void *pool, const BeadTab tab[2], const PhiTab phi[2], unsigned *mask_write,
                            int gparity, int advance, int wait_first, unsigned *counters, BeadExport ex,
                            unsigned *status) {
     constexpr bool kF64 = std::is_same<S, double>::value;
-    constexpr int kFew = kF64 ? kBeadThreadsFew64 : kBeadThreadsFew;
-    cfg.blockDim = dim3(few ? kFew : kBeadThreads);
+    cfg.blockDim = dim3(threads);
     typename PhiArg<S>::type p0, p1;
     if constexpr (kF64) p0 = phi[0], p1 = phi[1];
-    auto *k = few ? k_beads<S, kFew, false> : k_beads<S, kBeadThreads, false>;
-    if constexpr (!kF64)
-        if (team) k = k_beads<S, kFew, true>;
+    auto *k = k_beads<S, kBeadThreads, false>;
+    if constexpr (!kF64) {
+        if (threads == kBeadThreadsFew) k = team ? k_beads<S, kBeadThreadsFew, true> : k_beads<S, kBeadThreadsFew, false>;
+        if (threads == kBeadThreadsMid) k = k_beads<S, kBeadThreadsMid, false>;
+    }
     return cudaLaunchKernelEx(&cfg, k, inst_d, blist, (const S *)pool, tab[0], tab[1], p0, p1, mask_write, gparity,
                               advance, wait_first, counters, ex, status);
 }
@@ -1227,7 +1232,7 @@ int team_limit() {
 
 void prepare_bead_kernels() { (void)team_limit(); }
 
-cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, int nb_total, int each, int ntiles,
+cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, int nb_total, int each, int box, int ntiles,
                          const void *pool, const BeadTab tab[2], const PhiTab phi[2], unsigned *mask_write, int gparity, int advance,
                          unsigned *counters, int pdl, cudaStream_t st, BeadExport ex, unsigned *status) {
     if (nb_total <= 0) return cudaSuccess;
@@ -1246,11 +1251,30 @@ cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, i
         while (2 * parts <= kBeadParts && 2 * parts * nb_total <= 2 * sms) parts *= 2;
     // A sweep of up to a few waves has room for the bead CTAs beside it: they
     // list their supports while it runs.  They enter a longer sweep's SMs
-    // only as it drains; then the next sweep's release comes first
+    // only as it drains; then the next sweep's release comes first.  us a
+    // step, listing first / waiting first, FP32 (FP16): 2048 tiles 12.0 / 14.9
+    // (12.4 / 15.4), 4096 13.5 / 16.3 (13.0 / 16.7), 8192 23.3 / 22.4 (22.2 /
+    // 19.9 with one cell a thread, 16.6 / 17.9 with two), 16384 45.2 / 43.6
+    // (31.2 / 29.1)
     const int wait_first = ntiles > kEarlyListTiles ? 1 : 0;
     // Every instance of the launch has `each` beads (0: not all the same): its
     // CTAs form a cluster where there is room beside the sweep for one
     const bool team = precision != 0 && few && !wait_first && advance && !ex.ring && each >= 1 && each <= team_limit();
+    // Threads a CTA, us a step.  A short list beside a sweep of up to a few
+    // waves, 512 against 256: 1024 x 256 and 20 beads of a = 2 10.98 / 12.2,
+    // of a = 4 10.8 / 11.9, 160 x 160 and one bead of a 37 x 37 box 9.2 /
+    // 10.9; where the sweep is no more than two tiles an SM and the box
+    // small, 333 x 171 and 27 beads, 10.3 / 9.7.  Beside a long sweep the
+    // narrower CTAs leave it more room: 4096 x 1024 FP16 27.05 / 26.64, FP32
+    // 43.86 / 43.57 (128 threads: 26.89 and 44.85).  FP64, bound by its
+    // instructions, 512 / 256 / 128: 80 x 40 27.8 / 26.5 / 26.1, 200 x 100
+    // 256 / 128 26.2 / 25.6, 4096 x 1024 498 / 486.1 / 485.4.  Long lists: 128
+    // (six CTAs an SM).
+    int threads = kBeadThreads;
+    if (precision != 0 && few) {
+        const bool narrow = wait_first || (!team && box < kWideBox && ntiles <= 2 * sms);
+        threads = narrow ? kBeadThreadsMid : kBeadThreadsFew;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nb_total * parts);
     cfg.stream = st;
@@ -1270,13 +1294,13 @@ cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, i
     cfg.numAttrs = na;
     switch (precision) {
         case 0:
-            return launch_beads_t<double>(cfg, few, team, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
+            return launch_beads_t<double>(cfg, threads, team, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
                                           wait_first, counters, ex, status);
         case 1:
-            return launch_beads_t<float>(cfg, few, team, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
+            return launch_beads_t<float>(cfg, threads, team, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
                                          wait_first, counters, ex, status);
         case 2:
-            return launch_beads_t<__half>(cfg, few, team, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
+            return launch_beads_t<__half>(cfg, threads, team, inst_d, blist, pool, tab, phi, mask_write, gparity, advance,
                                           wait_first, counters, ex, status);
     }
     return cudaErrorInvalidValue;

@@ -9,12 +9,12 @@ namespace fpd {
 
 constexpr int kTileX = 32;       // lattice tile: 32 x 8 cells, one thread each
 constexpr int kTileY = 8;
-constexpr int kSplitCtas = 304, kSplitCtas64 = 608;  // a sweep's tiles are split by rows up to this many CTAs
+constexpr int kSplitCtas = 304, kSplitCtas64 = 608;  // a sweep's tiles are split by rows up to this many CTAs: row_split
 constexpr int kMaxBeads = 256;   // beads per instance (shared-memory tables)
 constexpr int kBeadThreads = 128;  // per bead CTA: more beads resident at once (batched sweep +9 %)
-constexpr int kBeadThreadsFew = 512;  // per bead CTA when the beads fit on the SMs one per SM
-constexpr int kBeadThreadsFew64 = 256;  // the same, FP64
-constexpr int kEarlyListTiles = 4096;  // longest sweep (tiles) whose bead phase lists its supports before waiting
+constexpr int kBeadThreadsMid = 256, kBeadThreadsFew = 512;  // FP32, FP16, the beads fit on the SMs one per SM: launch_beads
+constexpr int kWideBox = 900;  // support box (phi_cells) too large for kBeadThreadsMid beside a short sweep
+constexpr int kEarlyListTiles = 4096;  // longest sweep (tiles) whose bead phase lists its supports before waiting: launch_beads
 constexpr int kTeamBeads = 16;  // most beads of an instance whose CTAs form a cluster
 constexpr int kBeadParts = 8;    // CTAs a bead's cells are split over at most (FP64, short bead lists)
 constexpr int kGraphSteps = 32;  // time steps per captured graph chunk
@@ -87,16 +87,20 @@ cudaError_t launch_lattice(int precision, const Inst *inst_d, const Inst &inst_h
 // (blist[i] = (2 slot + par_xor, global bead index, the instance's first bead
 // and bead count); NULL = instance 0, bead i; every bead of an instance must
 // be in the same launch, side by side).  each: beads of every instance of the
-// launch, 0 if not all the same.  ntiles: tiles of the sweep before it.  With the instance's
+// launch, 0 if not all the same.  box: phi_cells of the instance with the
+// largest supports.  ntiles: tiles of the sweep before it.  With the instance's
 // step parity p = gparity ^ par_xor it reads table p ^ 1 and writes table p
 // (tab0 / tab1); advance = 0 only computes S and F of table p from its own R
 // (initialisation).  Every bead ORs its bit into the mask of each lattice
 // tile its support reaches (mask_write, zeroed beforehand).
 // pdl = 1 launches the bead phase as a programmatic dependent of the
-// previous sweep: it waits for that sweep first thing and releases the next
-// sweep at once, so the next sweep's unmarked tiles overlap the whole phase.
+// previous sweep.  Up to kEarlyListTiles tiles it lists its supports beside
+// that sweep and then waits for it; otherwise it waits first thing.  It then
+// releases the next sweep at once, so that sweep's unmarked tiles overlap the
+// rest of the phase.
 // Per-step export of a single instance's finished bead table to host
-// memory (ring == nullptr: none): the instance's last CTA writes R_x, R_y,
+// memory (ring == nullptr: none; with a ring no instance is a cluster): the
+// instance's last CTA writes R_x, R_y,
 // V_x, V_y, F_x, F_y, S (nb doubles each) after kExportHeader doubles into
 // slot k % slots of the ring (stride doubles a slot, device address of
 // mapped page-locked memory), then k + 1 into the slot's first 64-bit word,
@@ -111,11 +115,11 @@ struct BeadExport {
 // prepare_bead_kernels: kernel attributes on the current device, set when an
 // instance or batch is created (outside any stream capture).
 void prepare_bead_kernels();
-// status: per-instance status words (indexed by instance slot), where the
-// instance's last CTA sets kFlagFastBead (and kFlagNonFinite) when a bead
-// velocity component reaches kFastBead in magnitude (or is not finite), and
-// marks every tile of a flagged instance in mask_write; NULL: not checked.
-cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, int nb_total, int each, int ntiles,
+// status: per-instance status words (indexed by instance slot), where a
+// bead's CTA sets kFlagFastBead (and kFlagNonFinite) when a bead
+// velocity component reaches kFastBead in magnitude (or is not finite); the
+// forces' CTA marks every tile of a flagged instance in mask_write; NULL: not checked.
+cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, int nb_total, int each, int box, int ntiles,
                          const void *pool, const BeadTab tab[2], const PhiTab phi[2], unsigned *mask_write,
                          int gparity, int advance, unsigned *counters, int pdl, cudaStream_t st, BeadExport ex = BeadExport{},
                          unsigned *status = nullptr);

@@ -436,9 +436,8 @@ __device__ __forceinline__ int tile_order(int b, int n, int parity) { return (pa
 // that a CTA's registers keep in flight: each CTA has the populations of the
 // tile kAheadOne CTAs on brought to L2 by one bulk prefetch (its rows are
 // contiguous in its strip).  2048 x 2048, FP16, variant 1: 29.7 -> 27.2 us a
-// step (DRAM 5.08 -> 5.55 TB/s of the bytes it cannot do without).  1368 CTAs
-// on: the same; 684: 26.9 against 26.5 where these two take 26.5.  By one
-// thread.
+// step (5.08 -> 5.55 TB/s of the bytes it cannot do without).  In one session,
+// at 684, 1368 and 2736 CTAs: 26.9, 26.5 and 26.4, without 29.3.  By one thread.
 constexpr unsigned kAheadOne = 2736;
 template <class S>
 __device__ __forceinline__ void prefetch_ahead(const Inst &I, const S *__restrict__ pool, const int parity) {
@@ -1347,8 +1346,15 @@ static cudaError_t launch_staged(const Inst &I, void *pool, BeadTab tab, const S
 }
 
 // CTAs a tile of the single-lattice sweep is split into by rows (variants 0
-// and 1): a lattice of few tiles would leave most SMs idle.
-template <class S> static int row_split(int ntiles) {
+// and 1): a lattice of few tiles would leave most SMs idle.  us a step, whole
+// tiles / split.  FP64 without beads: 10 to 75 tiles 10.3 / 5.8 to 6.2, 140
+// 10.3 / 10.2, 200 19.1 / 14.8, 300 19.1 / 18.8; up to twice kSplitCtas64
+// CTAs: 560 tiles 36.3 / 36.0, the rest the same.  FP32 with beads (their
+// tiles' overlay): 100 tiles and a wide bead 9.35 / 9.23, 91 tiles and ten
+// beads 7.25 / 7.30; without, 10 tiles 1.70 / 1.93, 300 at 608 CTAs 2.20 / 2.48.
+template <class S> static int row_split(const Inst &I) {
+    const int ntiles = I.ntx * I.nty;
+    if (!std::is_same<S, double>::value && I.nb == 0) return 1;
     int sp = 1;
     while (sp < kTileY && 2 * sp * ntiles <= (std::is_same<S, double>::value ? kSplitCtas64 : kSplitCtas)) sp *= 2;
     return sp;
@@ -1390,7 +1396,7 @@ static cudaError_t lattice_v(int variant, const Inst &I, void *pool, BeadTab tab
     const auto pt = sweep_arg<S>(phi, I);
     cudaLaunchAttribute attr[1];
     const dim3 grid(I.ntx, I.nty);
-    const int sp = row_split<S>(I.ntx * I.nty), rows = kTileY / sp;
+    const int sp = row_split<S>(I), rows = kTileY / sp;
     const dim3 split(I.ntx, I.nty, sp);
     const int ec = after_beads ? mk.early_cold : 0;
     const int ahead = prefetch_one<S>(I, pool);
