@@ -228,6 +228,15 @@ __device__ __forceinline__ float min_image_yf(const Inst &I, float d) {
     return I.periodic_y ? d - (float)I.ny * rintf(d * I.f_inv_ny) : d;
 }
 
+// a - b of two places in [0, L] to the nearest periodic image.  The period
+// comes off the larger of them, which is exact (it is between L / 2 and L), so
+// that a difference across the edge is rounded at its own size and not at L's
+// (an ulp of 65536 is 1/128 of a cell).
+__device__ __forceinline__ float edge_diff(float a, float b, float L) {
+    const float d = a - b;
+    return d > 0.5f * L ? (a - L) - b : (d < -0.5f * L ? a - (b - L) : d);
+}
+
 // A double as a pair of floats, h + l equal to it within 2^-48 of its size,
 // from its bits: the conversions and subtractions are FP64 instructions, a
 // chain of which took the last CTA about a microsecond.  Sizes outside
@@ -599,13 +608,13 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         int fiber = 0;         // first bead of its fiber
         for (int q0 = 0; q0 < nb; q0 += 32) {
             const int q = q0 + lane, gq = first + q;
-            float dx = 0.f, dy = 0.f;
+            float qx = 0.f, qy = 0.f;
             Neighbour<R> nbr{};
             int4 qbox = make_int4(0, 0, 0, 0);
             if (q < nb) {
-                dx = xh - __ldcg(told.xh + gq);
+                qx = __ldcg(told.xh + gq);
                 const float lx = xl - __ldcg(told.xl + gq);
-                dy = yh - __ldcg(told.yh + gq);
+                qy = __ldcg(told.yh + gq);
                 const float ly = yl - __ldcg(told.yl + gq);
                 if constexpr (kF64) {
                     if (pold.box) qbox = __ldcg(pold.box + gq);
@@ -621,11 +630,9 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
                 }
             }
             if (q0 == 0) record_here();
-            // nearest image of the bead from bead q: the high parts' image
-            // shift is a whole number of cells, removed exactly
-            const float fnx = (float)I.nx, fny = (float)I.ny;
-            dx -= fnx * rintf(dx * I.f_inv_nx);
-            if (I.periodic_y) dy -= fny * rintf(dy * I.f_inv_ny);
+            // nearest image of the bead from bead q, by the high parts
+            const float dx = edge_diff(xh, qx, (float)I.nx);
+            const float dy = I.periodic_y ? edge_diff(yh, qy, (float)I.ny) : yh - qy;
             const float d2 = dx * dx + dy * dy, reach = 2.0f * I.f_rcut + 1.0f;
             const bool hit = q < nb && (d2 < reach * reach || gq == b);  // itself even if not finite
             const unsigned m = __ballot_sync(0xffffffffu, hit);

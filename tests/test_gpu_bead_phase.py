@@ -1,0 +1,60 @@
+"""Bead phase at the places where its FP32 arithmetic or its lists could go
+wrong, against FP64 references: neighbours across a periodic edge.
+"""
+import math
+import os
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2212_14153_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+THREADS = min(16, os.cpu_count() or 1)
+
+
+@pytest.fixture(scope="module")
+def fpd():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2212_14153_gb300 import build, fpd as binding
+    build.build()
+    return binding
+
+
+def box(nx, ny, a, xi, centres, n_beads, force, precision, **kw):
+    """Beads pushed through fluid at rest in a doubly periodic box."""
+    nb = n_beads * len(centres)
+    cfg = dict(nx=nx, ny=ny, u_bottom=0.0, u_top=0.0, nu_f=1.0 / 6.0, re=1.0, visc_ratio=50.0, xi=xi, a=a,
+               n_beads=n_beads, n_fibers=len(centres), k_s=-1.0, k_b=0.0, stiffness_K=0.0, k_ev=-1.0, phi_cut=8.0,
+               collision=0, s_e=1.64, s_eps=1.54, s_q=1.9, init_couette=0, periodic_y=1, bead_fx=force[0],
+               bead_fy=force[1], gx=-force[0] * nb / (nx * ny), gy=-force[1] * nb / (nx * ny), centres=centres,
+               theta0=[0.0] * len(centres), precision=precision)
+    cfg.update(kw)
+    return cfg
+
+
+@pytest.mark.parametrize("axis", [0, 1])
+def test_neighbours_across_the_edge_of_a_wide_lattice_vs_oracle(fpd, axis):
+    # a fiber over the periodic edge of 65536 columns (or 65535 rows), whose FP32
+    # positions have an ulp of 2^-8: the offset between beads on either side
+    # must not be rounded there.  An offset of up to 16 cells rounded to FP32
+    # (4.8e-7) twice, at a slope of phi of 1 / (2 xi) = 1 / 3, and phi's own
+    # 1.5e-7 make an error below 5e-7 a neighbour, of which there are four; V is
+    # a mean of these.  The beads on the right lie 0.45 of an ulp of the left
+    # ones' positions off that grid.
+    n = (65536, 64) if axis == 0 else (64, 65535)
+    at = 2.0 + 0.45 / 256.0
+    centre = [at, 32.2] if axis == 0 else [32.2, at]
+    cfg = box(*n, 2.0, 1.5, [centre], 5, (1e-3, 7e-4), 1, theta0=[axis * math.pi / 2])
+    sim, ref = fpd.Simulation(cfg), oracle.Sim(dict(cfg, precision=0, threads=THREADS))
+    sim.step(2)  # one bead phase: the force density is a third of V
+    ref.step(2)
+    V, rV = sim.beads()[1], ref.beads()[1]
+    sim.close()
+    e = np.abs(V - rV).max() / np.abs(rV).max()
+    print(f"axis {axis}: V {e:.1e}")
+    assert e < 1e-5
