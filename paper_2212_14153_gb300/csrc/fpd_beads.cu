@@ -55,17 +55,19 @@ namespace {
 // Sum of n terms x with |x| < 2^ex as integers x 2^s, s = kTop - ex -
 // ceil(log2(n + 1)): no sum can overflow, every addition is exact and order
 // does not matter.  One term is rounded at 2^-(s + 1): for velocities (ex =
-// kVelBits) over 784 box cells at 2^-41 (float) and 2^-117 (double), below a
-// float term's own unit roundoff for velocities above 1e-5 and, with the few
-// hundred roundings of a sum averaging out, below the sum's above 1e-6.  A
-// caller that meets a larger term (mag) repeats the sum with a larger ex.
+// kVelBits at first) over 784 box cells at 2^-41 (float) and 2^-117 (double).
+// Where the largest term (mag) is so small that this is more than its own half
+// ulp (below 2^-16 cells a step, 2^-63 in double), and where it does not fit
+// below 2^ex, the caller repeats the sum with the ex that the largest term
+// needs, so that a sum's relative accuracy does not depend on the speed.
 constexpr int kVelBits = 0;
+constexpr int kAgain = 4096;  // "once more with ex" is handed round as kAgain + ex, above zero
 constexpr float kEarlyMove = 0.499f;
 static_assert(kEarlyMove < kFastBead, "faster beads are judged by their FP64 velocity");
 template <class R> struct Fix;
 template <> struct Fix<float> {
     using T = long long;
-    static constexpr int kTop = 50;
+    static constexpr int kTop = 50, kMantissa = 24, kLowest = -72;  // kLowest: smallest ex, |s| stays below 126
     static __device__ __forceinline__ T term(float x, int s) {
         return __float2ll_rn(x * __int_as_float((s + 127) << 23));  // |s| < 126: x scaled by 2^s
     }
@@ -82,7 +84,7 @@ template <> struct Fix<float> {
 };
 template <> struct Fix<double> {
     using T = __int128;
-    static constexpr int kTop = 126;
+    static constexpr int kTop = 126, kMantissa = 53, kLowest = -800;
     static __device__ __forceinline__ T term(double x, int s) {
         // from the bits: no FP64 instruction
         const unsigned long long u = (unsigned long long)__double_as_longlong(x);
@@ -840,10 +842,17 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             // (2^-25) is far below the box offsets' own
             if (w == 0) {
                 const int need = F::need(mx);
-                int state = need > bound && F::finite(mx) ? need : -1;  // > 0: once more with this bound
+                // a term of magnitude 2^kVelBits or more (a diverging run), or
+                // all of them so small that they are rounded here: once more
+                const bool slow = bound == kVelBits && mx != 0u && need < kVelBits - (F::kTop - F::kMantissa - bit_length(ncell));
+                int state = (need > bound || slow) && F::finite(mx) ? kAgain + max(need, F::kLowest) : -1;
                 if constexpr (!kF64) {
-                    const float vx = (float)ax * s_unit_f, vy = (float)ay * s_unit_f;
-                    if (state < 0 && bound == kVelBits && F::finite(mx) && fabsf(vx) < kEarlyMove && fabsf(vy) < kEarlyMove &&
+                    float vx = (float)ax * s_unit_f, vy = (float)ay * s_unit_f;
+                    if (bound < kVelBits) {
+                        const float f = __int_as_float((bound - kVelBits + 127) << 23);
+                        vx *= f, vy *= f;
+                    }
+                    if (state < 0 && bound <= kVelBits && F::finite(mx) && fabsf(vx) < kEarlyMove && fabsf(vy) < kEarlyMove &&
                         !far_off(xh, yh)) {
                         state = 0;
                         if (lane < 2)
@@ -856,10 +865,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             __syncthreads();
             const int state = s_state;
             if (state > 0) {
-                // a term of magnitude 2^kVelBits or more (a diverging run): once
-                // more with room for it
-                bound = state;
-                n = make_list(c_lo, min(c_lo + kCap, c_hi));
+                bound = state - kAgain;
+                if (c_hi - c_lo > kCap) n = make_list(c_lo, min(c_lo + kCap, c_hi));  // else it is still in place
                 continue;
             }
             if constexpr (kTeam) cluster_wait();  // the cluster's CTAs all run

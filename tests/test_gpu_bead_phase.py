@@ -1,5 +1,5 @@
-"""Bead phase at the places where its FP32 arithmetic or its lists could go
-wrong, against FP64 references: neighbours across a periodic edge.
+"""Bead phase at the places where its FP32 arithmetic or its lists could go wrong,
+against FP64 references: neighbours across a periodic edge, slow beads.
 """
 import math
 import os
@@ -57,4 +57,21 @@ def test_neighbours_across_the_edge_of_a_wide_lattice_vs_oracle(fpd, axis):
     sim.close()
     e = np.abs(V - rV).max() / np.abs(rV).max()
     print(f"axis {axis}: V {e:.1e}")
+    assert e < 1e-5
+
+
+@pytest.mark.parametrize("force", [1e-4, 1e-8, 1e-12, 1e-18])
+def test_slow_beads_keep_their_relative_accuracy(fpd, force):
+    # the flow a weak force drives is linear in it: the FP32 path keeps the
+    # relative accuracy it has at ordinary speeds (FP32 arithmetic over 20
+    # steps: below 1e-5, as against the oracle) down to any speed
+    cfg = box(48, 40, 2.0, 0.5, [[47.2, 12.7]], 1, (force, -0.6 * force), 1)
+    V = []
+    for precision in (0, 1):
+        sim = fpd.Simulation(dict(cfg, precision=precision))
+        sim.step(20)
+        V.append(sim.beads()[1][0])
+        sim.close()
+    e = np.abs(V[1] - V[0]).max() / np.abs(V[0]).max()
+    print(f"force {force:.0e}: V {np.abs(V[0]).max():.1e}, error {e:.1e}")
     assert e < 1e-5
