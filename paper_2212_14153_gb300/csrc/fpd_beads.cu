@@ -441,7 +441,9 @@ __device__ __forceinline__ void support_axis(const Inst &I, int ax, float h, flo
         a = max(a, 0);
         b = min(b, L - 1);
     } else if (b - a + 1 >= L) {
-        a = (int)floorf(h - 0.5f * (float)L);
+        // the whole axis: the L columns (rows) whose centres are the nearest
+        // images, as the sweep takes them (phi is evaluated at these offsets)
+        a = (int)ceilf((h - 0.5f - 0.5f * (float)L) + l);
         b = a + L - 1;
     }
     n = max(b - a + 1, 0);

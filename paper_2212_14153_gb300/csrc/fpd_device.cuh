@@ -583,20 +583,20 @@ __device__ __forceinline__ Box support_box(const Inst &I, double Rx, double Ry) 
         int xlo = (int)floorf(rx - rc - 0.5f) - 1;
         int xhi = (int)ceilf(rx + rc - 0.5f) + 1;
         if (xhi - xlo + 1 >= I.nx) {
-            xlo = (int)floorf(rx - 0.5f * (float)I.nx);
+            xlo = (int)ceilf(rx - 0.5f - 0.5f * (float)I.nx);  // nearest images
             xhi = xlo + I.nx - 1;
         }
-        if (!box_rows(I, ylo, yhi, (long long)floorf(ry - 0.5f * (float)I.ny), b)) return b;
+        if (!box_rows(I, ylo, yhi, (long long)ceilf(ry - 0.5f - 0.5f * (float)I.ny), b)) return b;
         b.iu = (double)xlo;
         b.i0 = ((xlo % I.nx) + I.nx) % I.nx;  // in [0, nx)
         b.w = xhi - xlo + 1;
         return b;
     }
     const long long ylo = (long long)floor(Ry - I.rcut - 0.5) - 1, yhi = (long long)ceil(Ry + I.rcut - 0.5) + 1;
-    if (!box_rows(I, ylo, yhi, (long long)floor(Ry - 0.5 * I.ny), b)) return b;
+    if (!box_rows(I, ylo, yhi, (long long)ceil(Ry - 0.5 - 0.5 * I.ny), b)) return b;
     const double xl = floor(Rx - I.rcut - 0.5) - 1.0, xh = ceil(Rx + I.rcut - 0.5) + 1.0;
     if (xh - xl + 1.0 >= (double)I.nx) {
-        const double x0 = floor(Rx - 0.5 * I.nx);
+        const double x0 = ceil(Rx - 0.5 - 0.5 * I.nx);
         b.iu = x0;
         const long long xi = (long long)x0;
         b.i0 = (int)(((xi % I.nx) + I.nx) % I.nx);

@@ -1,5 +1,6 @@
 """Bead phase at the places where its FP32 arithmetic or its lists could go wrong,
-against FP64 references: neighbours across a periodic edge, slow beads.
+against FP64 references: neighbours across a periodic edge, slow beads,
+supports that span a periodic box.
 """
 import math
 import os
@@ -75,3 +76,28 @@ def test_slow_beads_keep_their_relative_accuracy(fpd, force):
     e = np.abs(V[1] - V[0]).max() / np.abs(V[0]).max()
     print(f"force {force:.0e}: V {np.abs(V[0]).max():.1e}, error {e:.1e}")
     assert e < 1e-5
+
+
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("centre", [[10.0, 10.2], [19.9, 0.4], [3.5, 14.8]])
+def test_support_that_spans_a_periodic_box(fpd, precision, centre):
+    # S = sum phi over the nearest images where phi is still 5e-3 half a box
+    # away, of a bead carried along by a uniform flow.  400 values of phi with
+    # errors of at most 4e-7 against S = 114 in FP32
+    L, a, xi = 20, 6.0, 1.5
+    # the wall speeds only set FP16's scale here: y is periodic
+    cfg = box(L, L, a, xi, [centre], 1, (0.0, 0.0), precision, visc_ratio=1.0, u_bottom=-0.2, u_top=0.2)
+    sim = fpd.Simulation(cfg)
+    f = oracle.feq(1.0, 0.31, -0.17)[:, None, None]
+    sim.set_populations(np.ascontiguousarray(np.broadcast_to(f, (9, L, L))))
+    c = np.arange(L) + 0.5
+    for n in range(6):
+        R, V, _, S = sim.beads()
+        assert n < 2 or abs(V[0, 0]) > 0.1
+        d = [x - L * np.floor(x / L + 0.5) for x in (c - R[0, 0], c - R[0, 1])]
+        r = np.hypot(d[0][None, :], d[1][:, None])
+        want = np.where(r < a + 8.0 * xi, 0.5 * (np.tanh((a - r) / xi) + 1.0), 0.0).sum()
+        print(f"precision {precision}, step {n}: S {S[0]:.6f}, error {abs(S[0] / want - 1):.1e}")
+        assert abs(S[0] / want - 1) < (1e-13 if precision == 0 else 2e-6)
+        sim.step(1)
+    sim.close()
