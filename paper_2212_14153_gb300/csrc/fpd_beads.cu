@@ -241,8 +241,11 @@ __device__ __forceinline__ float edge_diff(float a, float b, float L) {
 
 // A double as a pair of floats, h + l equal to it within 2^-48 of its size,
 // from its bits: the conversions and subtractions are FP64 instructions, a
-// chain of which took the last CTA about a microsecond.  Sizes outside
-// [2^-74, 2^127) do not occur for positions in use: 0 below, NaN above.
+// chain of which took the last CTA about a microsecond.  Taken of a bead's
+// position less that of its fiber's first bead, so that the pair is as good
+// wherever the fiber has drifted (a fiber's length times 2^-48; the unwrapped
+// position's after 4096 periods of 128 columns: 2e-9 of a cell).  Sizes outside
+// [2^-74, 2^127) do not occur in use: 0 below, NaN above.
 __device__ __forceinline__ float2 split(double x) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
     const int e = (int)(u >> 52) & 0x7ff;
@@ -333,8 +336,6 @@ __device__ __forceinline__ void screen_close(const Inst &I, const float *Xf, con
     }
 }
 
-__device__ __forceinline__ double place(double r) { return r; }
-__device__ __forceinline__ double place(float2 r) { return (double)r.x + (double)r.y; }
 // The same for bead q of at most 32, lane p holding bead p's place.
 __device__ __forceinline__ unsigned close_beads(const Inst &I, float x, float y, int q) {
     const int N = I.n_beads, p = threadIdx.x & 31, lo = q / N * N;
@@ -347,14 +348,14 @@ __device__ __forceinline__ unsigned close_beads(const Inst &I, float x, float y,
 
 // Excluded volume on bead q along axis ax (0 x, 1 y) from the beads in its
 // nw candidate words, in bead order; r: interleaved x, y positions.
-template <class R, class Place>
-__device__ __noinline__ R close_force(const Inst &I, const Place *r, const unsigned *cand, int nw, int q, int ax) {
+template <class R>
+__device__ __noinline__ R close_force(const Inst &I, const double *r, const unsigned *cand, int nw, int q, int ax) {
     R f = (R)0;
     for (int c = 0; c < nw; ++c)
         for (unsigned bits = cand[c]; bits; bits &= bits - 1u) {
             const int p = 32 * c + __ffs(bits) - 1;
-            const double dx = min_image(place(r[2 * q]) - place(r[2 * p]), I.nx, I.f_inv_nx);
-            const double dy = min_image_y(I, place(r[2 * q + 1]) - place(r[2 * p + 1]));
+            const double dx = min_image(r[2 * q] - r[2 * p], I.nx, I.f_inv_nx);
+            const double dy = min_image_y(I, r[2 * q + 1] - r[2 * p + 1]);
             if constexpr (std::is_same<R, double>::value) {
                 const double d = sqrt(dx * dx + dy * dy);
                 if (d < I.l0 && d > 0.0) f += I.k_ev * (I.l0 - d) / d * (ax ? dy : dx);
@@ -390,10 +391,14 @@ template <class R, int NT> struct ListCap {
 };
 
 // The last CTA's view of its instance, in the shared memory the list took;
-// x and y of a bead or segment side by side.
+// x and y of a bead or segment side by side.  FP32 paths: the segments are
+// taken from rel, the positions relative to the first bead of their fiber in
+// pairs of floats; pos takes its place for the excluded volume.
 template <class R> struct ForceShared {
-    using Place = typename std::conditional<std::is_same<R, double>::value, double, float2>::type;  // FP32 paths: split
-    Place r[2 * kMaxBeads];
+    union {
+        double pos[2 * kMaxBeads];
+        float2 rel[2 * kMaxBeads];
+    };
     R S[kMaxBeads], t[2 * kMaxBeads], pull[2 * kMaxBeads], len[kMaxBeads], str[kMaxBeads];
     float xf[kMaxBeads], yf[kMaxBeads];
     unsigned cand[kMaxBeads * (kMaxBeads / 32)];
@@ -1008,8 +1013,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         }
     }
     if constexpr (kTeam) {
+        const int q = b - first, N = I.n_beads, i0 = q - q / N * N, head = (lane >> 1) / N * N;
         cluster_wait();  // every bead's place is here, and its status bits are set
-        const int q = b - first, N = I.n_beads, i0 = q - q / N * N;
         // fast-bead guard, as below
         if (w != 0) {
             if (q == 0 && status && (__ldcg(status + ii) & kFlagFastBead))
@@ -1017,7 +1022,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
                     atomicOr(mask_write + (I.tile_base + t) * I.mask_words, 1u);
             return;
         }
-        if (lane < 2 * nb) s_place[lane] = split(s_peer[lane >> 1][lane & 1]);
+        if (lane < 2 * nb) s_place[lane] = split(s_peer[lane >> 1][lane & 1] - s_peer[head][lane & 1]);
         const bool crowd = I.k_ev != 0.0 && __any_sync(0xffffffffu, lane < nb && s_near[lane] != 0ull);
         __syncwarp();
         // lanes 2 m + ax, m < 4: axis ax of segment q - 2 + m of the fiber
@@ -1034,10 +1039,10 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         if (i0 > 0) f -= before;
         if (i0 < N - 1) f += pull;
         if (crowd) {
-            const float x = (float)(place(s_place[2 * (lane < nb ? lane : 0)]) - place(s_place[0]));
-            const float y = (float)(place(s_place[2 * (lane < nb ? lane : 0) + 1]) - place(s_place[1]));
+            const int p = lane < nb ? lane : 0;
+            const float x = (float)(s_peer[p][0] - s_peer[0][0]), y = (float)(s_peer[p][1] - s_peer[0][1]);
             const unsigned cand = close_beads(I, x, y, q);
-            f += close_force<float>(I, s_place, &cand, 1, q, ax);
+            f += close_force<float>(I, &s_peer[0][0], &cand, 1, q, ax);
         }
         f += ax ? I.f_ext_fy : I.f_ext_fx;
         if ((lane >> 1) == 2) {
@@ -1063,10 +1068,13 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     // warp 64 cycles each whatever its lanes do, so x and y share them)
     const int items = 2 * nb, N = I.n_beads;
     const float inv_n = 1.0f / (float)N;
+    // place of bead q < 256 within its fiber
+    auto in_fiber = [&](int q) { return q - N * (int)(((float)q + 0.5f) * inv_n); };
     for (int k = tid; k < items; k += NT) {
-        const double x = nb == 1 ? s_R[k] : __ldcg(((k & 1) ? tnew.Ry : tnew.Rx) + first + (k >> 1));
-        if constexpr (kF64) fs.r[k] = x;
-        else fs.r[k] = split(x);
+        const double *r = ((k & 1) ? tnew.Ry : tnew.Rx) + first;
+        const double x = nb == 1 ? s_R[k] : __ldcg(r + (k >> 1));
+        if constexpr (kF64) fs.pos[k] = x;
+        else fs.rel[k] = nb == 1 ? make_float2(0.f, 0.f) : split(x - __ldcg(r + (k >> 1) - in_fiber(k >> 1)));
         if (!(k & 1)) fs.S[k >> 1] = (R)(nb == 1 ? s_S : __ldcg(tnew.S + first + (k >> 1)));
     }
     __syncthreads();
@@ -1077,14 +1085,13 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     // phase's masks, so that the next sweeps wait on all of them
     if (st_now & kFlagFastBead)
         for (int t = tid; t < I.ntx * I.nty; t += NT) atomicOr(mask_write + (I.tile_base + t) * I.mask_words, 1u);
-    // place of bead q < 256 within its fiber
-    auto in_fiber = [&](int q) { return q - N * (int)(((float)q + 0.5f) * inv_n); };
     // Segment q (bead q to q + 1 of the fiber): length, tangent, stretch
     for (int k0 = 0; k0 < items; k0 += NT) {
         const int k = k0 + tid, q = k >> 1;
         const bool seg = k < items && in_fiber(q) < N - 1;
         R L, t, str;
-        segment_axis(I, fs.r[seg ? k : 0], fs.r[seg ? k + 2 : 1], L, t, str);
+        if constexpr (kF64) segment_axis(I, fs.pos[seg ? k : 0], fs.pos[seg ? k + 2 : 1], L, t, str);
+        else segment_axis(I, fs.rel[seg ? k : 0], fs.rel[seg ? k + 2 : 1], L, t, str);
         if (seg) {
             fs.t[k] = t;
             if (!(k & 1)) {
@@ -1094,9 +1101,14 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         }
     }
     if (crowd) {
+        if constexpr (!kF64) {
+            __syncthreads();  // the segments no longer read rel
+            for (int k = tid; k < items; k += NT) fs.pos[k] = __ldcg(((k & 1) ? tnew.Ry : tnew.Rx) + first + (k >> 1));
+            __syncthreads();
+        }
         for (int q = tid; q < nb; q += NT) {
-            fs.xf[q] = (float)(place(fs.r[2 * q]) - place(fs.r[0]));
-            fs.yf[q] = (float)(place(fs.r[2 * q + 1]) - place(fs.r[1]));
+            fs.xf[q] = (float)(fs.pos[2 * q] - fs.pos[0]);
+            fs.yf[q] = (float)(fs.pos[2 * q + 1] - fs.pos[1]);
         }
         __syncthreads();
         screen_close<NW>(I, fs.xf, fs.yf, fs.cand);
@@ -1121,7 +1133,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         R f = (R)0;
         if (i0 > 0) f -= fs.pull[k - 2];
         if (i0 < N - 1) f += fs.pull[k];
-        if (crowd) f += close_force<R>(I, fs.r, fs.cand + q * ((nb + 31) / 32), (nb + 31) / 32, q, ax);
+        if (crowd) f += close_force<R>(I, fs.pos, fs.cand + q * ((nb + 31) / 32), (nb + 31) / 32, q, ax);
         // constant external force F_0 (driven particle, Sec. 3.2)
         if constexpr (kF64) f += ax ? I.ext_fy : I.ext_fx;
         else f += ax ? I.f_ext_fy : I.f_ext_fx;

@@ -1,6 +1,6 @@
 """Bead phase at the places where its FP32 arithmetic or its lists could go wrong,
 against FP64 references: neighbours across a periodic edge, slow beads,
-supports that span a periodic box.
+supports that span a periodic box, fibers that have drifted far.
 """
 import math
 import os
@@ -100,4 +100,31 @@ def test_support_that_spans_a_periodic_box(fpd, precision, centre):
         print(f"precision {precision}, step {n}: S {S[0]:.6f}, error {abs(S[0] / want - 1):.1e}")
         assert abs(S[0] / want - 1) < (1e-13 if precision == 0 else 2e-6)
         sim.step(1)
+    sim.close()
+
+
+@pytest.mark.parametrize("n_beads", [6, 20])  # forces in a cluster; by the last CTA
+@pytest.mark.parametrize("periods", [0, 4096, 16384])
+def test_forces_do_not_depend_on_how_far_a_fiber_has_drifted(fpd, n_beads, periods):
+    # stiff springs stretched by up to 1e-4 after any number of passes over the
+    # periodic edge: the FP32 paths' force against the FP64 one at the same
+    # positions.  Roundings of FP32 (6e-8 each): the stretch from a difference of
+    # squares, a product with the tangent and a sum of two pulls, six or so.
+    rng = np.random.default_rng(n_beads)
+    nx, l0 = 128, 4.0
+    d = l0 + rng.uniform(-1e-4, 1e-4, n_beads)
+    t = 0.3 + 0.02 * np.arange(n_beads)
+    xy = np.stack([20.0 + np.cumsum(d * np.cos(t)), 8.0 + np.cumsum(d * np.sin(t))], 1)
+    xy = np.round(xy * 2.0 ** 24) / 2.0 ** 24  # exact after the shift as well
+    xy[:, 0] += periods * nx
+    cfg = box(nx, 128, 2.0, 0.5, [[0.0, 0.0]], n_beads, (0.0, 0.0), 1, bead_xy=xy, k_ev=0.0)
+    sim = fpd.Simulation(cfg)
+    k_s = 0.25 * math.pi * 4.0 * l0 ** 2
+    for steps in (0, 3):
+        sim.step(steps)
+        R, _, F, _ = sim.beads()
+        want = oracle.bead_forces(R, n_beads, 1, 2.0, k_s, 0.0, 0.0)
+        e = np.abs(F - want).max() / np.abs(want).max()
+        print(f"{n_beads} beads, {periods} periods, {steps} steps: F {e:.1e}")
+        assert e < 1e-6
     sim.close()
