@@ -1012,15 +1012,20 @@ int fpd_load(fpd_sim *s, const char *path) {
     if (why) return fail(s, FPD_EINVAL, "fpd_load: %s: %s", path, why);
     int rc = fpd_sync(s);
     if (rc) return rc;
-    cudaError_t e = cudaMemcpy(s->pool, pool.data(), pool.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(s->tabmem, tabs.data(), tabs.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(s->masks[0], masks.data(), masks.size(), cudaMemcpyHostToDevice);
+    // all on the instance's stream: a synchronous copy of pageable memory may
+    // return before its last piece has arrived, and nothing orders a
+    // non-blocking stream after it
+    cudaStream_t st = s->stream;
+    cudaError_t e = cudaMemcpyAsync(s->pool, pool.data(), pool.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(s->tabmem, tabs.data(), tabs.size(), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(s->masks[0], masks.data(), masks.size(), cudaMemcpyHostToDevice, st);
     // the kept profiles follow from the restored positions
     if (e == cudaSuccess && s->inst.phi_cap)
-        e = fpd::launch_phi(s->inst_d, nullptr, s->inst.nb, s->tab, s->phi, cur_of(h.nstep) ^ 1, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+        e = fpd::launch_phi(s->inst_d, nullptr, s->inst.nb, s->tab, s->phi, cur_of(h.nstep) ^ 1, st);
     // the status flags describe the replaced run: they start over
-    if (e == cudaSuccess) e = cudaMemset(s->status, 0, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMemsetAsync(s->status, 0, sizeof(unsigned), st);
+    const cudaError_t done = cudaStreamSynchronize(st);  // in every case: the copies read the buffers above
+    if (e == cudaSuccess) e = done;
     if (e != cudaSuccess) return cuda_fail(s, e, "fpd_load");
     s->nstep = h.nstep;
     s->watch_next = (s->nstep / fpd::kWatchSteps + 1) * fpd::kWatchSteps;

@@ -941,3 +941,25 @@ def test_fp64_in_a_caller_workspace_keeps_profiles_too():
     for x, y in zip(a.beads(), b.beads()):
         assert np.array_equal(x, y)
     b.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_checkpoint_on_a_stream_of_its_own(precision, tmp_path):
+    # a stream that does not wait for the default one: the restored state is
+    # complete before the profiles are made from it and before the next step
+    import torch
+    cfg = wl.random_fiber(np.random.default_rng(6), 700, 300, n_beads=20, a=3.0, xi=1.0, precision=precision)
+    whole = gpu_sim(cfg)
+    whole.step(23)
+    st = torch.cuda.Stream()
+    a = gpu_sim(cfg, stream=st.cuda_stream)
+    a.step(10)
+    a.save(str(tmp_path / "c"))
+    for n in (3, 40):  # over the state of another step
+        a.step(n)
+        a.load(str(tmp_path / "c"))
+        a.step(13)
+        assert np.array_equal(a.populations(), whole.populations())
+        for x, y in zip(a.beads(), whole.beads()):
+            assert np.array_equal(x, y)
+    a.close()
