@@ -501,8 +501,10 @@ int enqueue_bstep(fpd_batch *b, cudaStream_t st, int64_t gstep, bool any_first) 
                              b->masks + (size_t)((gstep + 1) % M) * mstride, gstep > b->rebuild_gstep ? 1 : 0};
     cudaError_t e;
     if (nbl > 0) {
+        // the first step after a rebuild follows kernels that wrote what the
+        // bead phase reads before its wait (launch_phi): not a dependent launch
         e = fpd::launch_beads(b->precision, b->insts_d, blist, nbl, b->each, b->box, b->ntiles, b->pool, b->tab, b->phi, mw, gp, 1,
-                              b->counters, 1, st, fpd::BeadExport{}, b->status);
+                              b->counters, gstep > b->rebuild_gstep ? 1 : 0, st, fpd::BeadExport{}, b->status);
         if (e != cudaSuccess) return bcuda(b, e, "batched bead phase");
     }
     e = fpd::launch_lattice_batch(b->precision, b->insts_d, b->tiles_d, b->ntiles, b->pool, b->tab, b->phi,

@@ -392,3 +392,19 @@ def test_slot_fields_take_in_every_bead_within_its_cutoff(fpd, precision, period
     np.testing.assert_allclose(rho, f.sum(0), rtol=0, atol=1e-14)
     np.testing.assert_allclose(ux, jx / f.sum(0), rtol=0, atol=1e-14)
     np.testing.assert_allclose(uy, jy / f.sum(0), rtol=0, atol=1e-14)
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_batch_whose_instances_leave_one_by_one_equals_alone(fpd, precision):
+    # each departure rebuilds the lists, and in FP64 moves the others' kept
+    # profiles, right before the next step's bead phase reads them
+    rng = np.random.default_rng(80 + precision)
+    cases = [wl.random_fiber(rng, 80 + 7 * k, 50, n_beads=8, a=2.0, xi=1.0, precision=precision) for k in range(9)]
+    steps = [5 + 4 * k for k in range(9)]
+    b = fpd.Batch(precision, 9, 64 << 20, 128)
+    slots = [b.add(c, n) for c, n in zip(cases, steps)]
+    while b.run(1000):
+        pass
+    for c, n, s in zip(cases, steps, slots):
+        _same((b.populations(s), b.beads(s)), _alone(fpd, c, n))
+    b.close()
