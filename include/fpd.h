@@ -358,7 +358,10 @@ typedef struct fpd_batch fpd_batch;
 /* Create an empty batch: every instance uses `precision`; at most
  * max_slots instances at a time; a device pool of pool_bytes for their
  * populations and room for max_beads beads in total.  stream: cudaStream_t
- * or NULL.  Errors: FPD_EINVAL, FPD_ENOMEM, FPD_ECUDA. */
+ * or NULL.  Beside the pool and the beads' tables a batch holds lists of its
+ * tiles and, in FP64, up to 256 MB of bead profiles (it runs without, slower,
+ * where no memory is left for them).  Errors: FPD_EINVAL, FPD_ENOMEM,
+ * FPD_ECUDA. */
 int fpd_batch_create(int32_t precision, int32_t max_slots, int64_t pool_bytes, int32_t max_beads, void *stream,
                      fpd_batch **out);
 

@@ -197,8 +197,9 @@ int ensure_bscratch(fpd_batch *b, size_t bytes) {
 }
 
 // Places of the active instances' kept profiles (FP64).  The buffer grows as
-// needed; without memory for it, or for an instance whose supports are very
-// wide, profiles are evaluated instead of kept (the same values).
+// needed up to kPhiBatchBytes; beyond that, without memory for it, or for an
+// instance whose supports are very wide, profiles are evaluated instead of
+// kept (the same values).
 void place_phi(fpd_batch *b) {
     if (b->precision != 0) return;
     int64_t n = 0;
@@ -207,7 +208,9 @@ void place_phi(fpd_batch *b) {
         if (sl.state != kActive) continue;
         I.phi_cap = I.phi_off = 0;
         const int64_t cells = fpd::phi_cells(I);
-        if (I.nb == 0 || 2 * sizeof(double) * I.nb * cells > fpd::kPhiBytes || n + I.nb * cells > INT32_MAX) continue;
+        if (I.nb == 0 || 2 * sizeof(double) * I.nb * cells > fpd::kPhiBytes ||
+            2 * sizeof(double) * (n + I.nb * cells) > fpd::kPhiBatchBytes)
+            continue;
         I.phi_cap = (int)cells;
         I.phi_off = (int)n;
         n += I.nb * cells;
@@ -216,7 +219,7 @@ void place_phi(fpd_batch *b) {
         cudaFree(b->phi_mem);  // waits for queued steps, which may still read it
         b->phi_mem = nullptr;
         b->phi_len = 0;
-        const int64_t want = 2 * n + n / 2;
+        const int64_t want = std::min(2 * n + n / 2, (int64_t)(fpd::kPhiBatchBytes / sizeof(double)));
         void *p = nullptr;
         if (cudaMalloc(&p, want * sizeof(double)) == cudaSuccess) {
             b->phi_mem = (double *)p;

@@ -128,6 +128,9 @@ cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, i
 // An instance's profiles are kept (PhiTab) if both its tables fit in this:
 // L2-sized, and 30 times what 40 beads of a = 4 cells take.
 constexpr size_t kPhiBytes = (size_t)16 << 20;
+// A batch's profiles together: twice L2, and what 512 instances of 30 beads of
+// a = 4 cells take.  Instances beyond it evaluate theirs (the same bits).
+constexpr size_t kPhiBatchBytes = (size_t)256 << 20;
 // Cells of the instance's largest support box (elements a bead needs in PhiTab::phi).
 int phi_cells(const Inst &inst_h);
 // FP64: fill phi and box from the positions in the table the next bead phase

@@ -408,3 +408,28 @@ def test_batch_whose_instances_leave_one_by_one_equals_alone(fpd, precision):
     for c, n, s in zip(cases, steps, slots):
         _same((b.populations(s), b.beads(s)), _alone(fpd, c, n))
     b.close()
+
+
+def test_kept_profiles_of_an_fp64_batch_are_bounded(fpd):
+    # 400 instances whose profiles would take 321 MB: at most 256 MB are taken
+    # beside the pool, and an instance beyond them gives the same bits
+    import torch
+
+    def run(n):
+        b = fpd.Batch(0, n, n * (600 << 10), 16 * n)
+        rng = np.random.default_rng(3)
+        cases = [wl.random_fiber(rng, 60, 60, n_beads=16, a=8.0, xi=2.0, k_ev=0.0, theta0=[0.1]) for _ in range(n)]
+        slots = [b.add(c, 4) for c in cases]
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        b.run(3)
+        torch.cuda.synchronize()
+        return b, cases, slots, free - torch.cuda.mem_get_info()[0]
+
+    run(2)[0].close()  # kernels are loaded here
+    b, cases, slots, taken = run(400)
+    print(f"taken beside the pool: {taken / 2 ** 20:.0f} MiB")
+    assert taken <= (256 + 16) << 20  # and the lists of tiles, in pages of 2 MB
+    for k in (0, 399):
+        _same((b.populations(slots[k]), b.beads(slots[k])), _alone(fpd, cases[k], 3))
+    b.close()
