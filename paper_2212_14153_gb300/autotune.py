@@ -60,9 +60,12 @@ def _store(d: dict) -> None:
 
 def time_variants(cfg: dict, steps: int = 256, warmup: int = 64, stream=None, rounds: int = 3) -> list[float]:
     """Milliseconds per step of every variant on a scratch instance: the
-    shortest of `rounds` timings each, taken in turn.  One timing in order
-    disfavoured the first variant, timed while the GPU was still warming up
-    (1024 x 256: variant 0, 5 % faster, lost to variant 1)."""
+    shortest of `rounds` timings each, taken in turn.  The step graphs a
+    timing replays are captured before it starts: captured within it, their
+    64 launches cost a variant whose steps are short more than it differs
+    from the others (300 x 200 in FP32, variants 0 and 1: 2.27 and 2.33 us a
+    step with them, 2.29 and 2.12 without).  FpdError if a variant's run
+    fails."""
     import torch
     st = stream or torch.cuda.Stream()
     sim = fpd.Simulation(cfg, stream=st.cuda_stream)
@@ -72,6 +75,7 @@ def time_variants(cfg: dict, steps: int = 256, warmup: int = 64, stream=None, ro
     def timed(k: int) -> float:
         a = torch.cuda.Event(enable_timing=True)
         b = torch.cuda.Event(enable_timing=True)
+        sim.prepare(k)
         a.record(st)
         sim.step(k)
         b.record(st)
@@ -85,8 +89,9 @@ def time_variants(cfg: dict, steps: int = 256, warmup: int = 64, stream=None, ro
     for _ in range(rounds):
         for v in range(n):
             sim.set_tuning(v)
-            sim.step(33)
+            sim.step(32)  # a whole chunk: the timed ones replay its graph
             best[v] = min(best[v], timed(steps))
+            sim.sync()
     sim.close()
     return best
 
