@@ -3,15 +3,18 @@
 Each sweep variant (see fpd_set_tuning) is timed with CUDA events on a
 scratch instance of the same workload (same parameters, so the same hot
 tiles), after warm-up, and the fastest is returned and cached per GPU,
-library build, precision and lattice size in a JSON file
-($FPD_TUNING_CACHE, default ~/.cache/fpd_gb300/tuning.json): a rebuilt
-library (changed kernels) is timed afresh.  Variants compute the same arithmetic
+library build, storage, lattice, collision model, boundaries, forces and
+beads in a JSON file ($FPD_TUNING_CACHE, default
+~/.cache/fpd_gb300/tuning.json): a rebuilt library (changed kernels) is timed
+afresh.  Constant rates (collision 1) run one shape whatever the variant:
+variant 0, untimed.  Variants compute the same arithmetic
 (they differ only in how the compiler contracts multiply-adds, i.e. at the
 rounding level), so the choice only affects speed.
 """
 from __future__ import annotations
 
 import json
+import math
 import os
 
 from . import fpd
@@ -34,8 +37,17 @@ def _lib_tag() -> str:
 
 
 def _key(cfg: dict, gpu: str) -> str:
-    return (f"{gpu}|lib{_lib_tag()}|p{cfg.get('precision', 0)}|{cfg['nx']}x{cfg['ny']}"
-            f"|nb{cfg.get('n_beads', 0) * cfg.get('n_fibers', 0)}")
+    """Everything that decides which kernels run, and how much of the lattice
+    its beads mark."""
+    nb = cfg.get("n_beads", 0) * cfg.get("n_fibers", 0)
+    beads = ""
+    if nb:  # cells from a bead to its cutoff: whole ones, so that runs of nearly the same beads share a timing
+        reach = cfg.get("a", 2.0) + cfg.get("phi_cut", 8.0) * cfg.get("xi", 1.0)  # defaults: fpd_default_params
+        beads = f"|n_beads{cfg['n_beads']}|reach{math.ceil(reach)}"
+    forced = int(bool(cfg.get("gx", 0.0) or cfg.get("gy", 0.0)))
+    sandwich = int(cfg.get("sandwich_zl", 0.0) > 0.0)
+    return (f"{gpu}|lib{_lib_tag()}|p{cfg.get('precision', 0)}|{cfg['nx']}x{cfg['ny']}|nb{nb}{beads}"
+            f"|collision{cfg.get('collision', 0)}|periodic_y{cfg.get('periodic_y', 0)}|forced{forced}|sandwich{sandwich}")
 
 
 def _load() -> dict:
@@ -99,6 +111,8 @@ def time_variants(cfg: dict, steps: int = 256, warmup: int = 64, stream=None, ro
 def tune(cfg: dict, steps: int = 256, warmup: int = 64, use_cache: bool = True) -> int:
     """Fastest sweep variant for this workload (cached)."""
     import torch
+    if cfg.get("collision", 0) == fpd.FPD_MRT_LL:
+        return 0
     gpu = torch.cuda.get_device_name()
     key = _key(cfg, gpu)
     cache = _load() if use_cache else {}

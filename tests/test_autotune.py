@@ -105,3 +105,24 @@ def test_a_variant_whose_run_fails_is_not_timed_in_silence(fakes, monkeypatch):
     monkeypatch.setattr(FakeSimulation, "failing", 3)
     with pytest.raises(fpd.FpdError):
         autotune.time_variants(CFG)
+
+
+def test_constant_rates_are_not_timed(fakes):
+    # every variant runs the same kernel there: their timings differ by noise
+    assert autotune.tune(dict(CFG, collision=fpd.FPD_MRT_LL)) == 0
+    assert FakeSimulation.made == 0
+    assert autotune.tune(dict(CFG, collision=fpd.FPD_BGK)) == 0 and FakeSimulation.made == 1
+
+
+@pytest.mark.parametrize("change", [dict(collision=2), dict(periodic_y=1), dict(gx=1e-5), dict(gy=-1e-5),
+                                    dict(sandwich_zl=8.0, sandwich_zr=16.0), dict(a=3.0), dict(xi=0.5),
+                                    dict(phi_cut=6.0), dict(n_beads=4, n_fibers=3), dict(n_beads=3), dict(nx=97),
+                                    dict(precision=0)])
+def test_the_cache_tells_workloads_of_other_kernels_apart(fakes, change):
+    import numpy as np
+    cfg = wl.random_fiber(np.random.default_rng(1), 96, 48, n_beads=6, a=2.0, xi=1.0, n_fibers=2, precision=1)
+    autotune.tune(cfg)
+    autotune.tune(dict(cfg, u_top=0.011, theta0=[0.1, 0.2]))  # the same kernels on the same work
+    assert FakeSimulation.made == 1
+    autotune.tune(dict(cfg, **change))
+    assert FakeSimulation.made == 2
