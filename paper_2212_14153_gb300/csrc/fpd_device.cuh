@@ -847,7 +847,10 @@ __device__ __forceinline__ void collide_trt(double g[9], const TrtRates &k) {
     const double jx = b13 + (b57 - b68), jy = b24 + (b57 + b68);
     const double irho = recip(1.0 + drho);
     const double ux = jx * irho, uy = jy * irho;
-    const double xx = jx * ux, yy = jy * uy, xy = jx * uy, t = xx + yy;
+    // spelled out: a product that feeds a sum could be contracted in one
+    // kernel and not in another (nothing else here could: every other sum is
+    // of sums or an fma)
+    const double xx = __dmul_rn(jx, ux), yy = __dmul_rn(jy, uy), xy = __dmul_rn(jx, uy), t = __dadd_rn(xx, yy);
     const double D = __fma_rn(-1.5, t, drho);  // rho - 1 - 1.5 rho u^2
     const double e1 = k.k1 * D, e3 = __fma_rn(k.k4, t, k.k3 * D);
     const double ev13 = __fma_rn(k.c1, a13, __fma_rn(k.k2, xx, e1)), ev24 = __fma_rn(k.c1, a24, __fma_rn(k.k2, yy, e1));

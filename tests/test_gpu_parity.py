@@ -963,3 +963,36 @@ def test_checkpoint_on_a_stream_of_its_own(precision, tmp_path):
         for x, y in zip(a.beads(), whole.beads()):
             assert np.array_equal(x, y)
     a.close()
+
+
+@pytest.mark.parametrize("case", ["flow", "fibers", "sandwich", "constant rates", "BGK"])
+def test_fp64_gives_the_same_bits_in_every_launch_shape(case):
+    # one or two cells a thread, rows split over CTAs or not (96 x 64 is, 700 x
+    # 520 is not), batches: the two-relaxation-time update is compiled into
+    # each kernel anew
+    from paper_2212_14153_gb300 import fpd
+    n = (700, 520) if case == "BGK" else (96, 64)
+    if case == "fibers":
+        cfg = wl.random_fiber(np.random.default_rng(3), *n, n_beads=6, a=2.0, xi=1.0, n_fibers=2)
+    else:
+        cfg = wl.couette_only(*n, u=0.013, nu=0.07, init_couette=0)
+    cfg.update({"sandwich": dict(sandwich_zl=16.0, sandwich_zr=48.0), "constant rates": dict(collision=1),
+                "BGK": dict(collision=2)}.get(case, {}))
+    got = []
+    for variant in range(5):
+        s = gpu_sim(cfg)
+        s.set_tuning(variant)
+        s.step(70)
+        got.append(s.populations())
+        s.close()
+    for variant in range(3):
+        b = fpd.Batch(0, 2, 256 << 20, 64)
+        b.set_tuning(variant)
+        slot = b.add(cfg, 70)
+        b.add(wl.couette_only(40, 24), 70)
+        while b.run(1000):
+            pass
+        got.append(b.populations(slot))
+        b.close()
+    for f in got[1:]:
+        assert np.array_equal(f, got[0])
