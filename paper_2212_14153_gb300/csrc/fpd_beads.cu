@@ -241,10 +241,7 @@ __device__ __forceinline__ float edge_diff(float a, float b, float L) {
 
 // A double as a pair of floats, h + l equal to it within 2^-48 of its size,
 // from its bits: the conversions and subtractions are FP64 instructions, a
-// chain of which took the last CTA about a microsecond.  Taken of a bead's
-// position less that of its fiber's first bead, so that the pair is as good
-// wherever the fiber has drifted (a fiber's length times 2^-48; the unwrapped
-// position's after 4096 periods of 128 columns: 2e-9 of a cell).  Sizes outside
+// chain of which took the last CTA about a microsecond.  Sizes outside
 // [2^-74, 2^127) do not occur in use: 0 below, NaN above.
 __device__ __forceinline__ float2 split(double x) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
@@ -276,15 +273,16 @@ __device__ __forceinline__ void segment_axis(const Inst &I, double A, double B, 
     t = d * (1.0 / L);
     str = L - I.l0;
 }
-// FP32 paths: differences and squares in pairs of floats (2^-46), as the
-// stretch L - l0 = (|d|^2 - l0^2) / (L + l0) of a stiff spring is small
-// against them and must not cancel away.
-__device__ __forceinline__ void segment_axis(const Inst &I, float2 A, float2 B, float &L, float &t, float &str) {
-    float dh, dl, p, pe, s, se, q, qe;
-    two_sum(B.x, -A.x, dh, dl);
-    dl += B.y - A.y;
-    const float d = dh + dl;
-    dl -= d - dh;
+// FP32 paths: the difference of the unwrapped positions in FP64 (one
+// instruction; pairs of floats of the positions themselves were 2e-9 of a cell
+// off after 4096 periods of 128 columns), its square in pairs of floats
+// (2^-46), as the stretch L - l0 = (|d|^2 - l0^2) / (L + l0) of a stiff spring
+// is small against it and must not cancel away.
+__device__ __forceinline__ void segment_axis(const Inst &I, double A, double B, float &L, float &t, float &str) {
+    float dl, p, pe, s, se, q, qe;
+    const float2 D = split(B - A);
+    const float d = D.x + D.y;
+    dl = D.y - (d - D.x);
     square2(d, dl, p, pe);
     two_sum(p, __shfl_xor_sync(0xffffffffu, p, 1), s, se);
     se += pe + __shfl_xor_sync(0xffffffffu, pe, 1);
@@ -391,14 +389,9 @@ template <class R, int NT> struct ListCap {
 };
 
 // The last CTA's view of its instance, in the shared memory the list took;
-// x and y of a bead or segment side by side.  FP32 paths: the segments are
-// taken from rel, the positions relative to the first bead of their fiber in
-// pairs of floats; pos takes its place for the excluded volume.
+// x and y of a bead or segment side by side.
 template <class R> struct ForceShared {
-    union {
-        double pos[2 * kMaxBeads];
-        float2 rel[2 * kMaxBeads];
-    };
+    double r[2 * kMaxBeads];
     R S[kMaxBeads], t[2 * kMaxBeads], pull[2 * kMaxBeads], len[kMaxBeads], str[kMaxBeads];
     float xf[kMaxBeads], yf[kMaxBeads];
     unsigned cand[kMaxBeads * (kMaxBeads / 32)];
@@ -553,7 +546,6 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     // team: every bead's place and whether it may be close to another
     __shared__ double s_peer[kTeam ? kTeamBeads : 1][2];
     __shared__ unsigned long long s_near[kTeam ? kTeamBeads : 1];
-    __shared__ float2 s_place[kTeam ? 2 * kTeamBeads : 1];
     if (parts > 1 || kTeam) cluster_arrive();  // waited for before the first push
     int uses = 0;
     // blist[i] = (2 slot + par_xor, global bead index, the instance's first
@@ -1013,8 +1005,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         }
     }
     if constexpr (kTeam) {
-        const int q = b - first, N = I.n_beads, i0 = q - q / N * N, head = (lane >> 1) / N * N;
         cluster_wait();  // every bead's place is here, and its status bits are set
+        const int q = b - first, N = I.n_beads, i0 = q - q / N * N;
         // fast-bead guard, as below
         if (w != 0) {
             if (q == 0 && status && (__ldcg(status + ii) & kFlagFastBead))
@@ -1022,14 +1014,12 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
                     atomicOr(mask_write + (I.tile_base + t) * I.mask_words, 1u);
             return;
         }
-        if (lane < 2 * nb) s_place[lane] = split(s_peer[lane >> 1][lane & 1] - s_peer[head][lane & 1]);
         const bool crowd = I.k_ev != 0.0 && __any_sync(0xffffffffu, lane < nb && s_near[lane] != 0ull);
-        __syncwarp();
         // lanes 2 m + ax, m < 4: axis ax of segment q - 2 + m of the fiber
         const int ax = lane & 1, m = (lane >> 1) & 3, j = q - 2 + m;
         const bool seg = i0 - 2 + m >= 0 && i0 - 2 + m < N - 1;
         float L, t, str;
-        segment_axis(I, s_place[seg ? 2 * j + ax : 0], s_place[seg ? 2 * j + 2 + ax : 1], L, t, str);
+        segment_axis(I, s_peer[seg ? j : 0][ax], s_peer[seg ? j + 1 : 0][ax], L, t, str);
         if (!seg) t = 0.f;
         const float tn = __shfl_down_sync(0xffffffffu, t, 2), tp = __shfl_up_sync(0xffffffffu, t, 2);
         const float v = tn + tp, vt1 = v * t, vt = vt1 + __shfl_xor_sync(0xffffffffu, vt1, 1);
@@ -1068,13 +1058,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     // warp 64 cycles each whatever its lanes do, so x and y share them)
     const int items = 2 * nb, N = I.n_beads;
     const float inv_n = 1.0f / (float)N;
-    // place of bead q < 256 within its fiber
-    auto in_fiber = [&](int q) { return q - N * (int)(((float)q + 0.5f) * inv_n); };
     for (int k = tid; k < items; k += NT) {
-        const double *r = ((k & 1) ? tnew.Ry : tnew.Rx) + first;
-        const double x = nb == 1 ? s_R[k] : __ldcg(r + (k >> 1));
-        if constexpr (kF64) fs.pos[k] = x;
-        else fs.rel[k] = nb == 1 ? make_float2(0.f, 0.f) : split(x - __ldcg(r + (k >> 1) - in_fiber(k >> 1)));
+        fs.r[k] = nb == 1 ? s_R[k] : __ldcg(((k & 1) ? tnew.Ry : tnew.Rx) + first + (k >> 1));
         if (!(k & 1)) fs.S[k >> 1] = (R)(nb == 1 ? s_S : __ldcg(tnew.S + first + (k >> 1)));
     }
     __syncthreads();
@@ -1085,13 +1070,14 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
     // phase's masks, so that the next sweeps wait on all of them
     if (st_now & kFlagFastBead)
         for (int t = tid; t < I.ntx * I.nty; t += NT) atomicOr(mask_write + (I.tile_base + t) * I.mask_words, 1u);
+    // place of bead q < 256 within its fiber
+    auto in_fiber = [&](int q) { return q - N * (int)(((float)q + 0.5f) * inv_n); };
     // Segment q (bead q to q + 1 of the fiber): length, tangent, stretch
     for (int k0 = 0; k0 < items; k0 += NT) {
         const int k = k0 + tid, q = k >> 1;
         const bool seg = k < items && in_fiber(q) < N - 1;
         R L, t, str;
-        if constexpr (kF64) segment_axis(I, fs.pos[seg ? k : 0], fs.pos[seg ? k + 2 : 1], L, t, str);
-        else segment_axis(I, fs.rel[seg ? k : 0], fs.rel[seg ? k + 2 : 1], L, t, str);
+        segment_axis(I, fs.r[seg ? k : 0], fs.r[seg ? k + 2 : 1], L, t, str);
         if (seg) {
             fs.t[k] = t;
             if (!(k & 1)) {
@@ -1101,14 +1087,9 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         }
     }
     if (crowd) {
-        if constexpr (!kF64) {
-            __syncthreads();  // the segments no longer read rel
-            for (int k = tid; k < items; k += NT) fs.pos[k] = __ldcg(((k & 1) ? tnew.Ry : tnew.Rx) + first + (k >> 1));
-            __syncthreads();
-        }
         for (int q = tid; q < nb; q += NT) {
-            fs.xf[q] = (float)(fs.pos[2 * q] - fs.pos[0]);
-            fs.yf[q] = (float)(fs.pos[2 * q + 1] - fs.pos[1]);
+            fs.xf[q] = (float)(fs.r[2 * q] - fs.r[0]);
+            fs.yf[q] = (float)(fs.r[2 * q + 1] - fs.r[1]);
         }
         __syncthreads();
         screen_close<NW>(I, fs.xf, fs.yf, fs.cand);
@@ -1133,7 +1114,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         R f = (R)0;
         if (i0 > 0) f -= fs.pull[k - 2];
         if (i0 < N - 1) f += fs.pull[k];
-        if (crowd) f += close_force<R>(I, fs.pos, fs.cand + q * ((nb + 31) / 32), (nb + 31) / 32, q, ax);
+        if (crowd) f += close_force<R>(I, fs.r, fs.cand + q * ((nb + 31) / 32), (nb + 31) / 32, q, ax);
         // constant external force F_0 (driven particle, Sec. 3.2)
         if constexpr (kF64) f += ax ? I.ext_fy : I.ext_fx;
         else f += ax ? I.f_ext_fy : I.f_ext_fx;
