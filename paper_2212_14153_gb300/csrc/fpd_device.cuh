@@ -727,14 +727,6 @@ __device__ __forceinline__ void collide(R g[9], R Fx, R Fy, R s_nu, R s_e, R s_e
 // advances two cells with it gets the bits each cell gets alone.  Every
 // operation is spelled out (no contraction left to the compiler).
 template <class V> struct Ar;
-template <> struct Ar<double> {
-    static __device__ __forceinline__ double c(double a) { return a; }
-    static __device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
-    static __device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
-    static __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
-    static __device__ __forceinline__ double fma(double a, double b, double d) { return __fma_rn(a, b, d); }
-    static __device__ __forceinline__ double rcp(double a) { return recip(a); }
-};
 template <> struct Ar<float> {
     static __device__ __forceinline__ float c(float a) { return a; }
     static __device__ __forceinline__ float add(float a, float b) { return __fadd_rn(a, b); }
