@@ -1,6 +1,7 @@
 """Bead phase at the places where its FP32 arithmetic or its lists could go wrong,
 against FP64 references: neighbours across a periodic edge, slow beads,
-supports that span a periodic box, fibers that have drifted far.
+supports that span a periodic box, fibers that have drifted far, supports about
+as large as a list.
 """
 import math
 import os
@@ -127,4 +128,51 @@ def test_forces_do_not_depend_on_how_far_a_fiber_has_drifted(fpd, n_beads, perio
         e = np.abs(F - want).max() / np.abs(want).max()
         print(f"{n_beads} beads, {periods} periods, {steps} steps: F {e:.1e}")
         assert e < 1e-6
+    sim.close()
+
+
+@pytest.mark.parametrize("precision,xi", [
+    (1, 1.4375), (1, 1.5), (2, 1.4375), (2, 1.5),  # boxes of 35 x 35 and 36 x 36, lists of 1280
+    (0, 1.1875), (0, 1.25),                        # 31 x 31 and 32 x 32, lists of 1000
+])
+def test_support_boxes_about_as_large_as_a_list(fpd, precision, xi):
+    # more beads than SMs run in the narrowest CTAs, each with all of its
+    # bead's cells; alone an instance's CTAs are wide or share a bead.  The same
+    # bits, on either side of a list's length
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.default_rng(7)
+    n = sms // 16 + 2
+    cases = [wl.random_fiber(rng, 150, 90, n_beads=8, a=4.0, xi=xi, n_fibers=2, precision=precision, theta0=[0.4, 2.5])
+             for _ in range(n)]
+    b = fpd.Batch(precision, n, 512 << 20, 16 * n)
+    slots = [b.add(c, 6) for c in cases]
+    while b.run(100):
+        pass
+    for c, s in list(zip(cases, slots))[::3]:
+        alone = fpd.Simulation(c)
+        alone.step(6)
+        assert np.array_equal(alone.populations(), b.populations(s))
+        for x, y in zip(alone.beads(), b.beads(s)):
+            assert np.array_equal(x, y)
+        alone.close()
+    if precision != 2:
+        ref = oracle.Sim(dict(cases[0], precision=0, threads=THREADS))
+        ref.step(6)
+        for x, y in zip(b.beads(slots[0])[:2], ref.beads()[:2]):
+            assert np.linalg.norm(x - y) < (1e-12 if precision == 0 else 2e-5) * np.linalg.norm(y)
+    b.close()
+
+
+@pytest.mark.parametrize("xi", [1.4375, 1.5])
+def test_support_box_of_two_lists_beside_a_long_sweep(fpd, xi):
+    # 4290 tiles: the bead CTAs wait for the sweep first, with 256 threads and
+    # lists of 1280 cells (FP32 against the oracle)
+    rng = np.random.default_rng(9)
+    cfg = wl.random_fiber(rng, 1030, 1040, n_beads=9, a=4.0, xi=xi, n_fibers=2, precision=1)
+    sim, ref = fpd.Simulation(cfg), oracle.Sim(dict(cfg, precision=0, threads=THREADS))
+    sim.step(10)
+    ref.step(10)
+    for x, y in zip(sim.beads()[:2], ref.beads()[:2]):
+        assert np.linalg.norm(x - y) < 2e-5 * np.linalg.norm(y)
     sim.close()
