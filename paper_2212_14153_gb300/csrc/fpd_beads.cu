@@ -1269,19 +1269,25 @@ cudaError_t launch_beads(int precision, const Inst *inst_d, const int4 *blist, i
     // Every instance of the launch has `each` beads (0: not all the same): its
     // CTAs form a cluster where there is room beside the sweep for one
     const bool team = precision != 0 && few && !wait_first && advance && !ex.ring && each >= 1 && each <= team_limit();
-    // Threads a CTA, us a step.  A short list beside a sweep of up to a few
-    // waves, 512 against 256: 1024 x 256 and 20 beads of a = 2 10.98 / 12.2,
-    // of a = 4 10.8 / 11.9, 160 x 160 and one bead of a 37 x 37 box 9.2 /
-    // 10.9; where the sweep is no more than two tiles an SM and the box
-    // small, 333 x 171 and 27 beads, 10.3 / 9.7.  Beside a long sweep the
-    // narrower CTAs leave it more room: 4096 x 1024 FP16 27.05 / 26.64, FP32
-    // 43.86 / 43.57 (128 threads: 26.89 and 44.85).  FP64, bound by its
-    // instructions, 512 / 256 / 128: 80 x 40 27.8 / 26.5 / 26.1, 200 x 100
-    // 256 / 128 26.2 / 25.6, 4096 x 1024 498 / 486.1 / 485.4.  Long lists: 128
-    // (six CTAs an SM).
+    // Threads a CTA, us a step.  A short list without clusters beside a sweep of
+    // up to a few waves, 512 against 256, FP32 (FP16): boxes of up to 512 cells,
+    // two rounds of 256 threads (kWideBox; phi_cells has four more an axis), at
+    // 242 tiles and 3 x 9 beads, box of 225 cells 10.07 / 9.57 (11.34 / 10.90),
+    // 484 10.55 / 10.20 (11.61 / 11.36); 600 tiles 10.22 / 9.71 (11.69 / 11.70),
+    // 10.74 / 10.33 (11.98 / 11.92); 1024 tiles 10.46 / 10.40 (12.10 / 11.77),
+    // 10.94 / 10.94 (12.36 / 11.80); 3616 tiles 11.55 / 11.63 (12.50 / 12.42),
+    // 12.0 / 12.38 (12.87 / 12.84): past two tiles an SM the gain is not there
+    // in every storage.  Larger boxes, 242 tiles: 576 cells 9.88 / 10.39, 625
+    // 10.67 / 10.92 (11.46 / 11.33), 784 10.2 / 11.2, 1296 12.3 / 14.7; 1024
+    // tiles, 625 cells 10.77 / 11.66 (12.06 / 12.30).  Clusters: 160 x 160 and
+    // one bead of a 37 x 37 box 9.2 / 10.9.  Beside a long sweep the narrower
+    // CTAs leave it more room: 4096 x 1024 FP16 27.05 / 26.64, FP32 43.86 /
+    // 43.57 (128 threads: 26.89 and 44.85).  FP64, bound by its instructions,
+    // 512 / 256 / 128: 80 x 40 27.8 / 26.5 / 26.1, 200 x 100 256 / 128 26.2 /
+    // 25.6, 4096 x 1024 498 / 486.1 / 485.4.  Long lists: 128 (six CTAs an SM).
     int threads = kBeadThreads;
     if (precision != 0 && few) {
-        const bool narrow = wait_first || (!team && box < kWideBox && ntiles <= 2 * sms);
+        const bool narrow = wait_first || (!team && box <= kWideBox && ntiles <= 2 * sms);
         threads = narrow ? kBeadThreadsMid : kBeadThreadsFew;
     }
     cudaLaunchConfig_t cfg = {};

@@ -13,7 +13,7 @@ constexpr int kSplitCtas = 304, kSplitCtas64 = 608;  // a sweep's tiles are spli
 constexpr int kMaxBeads = 256;   // beads per instance (shared-memory tables)
 constexpr int kBeadThreads = 128;  // per bead CTA: more beads resident at once (batched sweep +9 %)
 constexpr int kBeadThreadsMid = 256, kBeadThreadsFew = 512;  // FP32, FP16, the beads fit on the SMs one per SM: launch_beads
-constexpr int kWideBox = 900;  // support box (phi_cells) too large for kBeadThreadsMid beside a short sweep
+constexpr int kWideBox = 700;  // phi_cells of a box of 512 cells, two rounds of kBeadThreadsMid threads: launch_beads
 constexpr int kEarlyListTiles = 4096;  // longest sweep (tiles) whose bead phase lists its supports before waiting: launch_beads
 constexpr int kTeamBeads = 16;  // most beads of an instance whose CTAs form a cluster
 constexpr int kBeadParts = 8;    // CTAs a bead's cells are split over at most (FP64, short bead lists)

@@ -176,3 +176,24 @@ def test_support_box_of_two_lists_beside_a_long_sweep(fpd, xi):
     for x, y in zip(sim.beads()[:2], ref.beads()[:2]):
         assert np.linalg.norm(x - y) < 2e-5 * np.linalg.norm(y)
     sim.close()
+
+
+@pytest.mark.parametrize("precision", [1, 2])
+@pytest.mark.parametrize("xi", [0.875, 0.9375, 1.0])  # boxes of 484, 529 and 576 cells
+def test_widths_of_the_bead_ctas_give_the_same_bits(fpd, precision, xi):
+    # 18 beads: 256 threads with a box of up to 512 cells, 512 above; in a
+    # batch of 11 such instances 128
+    rng = np.random.default_rng(5)
+    cases = [wl.random_fiber(rng, 180, 70, n_beads=9, a=2.25, xi=xi, n_fibers=2, precision=precision) for _ in range(11)]
+    b = fpd.Batch(precision, 11, 256 << 20, 198)
+    slots = [b.add(c, 8) for c in cases]
+    while b.run(100):
+        pass
+    for c, s in list(zip(cases, slots))[::5]:
+        alone = fpd.Simulation(c)
+        alone.step(8)
+        assert np.array_equal(alone.populations(), b.populations(s))
+        for x, y in zip(alone.beads(), b.beads(s)):
+            assert np.array_equal(x, y)
+        alone.close()
+    b.close()
