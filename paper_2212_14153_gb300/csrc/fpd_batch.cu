@@ -500,8 +500,9 @@ int enqueue_bstep(fpd_batch *b, cudaStream_t st, int64_t gstep, bool any_first) 
     unsigned *mw = b->masks + (size_t)(gstep % M) * mstride;
     // the previous buffer holds the previous bead phase's marks unless the
     // masks were reset before this step
-    const fpd::SweepMasks mk{mw, b->masks + (size_t)((gstep + M - 1) % M) * mstride,
-                             b->masks + (size_t)((gstep + 1) % M) * mstride, gstep > b->rebuild_gstep ? 1 : 0};
+    fpd::SweepMasks mk{mw, b->masks + (size_t)((gstep + M - 1) % M) * mstride,
+                       b->masks + (size_t)((gstep + 1) % M) * mstride, gstep > b->rebuild_gstep ? 1 : 0};
+    mk.unmarked = b->n_all == 0;
     cudaError_t e;
     if (nbl > 0) {
         // the first step after a rebuild follows kernels that wrote what the

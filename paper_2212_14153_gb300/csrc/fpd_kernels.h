@@ -41,6 +41,9 @@ struct SweepMasks {
     // are in place when that one ends, and wait for it before they read
     int chained = 0;
     unsigned copy_shortfall = 0;  // test only: extra bytes the staged copies expect (their waits run out)
+    // batched sweep, 1: no instance has beads, so no tile is ever marked and all
+    // of them update as unmarked tiles do (there is no bead phase to wait for)
+    int unmarked = 0;
 };
 
 // Sticky per-instance status bits, set on the device (values of the

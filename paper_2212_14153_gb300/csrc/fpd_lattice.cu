@@ -1472,12 +1472,19 @@ static cudaError_t lattice_batch_v(int variant, const Inst *insts, const int2 *t
     cudaLaunchAttribute attr[1];
     const dim3 grid(ntiles);
     const int ec = after_beads ? mk.early_cold : 0;
+    // tiles updated from their records: without beads in the batch as well (they
+    // read the record in any case and otherwise copied the instance's too; us a
+    // step of 300 x 200 flows, without records / copied too / from records: 16
+    // in FP32 11.2 / 12.6 / 9.7, 64 57.1 / 53.8 / 44.8, 16 in FP16 11.5 / 12.9 /
+    // 9.7, 64 46.5 / 48.4 / 35.6).  The other shapes have no record, and only
+    // lose a read of the mask by it (vectors 2 to 4 %)
+    const int ec_rec = after_beads || std::is_same<S, double>::value ? ec : mk.unmarked;
     // a batch holding instances with constant Lallemand-Luo rates: both
     // collision forms, one cell per thread
     if (any_mrt) {
         const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX, kTileY), after_beads, st, attr);
         return cudaLaunchKernelEx(&cfg, k_lattice_batch<S, 1, false, kCollAny>, insts, tiles, (S *)pool, tab0, tab1,
-                                  mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1, recs, mask_words);
+                                  mk.read, mk.prev, mk.clear, gparity, after_beads, ec_rec, phi0, phi1, recs, mask_words);
     }
     if (variant == 2) {
         const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX / VecWidth<S>::value, kTileY), after_beads,
@@ -1492,7 +1499,7 @@ static cudaError_t lattice_batch_v(int variant, const Inst *insts, const int2 *t
     }
     const cudaLaunchConfig_t cfg = sweep_config(grid, dim3(kTileX, kTileY), after_beads, st, attr);
     return cudaLaunchKernelEx(&cfg, k_lattice_batch<S, 1, false, kCollTrt>, insts, tiles, (S *)pool, tab0, tab1,
-                              mk.read, mk.prev, mk.clear, gparity, after_beads, ec, phi0, phi1, recs, mask_words);
+                              mk.read, mk.prev, mk.clear, gparity, after_beads, ec_rec, phi0, phi1, recs, mask_words);
 }
 
 cudaError_t launch_lattice_batch(int precision, const Inst *insts, const int2 *tiles, int ntiles, void *pool,

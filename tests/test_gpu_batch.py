@@ -433,3 +433,35 @@ def test_kept_profiles_of_an_fp64_batch_are_bounded(fpd):
     for k in (0, 399):
         _same((b.populations(slots[k]), b.beads(slots[k])), _alone(fpd, cases[k], 3))
     b.close()
+
+
+@pytest.mark.parametrize("variant", [0, 1, 2])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+def test_batch_without_any_beads_equals_alone(fpd, precision, variant):
+    # no tile is ever marked, so every tile but the first takes the update of
+    # unmarked tiles, from the first step on; body force, sandwich layers and
+    # constant rates keep theirs.  A fiber admitted later ends that
+    cases = [
+        wl.couette_only(45, 1900, u=0.01, nu=0.2, init_couette=0, precision=precision),
+        dict(wl.couette_only(70, 40, u=0.01, nu=0.1, init_couette=0, precision=precision), gx=1e-5),
+        dict(wl.couette_only(50, 41, u=0.01, nu=0.1, precision=precision), sandwich_zl=8.0, sandwich_zr=32.0),
+        dict(wl.couette_only(33, 9, u=0.02, nu=0.05, init_couette=0, precision=precision), collision=2),
+        dict(wl.couette_only(96, 33, u=0.01, nu=0.2, precision=precision), periodic_y=1),
+    ]
+    if variant == 0:
+        cases.append(dict(wl.couette_only(64, 24, u=0.01, nu=0.1, init_couette=0, precision=precision), collision=1))
+    late = wl.random_fiber(np.random.default_rng(2), 64, 48, n_beads=4, a=2.0, xi=0.5, precision=precision)
+    b = fpd.Batch(precision, 8, 64 << 20, 16)
+    b.set_tuning(variant)
+    slots = [b.add(c, 75) for c in cases]
+    b.step(41)
+    slots.append(b.add(late, 34))
+    b.step(34)
+    for c, s in zip(cases + [late], slots):
+        n = 34 if c is late else 75
+        sim = fpd.Simulation(c)
+        sim.set_tuning(variant)
+        sim.step(n)
+        _same((b.populations(s), b.beads(s)), (sim.populations(), sim.beads()))
+        sim.close()
+    b.close()
