@@ -1125,6 +1125,15 @@ __device__ __forceinline__ void overlay_f64(const Inst &I, const BeadTab &tab, c
     fx = I.gx;
     fy = I.gy;
     const int tile = I.tile_base + (y / kTileY) * I.ntx + x / kTileX;
+    // what follows is FP64 work before its loop as well (places, half a period),
+    // which a cell without beads need not pay for: a field read of 1024 x 512
+    // without beads 169 -> 157 us, of 4096 x 1024 with 40 1086 -> 1023 (FP32)
+    unsigned any = I.nb;
+    if (mask) {
+        any = 0u;
+        for (int w = 0; w < I.mask_words; ++w) any |= mask[tile * I.mask_words + w];
+    }
+    if (any == 0u) return;
     const double xc = x + 0.5, yc = y + 0.5;
     const float fxc = (float)x + 0.5f, fyc = (float)y + 0.5f, reach = I.f_rcut + 1.0f;
     for (int w = 0; w < I.mask_words; ++w) {
