@@ -501,21 +501,17 @@ StateLayout state_layout(const fpd::Inst &I, size_t elem) {
     return L;
 }
 
-// FP64: room for the beads' profiles over their support boxes (PhiTab), beside
-// the state block, unless the supports are so wide that the two tables would
-// outgrow kPhiBytes.  Without it (no memory left) the instance evaluates them.
-void alloc_profiles(fpd_sim *s) {
+// FP64: bytes of the beads' profiles over their support boxes (PhiTab), 0 where
+// the supports are so wide that the two tables would outgrow kPhiBytes.
+size_t profile_bytes(const fpd::Inst &I, size_t elem) {
+    if (elem != 8 || I.nb <= 0) return 0;
+    const size_t bytes = 2 * (size_t)I.nb * fpd::phi_cells(I) * sizeof(double);
+    return bytes > fpd::kPhiBytes ? 0 : bytes + 2 * (size_t)I.nb * sizeof(int4);
+}
+void place_profiles(fpd_sim *s, void *mem) {
     const fpd::Inst &I = s->inst;
-    if (s->elem != 8 || I.nb <= 0) return;
-    const size_t one = (size_t)I.nb * fpd::phi_cells(I), bytes = 2 * one * sizeof(double);
-    const size_t box = 2 * (size_t)I.nb * sizeof(int4);
-    if (bytes > fpd::kPhiBytes) return;
-    if (cudaMalloc(&s->phimem, bytes + box) != cudaSuccess) {
-        s->phimem = nullptr;
-        (void)cudaGetLastError();
-        return;
-    }
-    int4 *b = (int4 *)s->phimem;
+    const size_t one = (size_t)I.nb * fpd::phi_cells(I);
+    int4 *b = (int4 *)mem;
     double *f = (double *)(b + 2 * I.nb);
     for (int t = 0; t < 2; ++t) s->phi[t] = fpd::PhiTab{f + t * one, b + t * I.nb};
     s->inst.phi_cap = fpd::phi_cells(I);
@@ -594,10 +590,23 @@ int create_impl(const fpd_params *p, void *stream, void *workspace, uint64_t wor
         }
         s->state = workspace;
         s->owns_state = false;
-    } else {
-        FPD_TRY(cudaMalloc(&s->state, L.total), "cudaMalloc simulation state");
     }
-    FPD_TRY(cudaMemsetAsync(s->state, 0, L.total, s->stream), "cudaMemset simulation state");
+    // the profiles lie behind the state in its block, beside a workspace in one
+    // of their own; without memory for them the instance evaluates profiles
+    const size_t prof = profile_bytes(I, s->elem), tail = up(L.total);
+    size_t zeroed = L.total;
+    if (prof) {
+        if (cudaMalloc(workspace ? &s->phimem : &s->state, prof + (workspace ? 0 : tail)) == cudaSuccess) {
+            place_profiles(s, workspace ? s->phimem : (char *)s->state + tail);
+            if (workspace) FPD_TRY(cudaMemsetAsync(s->phimem, 0, prof, s->stream), "cudaMemset kept profiles");
+            else zeroed = tail + prof;
+        } else {
+            (workspace ? s->phimem : s->state) = nullptr;
+            (void)cudaGetLastError();
+        }
+    }
+    if (!s->state) FPD_TRY(cudaMalloc(&s->state, L.total), "cudaMalloc simulation state");
+    FPD_TRY(cudaMemsetAsync(s->state, 0, zeroed, s->stream), "cudaMemset simulation state");
     char *base = (char *)s->state;
     const int nbm = nb > 0 ? nb : 1;
     s->pool = base + L.pool;
@@ -611,10 +620,6 @@ int create_impl(const fpd_params *p, void *stream, void *workspace, uint64_t wor
                                  b + 5 * nbm, b + 6 * nbm, b + 7 * nbm, b + 8 * nbm, f,
                                  f + nbm,     f + 2 * nbm, f + 3 * nbm, f + 4 * nbm, f + 5 * nbm};
     }
-    alloc_profiles(s);
-    if (s->phimem)
-        FPD_TRY(cudaMemsetAsync(s->phimem, 0, 2 * (size_t)nb * (sizeof(int4) + I.phi_cap * sizeof(double)), s->stream),
-                "cudaMemset kept profiles");
     // tile masks, one buffer per step of the rotation (zeroed with the block)
     s->masks[0] = (unsigned *)(base + L.masks);
     for (int m = 1; m < fpd::kMaskBufs; ++m) s->masks[m] = s->masks[0] + m * L.mask_words;

@@ -22,7 +22,7 @@ struct fpd_sim {
     double *tabmem = nullptr;       // two bead tables
     fpd::BeadTab tab[2]{};
     fpd::PhiTab phi[2]{};           // FP64: profiles kept beside the tables
-    void *phimem = nullptr;         // their memory
+    void *phimem = nullptr;         // their memory beside a caller's workspace (otherwise in state)
     unsigned *counters = nullptr;   // one per instance (bead-phase last-block)
     unsigned *status = nullptr;     // sticky FPD_FLAG_* bits of the instance (device word)
     unsigned *masks[fpd::kMaskBufs] = {};  // per-tile bead masks, in rotation by step (t % kMaskBufs)
