@@ -128,7 +128,7 @@ struct fpd_batch {
     cudaStream_t cap_stream = nullptr;
     double *phi_mem = nullptr;  // FP64: both tables' kept profiles (PhiTab::phi)
     int64_t phi_len = 0;        // doubles in phi_mem
-    std::mutex stage_lock;         // of the next two
+    std::mutex stage_lock;         // of the next two (fpd_batch_read_beads)
     double *host_stage = nullptr;  // pinned staging for bead reads (7 doubles a bead of the largest read so far)
     int host_beads = 0;
     double *scratch = nullptr;
@@ -758,7 +758,9 @@ int fpd_batch_read_beads(fpd_batch *b, int32_t slot, double *pos, double *vel, d
     const Slot &sl = b->slots[slot];
     const int nb = sl.inst.nb, off = sl.inst.bead_off;
     if (nb == 0) return fpd_batch_sync(b);
-    // one read at a time uses the staging, threads reading different slots wait
+    // one read at a time uses the staging.  A handle is for one thread at a time
+    // (fpd.h); reads of different slots from several happened to work while each
+    // had arrays of its own, and the lock keeps that much
     std::lock_guard<std::mutex> own(b->stage_lock);
     std::vector<double> plain;
     if (nb > b->host_beads) {

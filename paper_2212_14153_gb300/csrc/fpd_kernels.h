@@ -9,7 +9,9 @@ namespace fpd {
 
 constexpr int kTileX = 32;       // lattice tile: 32 x 8 cells, one thread each
 constexpr int kTileY = 8;
-constexpr int kSplitCtas = 304, kSplitCtas64 = 608;  // a sweep's tiles are split by rows up to this many CTAs: row_split
+// Launch shapes counted in CTAs are multiples of this GPU's 152 SMs.
+constexpr int kSms = 152;
+constexpr int kSplitCtas = 2 * kSms, kSplitCtas64 = 4 * kSms;  // a sweep's tiles are split by rows up to this many CTAs: row_split
 constexpr int kMaxBeads = 256;   // beads per instance (shared-memory tables)
 constexpr int kBeadThreads = 128;  // per bead CTA: more beads resident at once (batched sweep +9 %)
 constexpr int kBeadThreadsMid = 256, kBeadThreadsFew = 512;  // FP32, FP16, the beads fit on the SMs one per SM: launch_beads

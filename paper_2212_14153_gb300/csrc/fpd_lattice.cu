@@ -438,7 +438,7 @@ __device__ __forceinline__ int tile_order(int b, int n, int parity) { return (pa
 // contiguous in its strip).  2048 x 2048, FP16, variant 1: 29.7 -> 27.2 us a
 // step (5.08 -> 5.55 TB/s of the bytes it cannot do without).  In one session,
 // at 684, 1368 and 2736 CTAs: 26.9, 26.5 and 26.4, without 29.3.  By one thread.
-constexpr unsigned kAheadOne = 2736;
+constexpr unsigned kAheadOne = 18 * kSms;
 template <class S>
 __device__ __forceinline__ void prefetch_ahead(const Inst &I, const S *__restrict__ pool, const int parity) {
     const unsigned c = blockIdx.y * gridDim.x + blockIdx.x + kAheadOne;
@@ -719,7 +719,7 @@ template <class S, int CY, bool kAlongX> struct BatchInner {
 // The same pulls and the same one-cell update as lattice_tile's, so the same
 // bits.  A warp owns one row of the tile, so that rows next to a wall or a
 // periodic edge branch off as a whole.
-constexpr unsigned kAhead = 1216;
+constexpr unsigned kAhead = 8 * kSms;
 __device__ __forceinline__ TileRec tile_rec(const TileRec *__restrict__ recs) {
     TileRec r;
     const int4 *q = reinterpret_cast<const int4 *>(recs);
