@@ -293,6 +293,17 @@ __device__ __forceinline__ void segment_axis(const Inst &I, double A, double B, 
     str = ((s - q) + (se - qe)) / (L + I.f_l0);
 }
 
+// v.t of a segment from its two axes' lanes, the same in both, every rounding
+// spelled out (two kernels share it).
+__device__ __forceinline__ double dot_axes(double v, double t) {
+    const double a = __dmul_rn(v, t);
+    return __dadd_rn(a, __shfl_xor_sync(0xffffffffu, a, 1));
+}
+__device__ __forceinline__ float dot_axes(float v, float t) {
+    const float vo = __shfl_xor_sync(0xffffffffu, v, 1), to = __shfl_xor_sync(0xffffffffu, t, 1);
+    return threadIdx.x & 1 ? __fmaf_rn(vo, to, __fmul_rn(v, t)) : __fmaf_rn(v, t, __fmul_rn(vo, to));
+}
+
 // What a segment pulls its first bead with along one axis (and its second the
 // other way): Eq. 11's spring, and Eq. 12's bending, k_b (t_{q+1} + t_{q-1}).
 // (I - t_q t_q) / L with the tangents of missing segments zero (v their sum,
@@ -1022,7 +1033,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         segment_axis(I, s_peer[seg ? j : 0][ax], s_peer[seg ? j + 1 : 0][ax], L, t, str);
         if (!seg) t = 0.f;
         const float tn = __shfl_down_sync(0xffffffffu, t, 2), tp = __shfl_up_sync(0xffffffffu, t, 2);
-        const float v = tn + tp, vt1 = v * t, vt = vt1 + __shfl_xor_sync(0xffffffffu, vt1, 1);
+        const float v = tn + tp, vt = dot_axes(v, t);
         const float pull = seg ? segment_pull(I, v, vt, t, str, L) : 0.f;
         const float before = __shfl_up_sync(0xffffffffu, pull, 2);
         float f = 0.f;  // in lanes 4 and 5 (m = 2)
@@ -1105,7 +1116,7 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             if (i0 < N - 2) v = fs.t[k + 2];
             if (i0 > 0) v += fs.t[k - 2];
         }
-        const R vt1 = v * t, vt = vt1 + __shfl_xor_sync(0xffffffffu, vt1, 1);
+        const R vt = dot_axes(v, t);
         if (seg) fs.pull[k] = segment_pull(I, v, vt, t, fs.str[q], fs.len[q]);
     }
     __syncthreads();
