@@ -24,11 +24,12 @@
 // are listed in shared memory before the kernel waits for the sweep (it is
 // launched while the sweep still runs).  Left on the chain are one round of
 // population loads, one sum, the move, the support sum, and the forces.  us a
-// step, before (list after the wait, sums in a tree, forces in FP64) and now:
-// 100 x 200 with 10 beads 17.9 -> 8.1, 1024 x 256 with 20 (last CTA) 23.0 ->
-// 11.0, FP64 80 x 40 with 8 153 -> 30.
+// step, before (list after the wait, sums in a tree, segments in FP64) and now:
+// 100 x 200 with 10 beads 17.9 -> 7.4, 1024 x 256 with 20 (last CTA) 23.0 ->
+// 10.6, FP64 80 x 40 with 8 153 -> 26.
 //
-// Sums are taken in fixed point (Fix below): exact integer additions, so
+// Sums are taken in fixed point (Fix below): exact integer additions of terms
+// rounded to the point, at the scale of the largest one where it is small.  So
 // they do not depend on which thread or CTA adds which cell, and a warp adds
 // its lanes with redux instructions.  A bead gives the same bits in every
 // launch shape (alone, in a batch, split over a cluster).

@@ -100,8 +100,9 @@ cudaError_t launch_lattice(int precision, const Inst *inst_d, const Inst &inst_h
 // tile its support reaches (mask_write, zeroed beforehand).
 // pdl = 1 launches the bead phase as a programmatic dependent of the
 // previous sweep (the launch right before it: before its wait it reads the
-// instance records, the bead list, the old table and the kept profiles).  Up to kEarlyListTiles tiles it lists its supports beside
-// that sweep and then waits for it; otherwise it waits first thing.  It then
+// instance records, the bead list, the old table and the kept profiles).  Up
+// to kEarlyListTiles tiles it lists its supports beside that sweep and then
+// waits for it; otherwise it waits first thing.  It then
 // releases the next sweep at once, so that sweep's unmarked tiles overlap the
 // rest of the phase.
 // Per-step export of a single instance's finished bead table to host
