@@ -44,6 +44,7 @@
 #include <cuda_fp16.h>
 
 #include <atomic>
+#include <climits>
 #include <type_traits>
 
 #include "fpd_kernels.h"
@@ -237,7 +238,7 @@ __device__ __forceinline__ float min_image_yf(const Inst &I, float d) {
 // (an ulp of 65536 is 1/128 of a cell).
 __device__ __forceinline__ float edge_diff(float a, float b, float L) {
     const float d = a - b;
-    return d > 0.5f * L ? (a - L) - b : (d < -0.5f * L ? a - (b - L) : d);
+    return (a - (d > 0.5f * L ? L : 0.f)) - (b - (d < -0.5f * L ? L : 0.f));
 }
 
 // A double as a pair of floats, h + l equal to it within 2^-48 of its size,
@@ -801,6 +802,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             pdl_wait();
             pdl_trigger();
         }
+        // a largest term that needs less is rounded by the sum (once more, then)
+        int least = kVelBits - (F::kTop - F::kMantissa - bit_length(ncell));
 #pragma unroll 1
         for (int bound = kVelBits;;) {
             const int s = F::kTop - bound - bit_length(ncell);
@@ -854,15 +857,11 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             if (w == 0) {
                 const int need = F::need(mx);
                 // a term of magnitude 2^kVelBits or more (a diverging run), or
-                // all of them so small that they are rounded here: once more
-                const bool slow = bound == kVelBits && mx != 0u && need < kVelBits - (F::kTop - F::kMantissa - bit_length(ncell));
-                int state = (need > bound || slow) && F::finite(mx) ? kAgain + max(need, F::kLowest) : -1;
+                // all of them so small that they were rounded: once more
+                int state = -1;
+                if ((need > bound || need < least) && mx != 0u && F::finite(mx)) state = kAgain + max(need, F::kLowest);
                 if constexpr (!kF64) {
-                    float vx = (float)ax * s_unit_f, vy = (float)ay * s_unit_f;
-                    if (bound < kVelBits) {
-                        const float f = __int_as_float((bound - kVelBits + 127) << 23);
-                        vx *= f, vy *= f;
-                    }
+                    const float vx = (float)ax * s_unit_f, vy = (float)ay * s_unit_f;
                     if (state < 0 && bound <= kVelBits && F::finite(mx) && fabsf(vx) < kEarlyMove && fabsf(vy) < kEarlyMove &&
                         !far_off(xh, yh)) {
                         state = 0;
@@ -877,6 +876,9 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
             const int state = s_state;
             if (state > 0) {
                 bound = state - kAgain;
+                least = INT_MIN;
+                if constexpr (!kF64)
+                    if (tid == 0 && bound < kVelBits) s_unit_f *= __int_as_float((bound - kVelBits + 127) << 23);
                 if (c_hi - c_lo > kCap) n = make_list(c_lo, min(c_lo + kCap, c_hi));  // else it is still in place
                 continue;
             }
@@ -1017,8 +1019,8 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         }
     }
     if constexpr (kTeam) {
+        const int q = b - first, N = I.n_beads, i0 = q - N * (int)(((float)q + 0.5f) * (1.0f / (float)N));
         cluster_wait();  // every bead's place is here, and its status bits are set
-        const int q = b - first, N = I.n_beads, i0 = q - q / N * N;
         // fast-bead guard, as below
         if (w != 0) {
             if (q == 0 && status && (__ldcg(status + ii) & kFlagFastBead))
@@ -1030,16 +1032,18 @@ __global__ void __launch_bounds__(NT, BeadMinBlocks<S, NT>::value)
         // lanes 2 m + ax, m < 4: axis ax of segment q - 2 + m of the fiber
         const int ax = lane & 1, m = (lane >> 1) & 3, j = q - 2 + m;
         const bool seg = i0 - 2 + m >= 0 && i0 - 2 + m < N - 1;
-        float L, t, str;
-        segment_axis(I, s_peer[seg ? j : 0][ax], s_peer[seg ? j + 1 : 0][ax], L, t, str);
-        if (!seg) t = 0.f;
-        const float tn = __shfl_down_sync(0xffffffffu, t, 2), tp = __shfl_up_sync(0xffffffffu, t, 2);
-        const float v = tn + tp, vt = dot_axes(v, t);
-        const float pull = seg ? segment_pull(I, v, vt, t, str, L) : 0.f;
-        const float before = __shfl_up_sync(0xffffffffu, pull, 2);
         float f = 0.f;  // in lanes 4 and 5 (m = 2)
-        if (i0 > 0) f -= before;
-        if (i0 < N - 1) f += pull;
+        if (N > 1) {
+            float L, t, str;
+            segment_axis(I, s_peer[seg ? j : 0][ax], s_peer[seg ? j + 1 : 0][ax], L, t, str);
+            if (!seg) t = 0.f;
+            const float tn = __shfl_down_sync(0xffffffffu, t, 2), tp = __shfl_up_sync(0xffffffffu, t, 2);
+            const float v = tn + tp, vt = dot_axes(v, t);
+            const float pull = seg ? segment_pull(I, v, vt, t, str, L) : 0.f;
+            const float before = __shfl_up_sync(0xffffffffu, pull, 2);
+            if (i0 > 0) f -= before;
+            if (i0 < N - 1) f += pull;
+        }
         if (crowd) {
             const int p = lane < nb ? lane : 0;
             const float x = (float)(s_peer[p][0] - s_peer[0][0]), y = (float)(s_peer[p][1] - s_peer[0][1]);
